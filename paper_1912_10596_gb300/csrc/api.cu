@@ -371,12 +371,17 @@ __global__ void k_flux_spectra(const Real* src, uint64_t stride, uint32_t ne, ui
   flux[t] = f;
 }
 
+// rows of an instance's energy table: vacuum entries, then the weights of nu and nubar
+constexpr int energy_rows(int nf) { return nf == 2 ? Phys2<double>::kERows : Phys3<double>::kERows; }
+
 // ---- host helpers ------------------------------------------------------------------------------
 void build_tables(xflat_t h, HostInst& I, std::vector<double>& et, InstConst& ic) {
   const xflat_config& c = I.cfg;
   const uint32_t ne = c.n_energy, nf = c.n_flavor;
   const double dE = (c.E_max_MeV - c.E_min_MeV) / ne;
-  const int ntab = nf == 2 ? 3 : 4;
+  const int ntab = energy_rows((int)nf);
+  double M21[6] = {}, M31[6] = {};
+  if (nf == 3) vacuum_matrices_3f(c.theta, M21, M31);
   et.assign((size_t)ntab * ne, 0.0);
   // weight scale: total number luminosity of every listed species, flavour and bin
   double S = 0;
@@ -392,10 +397,13 @@ void build_tables(xflat_t h, HostInst& I, std::vector<double>& et, InstConst& ic
       et[ne + k] = (Ne - Nx) / wscale;
       et[2 * ne + k] = -(Nbe - Nbx) / wscale;
     } else {
-      et[k] = c.dm2_eV2[0] * inv2E;
-      et[ne + k] = c.dm2_eV2[1] * inv2E;
-      et[2 * ne + k] = (Ne - Nx) / wscale;
-      et[3 * ne + k] = -(Nbe - Nbx) / wscale;
+      // the vacuum generator without its trace: entries 00 - 22, 11 - 22, 01, 02, 12
+      const double o21 = c.dm2_eV2[0] * inv2E, o31 = c.dm2_eV2[1] * inv2E;
+      const double m21[5] = {M21[0] - M21[2], M21[1] - M21[2], M21[3], M21[4], M21[5]};
+      const double m31[5] = {M31[0] - M31[2], M31[1] - M31[2], M31[3], M31[4], M31[5]};
+      for (int i = 0; i < 5; ++i) et[(size_t)i * ne + k] = o21 * m21[i] + o31 * m31[i];
+      et[5 * ne + k] = (Ne - Nx) / wscale;
+      et[6 * ne + k] = -(Nbe - Nbx) / wscale;
     }
   }
   ic.wscale = wscale;
@@ -425,7 +433,6 @@ void fill_inst_const(HostInst& I, InstConst& ic) {
   ic.B[0] = std::sin(2 * c.theta[0]);
   ic.B[1] = 0.0;
   ic.B[2] = -std::cos(2 * c.theta[0]);
-  if (c.n_flavor == 3) vacuum_matrices_3f(c.theta, ic.M21, ic.M31);
   ic.rtol = c.rtol;
   ic.atol = c.atol;
   ic.h_min = c.h_min_km;
@@ -461,7 +468,7 @@ int upload_tables(xflat_t h, uint32_t i) {
     // r = R).  The kernel accepts thread and block partials below 2^52 units, so no integer sum
     // can overflow; the resolution 2^-S of the normalised moments is 2^-50 or finer for B <= 2.
     const uint32_t ne = I.cfg.n_energy, na = (uint32_t)I.u.size();
-    const int wrow = I.cfg.n_flavor == 2 ? 1 : 2;     // first of the two weight rows (nu, nubar)
+    const int wrow = energy_rows((int)I.cfg.n_flavor) - 2;   // first of the two weight rows (nu, nubar)
     double B = 0.0;
     for (uint32_t a = 0; a < na; ++a) {
       double gs = 0.0;
@@ -572,7 +579,7 @@ void build_pieces(xflat_t h, int G) {
 // Phys3::KT), and the cap on angle bins per piece that bounds the table's shared memory.
 int table_row_values(int nf, size_t real_size, bool ext = false) {
   if (ext) return real_size == 4 ? 18 : 10;
-  return nf == 2 ? (real_size == 4 ? 24 : 8) : 4;
+  return nf == 2 ? (real_size == 4 ? 24 : 8) : Phys3<double>::KT;
 }
 // combined angle rows per piece: bounded by the shared-memory table ([stage slots][rows][row values]);
 // the extended model has ten times the rows per beam, so its rows are kept narrow and a block's
@@ -954,7 +961,7 @@ int create_impl(const xflat_config* cfgs, uint32_t n, xflat_t* out) {
     I.off = off;
     off += I.n_pad;
     I.e_off = eoff;
-    eoff += (h->nf == 2 ? 3 : 4) * I.cfg.n_energy;
+    eoff += energy_rows(h->nf) * I.cfg.n_energy;
     I.a_off = aoff;
     aoff += na_tot;
     // combined angle bins a = j n_phi + p: u_j and du_j / n_phi (the azimuthal measure dphi / 2 pi)

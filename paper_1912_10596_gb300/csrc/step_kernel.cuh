@@ -278,7 +278,8 @@ struct Phys2 {
   static constexpr bool kF32 = sizeof(Real) == 4;
   static constexpr bool kPairable = kF32;       // FP32 passes run beam pairs (PairRK)
   static constexpr bool kNegated = kF32;        // FP32 rows carry -G0_y (saves a multiply per stage)
-  static constexpr int NC = 3, NM = kNM2, NSC = kNSC2, KT = kF32 ? 24 : 8;
+  static constexpr int NC = 3, NG = 3, NM = kNM2, NSC = kNSC2, KT = kF32 ? 24 : 8;
+  static constexpr int kERows = 3;              // energy table: omega_k, weights of nu and nubar
   enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6,
                vNQBX = 7, vNQBZ = 8, vNG0X = 9, vNG0Y = 10, vNG0Z = 11 };
   struct Consts { double B[3]; int geom; };
@@ -322,8 +323,7 @@ struct Phys2 {
       put(t, vNG0Z, -gz);
     }
   }
-  __device__ static inline void K(const Real* t, const Beam& bm, const Real*, const Real*,
-                                  Real (&Kv)[3]) {
+  __device__ static inline void K(const Real* t, const Beam& bm, Real (&Kv)[3]) {
     Kv[0] = bm.eo * val(t, vQBX) + val(t, vG0X);
     Kv[1] = val(t, vG0Y);
     Kv[2] = bm.eo * val(t, vQBZ) + val(t, vG0Z);
@@ -383,74 +383,73 @@ struct Phys2 {
 // is -i [K, P] with the Hermitian
 //   K = [eta (omega21 M21 + omega31 M31) + lambda E_ee + mu (D + (1 - cos) J1)] / cos,
 // M21/M31 the real unit vacuum matrices U diag(0,1,0) U^T and U diag(0,0,1) U^T.
-// Table row (KT = 4): q, t1, t2, pad; the stage constants mu D, mu J1, lambda stay per stage.
+//
+// Commutators and propagators do not see a multiple of the unit matrix in K, so a generator is 8
+// reals (NG): K00 - K22, K11 - K22, then real and imaginary parts of K01, K02, K12.  The energy
+// table holds the 5 real vacuum entries of each bin (kVac) and a table row (KT = 10) the rest of the
+// generator, G = q (lambda E_ee + mu D + (1 - cos) mu J1), so an assembled generator is one FMA for
+// each real entry, K = q v + G.  These kernels are bound by arithmetic (FP64: the two-lane pipe).
 template <typename Real>
 struct Phys3 {
   static constexpr bool kPairable = false;
-  static constexpr int NC = 9, NM = kNM3, NSC = kNSC3, KT = 4;
-  struct Consts { double M21[6], M31[6]; int geom; };
-  struct Beam { Real o21, o31; Real w; };
+  static constexpr int NC = 9, NG = 8, NM = kNM3, NSC = kNSC3, KT = 10;
+  static constexpr int kVac = 5, kERows = kVac + 2;
+  enum : int { vT1 = 0, vQ = 1, vG = 2 };
+  struct Consts { int geom; };
+  struct Beam { Real v[kVac]; Real w; };
 
-  __device__ static inline Real t1(const Real* t) { return t[1]; }
-  __device__ static inline void fill(Real* t, const Geo& g, const double*, const Consts&) {
-    t[0] = (Real)g.q;
-    t[1] = (Real)g.t1;
-    t[2] = (Real)g.t2;
-    t[3] = 0;
+  __device__ static inline Real t1(const Real* t) { return t[vT1]; }
+  // entry i of the generator's matrix-independent part (sc: mu D (9), mu J1 (9), lambda)
+  template <typename T>
+  __device__ static inline T coupling(const T* sc, T t2, int i) { return sc[i] + t2 * sc[9 + i]; }
+  template <typename T>
+  __device__ static inline void fill(Real* t, T q, T t1v, T t2, const T* sc) {
+    const T g22 = coupling(sc, t2, 2);
+    t[vT1] = (Real)t1v;
+    t[vQ] = (Real)q;
+    t[vG + 0] = (Real)(q * (sc[18] + coupling(sc, t2, 0) - g22));
+    t[vG + 1] = (Real)(q * (coupling(sc, t2, 1) - g22));
+#pragma unroll
+    for (int i = 2; i < NG; ++i) t[vG + i] = (Real)(q * coupling(sc, t2, i + 1));
   }
-  __device__ static inline void fill_f(Real* t, float q, float t1, float t2, const float*, const Consts&) {
-    t[0] = q;
-    t[1] = t1;
-    t[2] = t2;
-    t[3] = 0;
+  // the generator: v holds eta (omega21 M21 + omega31 M31) of the beam's energy bin (00 - 22,
+  // 11 - 22, 01, 02, 12)
+  __device__ static inline void K(const Real* t, const Beam& bm, Real (&Kv)[NG]) {
+    const Real q = t[vQ];
+    const Real* g = t + vG;
+    Kv[0] = q * bm.v[0] + g[0];
+    Kv[1] = q * bm.v[1] + g[1];
+    Kv[2] = q * bm.v[2] + g[2];
+    Kv[3] = g[3];
+    Kv[4] = q * bm.v[3] + g[4];
+    Kv[5] = g[5];
+    Kv[6] = q * bm.v[4] + g[6];
+    Kv[7] = g[7];
   }
-  // vac: the six real entries (00,11,22,01,02,12) of M21, M31 in working precision;
-  // sc (working precision): mu D (9), mu J1 (9), lambda
-  __device__ static inline void K(const Real* t, const Beam& bm, const Real* vac, const Real* sc,
-                                  Real (&Kv)[9]) {
-    const Real q = t[0], t2 = t[2];
-    Real v[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) v[i] = bm.o21 * vac[i] + bm.o31 * vac[6 + i];
-    Kv[0] = q * (v[0] + sc[18] + sc[0] + t2 * sc[9]);
-    Kv[1] = q * (v[1] + sc[1] + t2 * sc[10]);
-    Kv[2] = q * (v[2] + sc[2] + t2 * sc[11]);
-    Kv[3] = q * (v[3] + sc[3] + t2 * sc[12]);
-    Kv[4] = q * (sc[4] + t2 * sc[13]);
-    Kv[5] = q * (v[4] + sc[5] + t2 * sc[14]);
-    Kv[6] = q * (sc[6] + t2 * sc[15]);
-    Kv[7] = q * (v[5] + sc[7] + t2 * sc[16]);
-    Kv[8] = q * (sc[8] + t2 * sc[17]);
-  }
-  // Z = -i [K, Y] for Hermitian K, Y; A = K Y, Z_aa = 2 Im A_aa, Z_ab = -i (A_ab - conj(A_ba)).
-  __device__ static inline void f(const Real (&Kv)[9], const Real (&y)[9], Real (&z)[9]) {
-    const Real kr[3][3] = {{Kv[0], Kv[3], Kv[5]}, {Kv[3], Kv[1], Kv[7]}, {Kv[5], Kv[7], Kv[2]}};
-    const Real ki[3][3] = {{0, Kv[4], Kv[6]}, {-Kv[4], 0, Kv[8]}, {-Kv[6], -Kv[8], 0}};
-    const Real yr[3][3] = {{y[0], y[3], y[5]}, {y[3], y[1], y[7]}, {y[5], y[7], y[2]}};
-    const Real yi[3][3] = {{0, y[4], y[6]}, {-y[4], 0, y[8]}, {-y[6], -y[8], 0}};
-    Real ar[3][3], ai[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        Real sr = 0, si = 0;
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) {
-          sr += kr[a][cc] * yr[cc][b] - ki[a][cc] * yi[cc][b];
-          si += kr[a][cc] * yi[cc][b] + ki[a][cc] * yr[cc][b];
-        }
-        ar[a][b] = sr;
-        ai[a][b] = si;
-      }
-    z[0] = 2 * ai[0][0];
-    z[1] = 2 * ai[1][1];
-    z[2] = 2 * ai[2][2];
-    z[3] = ai[0][1] + ai[1][0];
-    z[4] = ar[1][0] - ar[0][1];
-    z[5] = ai[0][2] + ai[2][0];
-    z[6] = ar[2][0] - ar[0][2];
-    z[7] = ai[1][2] + ai[2][1];
-    z[8] = ar[2][1] - ar[1][2];
+  // Z = -i [K, Y] entry by entry.  With x, y, z = K01, K02, K12 and a, b, c = Y01, Y02, Y12:
+  //   [K,Y]_01 = (K00 - K11) a - (Y00 - Y11) x + y conj(c) - b conj(z),
+  //   [K,Y]_02 = (K00 - K22) b - (Y00 - Y22) y + x c - a z,
+  //   [K,Y]_12 = (K11 - K22) c - (Y11 - Y22) z + conj(x) b - conj(a) y,
+  // and the diagonal is 2i Im(x conj(a) + y conj(b)), 2i Im(z conj(c) - x conj(a)), minus their sum:
+  // 52 operations where the two full complex products take about 170.  (262,144 beams, FP64 DP45,
+  // GB300, a call of 8 steps: 7.80 ms with the full products and 39 operations per assembled K,
+  // 4.97 ms so.)
+  __device__ static inline void f(const Real (&Kv)[NG], const Real (&y)[9], Real (&z)[9]) {
+    const Real d02 = Kv[0], d12 = Kv[1], d01 = d02 - d12;
+    const Real xr = Kv[2], xi = Kv[3], yr = Kv[4], yi = Kv[5], zr = Kv[6], zi = Kv[7];
+    const Real ar = y[3], ai = y[4], br = y[5], bi = y[6], cr = y[7], ci = y[8];
+    const Real e01 = y[0] - y[1], e02 = y[0] - y[2], e12 = y[1] - y[2];
+    const Real A = xi * ar - xr * ai, B = yi * br - yr * bi, C = zi * cr - zr * ci;
+    const Real z0 = A + B, z2 = B + C, z1 = C - A;
+    z[0] = z0 + z0;
+    z[1] = z1 + z1;
+    z[2] = -(z2 + z2);
+    z[3] = d01 * ai - e01 * xi + yi * cr - yr * ci - bi * zr + br * zi;
+    z[4] = e01 * xr - d01 * ar - yr * cr - yi * ci + br * zr + bi * zi;
+    z[5] = d02 * bi - e02 * yi + xr * ci + xi * cr - ar * zi - ai * zr;
+    z[6] = e02 * yr - d02 * br - xr * cr + xi * ci + ar * zr - ai * zi;
+    z[7] = d12 * ci - e12 * zi + xr * bi - xi * br - ar * yi + ai * yr;
+    z[8] = e12 * zr - d12 * cr - xr * br - xi * bi + ar * yr + ai * yi;
   }
   template <class Acc>
   __device__ static inline void accum(Acc& acc, Real w, Real t1, const Real (&y)[9]) {
@@ -535,9 +534,10 @@ struct Phys3 {
     if constexpr (sizeof(Real) == 4) {
       float q, t1v, t2;
       geometry_f(u, x, q, t1v, t2, C.geom);
-      fill_f(row, q, t1v, t2, reinterpret_cast<const float*>(scr), C);
+      fill<float>(row, q, t1v, t2, scr);
     } else {
-      fill(row, geometry(u, x, C.geom), sc, C);
+      const Geo g = geometry(u, x, C.geom);
+      fill<double>(row, g.q, g.t1, g.t2, sc);
     }
   }
 };
@@ -553,7 +553,8 @@ struct Phys2E {
   static constexpr bool kF32 = sizeof(Real) == 4;
   static constexpr bool kPairable = kF32;       // FP32 passes run beam pairs (PairRK)
   static constexpr bool kNegated = false;       // no negated copies: rows stay small (many rows)
-  static constexpr int NC = 3, NM = 12, NSC = 14, KT = kF32 ? 18 : 10;
+  static constexpr int NC = 3, NG = 3, NM = 12, NSC = 14, KT = kF32 ? 18 : 10;
+  static constexpr int kERows = Phys2<Real>::kERows;
   // t1, q, q Bx, q Bz, G0 (3), then the azimuthal moment weights (sin th / cos th) cos phi and
   // (sin th / cos th) sin phi; FP32 rows store each value twice (one 64-bit load per packed operand)
   enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6, vSCC = 7, vSCS = 8 };
@@ -607,7 +608,7 @@ struct Phys2E {
     put(t, vSCS, so * sp);
     if constexpr (!kF32) t[9] = 0;
   }
-  __device__ static inline void K(const Real* t, const Beam& bm, const Real*, const Real*, Real (&Kv)[3]) {
+  __device__ static inline void K(const Real* t, const Beam& bm, Real (&Kv)[3]) {
     Kv[0] = bm.eo * val(t, vQBX) + val(t, vG0X);
     Kv[1] = val(t, vG0Y);
     Kv[2] = bm.eo * val(t, vQBZ) + val(t, vG0Z);
@@ -1172,16 +1173,16 @@ __device__ __forceinline__ void jacobi3_rotate(Real (&ar)[3][3], Real (&ai)[3][3
   ar[p][q] = ar[q][p] = ai[p][q] = ai[q][p] = Real(0);
 }
 
-// Three flavours: y <- U y U^dagger with U = exp(-i Om) for Hermitian Om (9 reals: the diagonal,
-// then real and imaginary parts of the 01, 02 and 12 entries), the propagator of Eq. U for a
+// Three flavours: y <- U y U^dagger with U = exp(-i Om) for Hermitian Om (8 reals: the 00 and 11
+// entries less the 22 entry, then real and imaginary parts of the 01, 02 and 12 entries), the propagator of Eq. U for a
 // 3 x 3 generator.  Om = V diag(l) V^dagger by cyclic Jacobi sweeps (a 3 x 3 Hermitian matrix
 // converges quadratically: to the working precision in four sweeps, five in FP64); in the
 // eigenbasis the entry (a, b) of V^dagger y V turns by exp(-i (l_a - l_b)), so U is never formed.
 template <typename Real>
-__device__ __noinline__ void propagate3(const Real (&Om)[9], Real (&y)[9]) {
+__device__ __noinline__ void propagate3(const Real (&Om)[8], Real (&y)[9]) {
   constexpr int kSweeps = sizeof(Real) == 8 ? 5 : 4;
-  Real ar[3][3] = {{Om[0], Om[3], Om[5]}, {Om[3], Om[1], Om[7]}, {Om[5], Om[7], Om[2]}};
-  Real ai[3][3] = {{0, Om[4], Om[6]}, {-Om[4], 0, Om[8]}, {-Om[6], -Om[8], 0}};
+  Real ar[3][3] = {{Om[0], Om[2], Om[4]}, {Om[2], Om[1], Om[6]}, {Om[4], Om[6], 0}};
+  Real ai[3][3] = {{0, Om[3], Om[5]}, {-Om[3], 0, Om[7]}, {-Om[5], -Om[7], 0}};
   Real vr[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
   Real vi[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
 #pragma unroll 1
@@ -1279,7 +1280,7 @@ __device__ __noinline__ void propagate3(const Real (&Om)[9], Real (&y)[9]) {
 template <typename Real>
 __device__ __forceinline__ void propagate(const Real (&Om)[3], Real (&y)[3]) { rotate(Om, y); }
 template <typename Real>
-__device__ __forceinline__ void propagate(const Real (&Om)[9], Real (&y)[9]) { propagate3(Om, y); }
+__device__ __forceinline__ void propagate(const Real (&Om)[8], Real (&y)[9]) { propagate3(Om, y); }
 
 // Per-block shared state of the piece being processed.
 template <typename Real, class Phys>
@@ -1293,7 +1294,6 @@ struct BlockShared {
   Real hA[kMaxStages][kMaxStages];
   Real hB[kMaxStages];
   Real hE[kMaxStages];
-  Real vac[12];                        // three flavours: M21, M31 in working precision
   Real rtol, atol;
   double fx[kNMMax];
   int active;
@@ -1400,8 +1400,8 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
           Y[i] = v;
         }
       }
-      Real Kv[NC];
-      Phys::K(tv.row(l, tj), bm, bs.vac, bs.scr[l], Kv);
+      Real Kv[Phys::NG];
+      Phys::K(tv.row(l, tj), bm, Kv);
       Phys::f(Kv, Y, k[l]);
     }
     if constexpr (kStoreK) {
@@ -1465,8 +1465,8 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       const bool ynok = Phys::tnorm2(yn) <= rbig<Real>();
       if (mixed && ynok) Phys::normalise(yn);
       if (!(Phys::tnorm2(y) <= rbig<Real>())) bad = 1;     // non-finite input state: fatal
-      Real Kv[NC];
-      Phys::K(tv.row(Tab::S, tj), bm, bs.vac, bs.scr[Tab::S], Kv);
+      Real Kv[Phys::NG];
+      Phys::K(tv.row(Tab::S, tj), bm, Kv);
       Phys::f(Kv, yn, k[Tab::S]);
       Real e[NC];
 #pragma unroll
@@ -1489,8 +1489,8 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       // split final pass (y holds y5): k_S = f(y5) with the moments of y5, the embedded error,
       // and the squared error ratio (its square root is taken once per block)
       const bool ynok = Phys::tnorm2(y) <= rbig<Real>();
-      Real Kv[NC], kS[NC], e[NC];
-      Phys::K(tv.row(Tab::S, tj), bm, bs.vac, bs.scr[Tab::S], Kv);
+      Real Kv[Phys::NG], kS[NC], e[NC];
+      Phys::K(tv.row(Tab::S, tj), bm, Kv);
       Phys::f(Kv, y, kS);
 #pragma unroll
       for (int i = 0; i < NC; ++i) {
@@ -1527,40 +1527,41 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
 template <class Phys, class Tab, typename Real, int kPass, int kKind>
 struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
   static constexpr int NC = Phys::NC;          // 3: Bloch vectors; 9: Hermitian 3 x 3 matrices
+  static constexpr int NG = Phys::NG;          // reals of a generator: 3, or 8 (a 3 x 3 without its trace)
   static constexpr bool kStore = false;
   // rotation of y by d K (the propagator of Eq. U over the path length d for generator K)
-  __device__ static inline void rot(Real (&y)[NC], const Real (&K)[NC], Real d) {
-    Real Om[NC];
+  __device__ static inline void rot(Real (&y)[NC], const Real (&K)[NG], Real d) {
+    Real Om[NG];
 #pragma unroll
-    for (int i = 0; i < NC; ++i) Om[i] = d * K[i];
+    for (int i = 0; i < NG; ++i) Om[i] = d * K[i];
     propagate(Om, y);
   }
   // the fourth stage state of a CF4 step of size hh from y with generators Ka (its first stage)
   // and Kc (its third): exp(hh (Kc - Ka/2)) exp(hh/2 Ka) y
-  __device__ static inline void cf4_stage4(Real (&y)[NC], const Real (&Ka)[NC], const Real (&Kc)[NC], Real hh) {
+  __device__ static inline void cf4_stage4(Real (&y)[NC], const Real (&Ka)[NG], const Real (&Kc)[NG], Real hh) {
     rot(y, Ka, Real(0.5) * hh);
-    Real D[NC];
+    Real D[NG];
 #pragma unroll
-    for (int i = 0; i < NC; ++i) D[i] = Kc[i] - Real(0.5) * Ka[i];
+    for (int i = 0; i < NG; ++i) D[i] = Kc[i] - Real(0.5) * Ka[i];
     rot(y, D, hh);
   }
   // the CF4 update of size hh from y with the step's four generators
-  __device__ static inline void cf4_final(Real (&y)[NC], const Real (&K1)[NC], const Real (&K2)[NC],
-                                          const Real (&K3)[NC], const Real (&K4)[NC], Real hh) {
-    Real Om[NC];
+  __device__ static inline void cf4_final(Real (&y)[NC], const Real (&K1)[NG], const Real (&K2)[NG],
+                                          const Real (&K3)[NG], const Real (&K4)[NG], Real hh) {
+    Real Om[NG];
 #pragma unroll
-    for (int i = 0; i < NC; ++i)
+    for (int i = 0; i < NG; ++i)
       Om[i] = hh * (Real(0.25) * K1[i] + Real(1.0 / 6.0) * (K2[i] + K3[i]) - Real(1.0 / 12.0) * K4[i]);
     propagate(Om, y);
 #pragma unroll
-    for (int i = 0; i < NC; ++i)
+    for (int i = 0; i < NG; ++i)
       Om[i] = hh * (Real(-1.0 / 12.0) * K1[i] + Real(1.0 / 6.0) * (K2[i] + K3[i]) + Real(0.25) * K4[i]);
     propagate(Om, y);
   }
   template <class BS>
   __device__ static inline void gen(const BS& bs, const typename Phys::Beam& bm, const TabView<Real, Phys>& tv,
-                                    int tj, int s, Real (&K)[NC]) {
-    Phys::K(tv.row(s, tj), bm, bs.vac, bs.scr[s], K);
+                                    int tj, int s, Real (&K)[NG]) {
+    Phys::K(tv.row(s, tj), bm, K);
   }
   // Richardson-controlled CF4 (TabCFR): pass p forms the stage state of slot p + 2 from y; the
   // final pass forms both results, the error ratio and the moments of the kept result.
@@ -1570,18 +1571,18 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
                                            Real& emax, int& bad, bool mixed) {
     const Real h = bs.hB[0], hh = Real(0.5) * h;
     constexpr int I = kKind == kFinalPass ? 0 : kPass + 2;   // slot formed by this pass
-    Real K1[NC];
+    Real K1[NG];
     gen(bs, bm, tv, tj, 1, K1);
     if constexpr (I >= 2 && I <= 4) {
       // full step: Y2 = exp(h/2 K1) y, Y3 = exp(h/2 K2) y, Y4 = exp(h (K3 - K1/2)) exp(h/2 K1) y
       if constexpr (I == 2) {
         rot(y, K1, hh);
       } else if constexpr (I == 3) {
-        Real K2[NC];
+        Real K2[NG];
         gen(bs, bm, tv, tj, 2, K2);
         rot(y, K2, hh);
       } else {
-        Real K3[NC];
+        Real K3[NG];
         gen(bs, bm, tv, tj, 3, K3);
         cf4_stage4(y, K1, K3, h);
       }
@@ -1593,11 +1594,11 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
       if constexpr (I == 5) {
         rot(y, K1, Real(0.5) * hh);
       } else if constexpr (I == 6) {
-        Real K5[NC];
+        Real K5[NG];
         gen(bs, bm, tv, tj, 5, K5);
         rot(y, K5, Real(0.5) * hh);
       } else {
-        Real K6[NC];
+        Real K6[NG];
         gen(bs, bm, tv, tj, 6, K6);
         cf4_stage4(y, K1, K6, hh);
       }
@@ -1609,7 +1610,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
 #pragma unroll
     for (int i = 0; i < NC; ++i) y0[i] = y[i];
     {
-      Real K5[NC], K6[NC], K7[NC];
+      Real K5[NG], K6[NG], K7[NG];
       gen(bs, bm, tv, tj, 5, K5);
       gen(bs, bm, tv, tj, 6, K6);
       gen(bs, bm, tv, tj, 7, K7);
@@ -1619,17 +1620,17 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
       Phys::accum_row(acc, bm.w, tv.row(8, tj), y);
       return;
     }
-    Real K8[NC];
+    Real K8[NG];
     gen(bs, bm, tv, tj, 8, K8);
     if constexpr (I >= 9 && I <= 11) {
       if constexpr (I == 9) {
         rot(y, K8, Real(0.5) * hh);
       } else if constexpr (I == 10) {
-        Real K9[NC];
+        Real K9[NG];
         gen(bs, bm, tv, tj, 9, K9);
         rot(y, K9, Real(0.5) * hh);
       } else {
-        Real K10[NC];
+        Real K10[NG];
         gen(bs, bm, tv, tj, 10, K10);
         cf4_stage4(y, K8, K10, hh);
       }
@@ -1638,7 +1639,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
     } else {
       // final pass: y_b = the second half step from y_a, y_full = the full step from y0
       {
-        Real K9[NC], K10[NC], K11[NC];
+        Real K9[NG], K10[NG], K11[NG];
         gen(bs, bm, tv, tj, 9, K9);
         gen(bs, bm, tv, tj, 10, K10);
         gen(bs, bm, tv, tj, 11, K11);
@@ -1648,7 +1649,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
 #pragma unroll
       for (int i = 0; i < NC; ++i) yf[i] = y0[i];
       {
-        Real K2[NC], K3[NC], K4[NC];
+        Real K2[NG], K3[NG], K4[NG];
         gen(bs, bm, tv, tj, 2, K2);
         gen(bs, bm, tv, tj, 3, K3);
         gen(bs, bm, tv, tj, 4, K4);
@@ -1685,22 +1686,24 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
     if constexpr (Tab::kEM2) {
       // exponential midpoint rule: half step with K1 -> Y_half (moments at r + h/2); final pass:
       // y' = exp(h K2) y, the estimate exp(h K1) y, the error ratio, moments of y' at r + h
-      Real K1[NC], Om[NC];
-      Phys::K(tv.row(1, tj), bm, bs.vac, bs.scr[1], K1);
+      Real K1[NG], Om[NG];
+      Phys::K(tv.row(1, tj), bm, K1);
       if (kKind == kStagePass) {
 #pragma unroll
-        for (int i = 0; i < NC; ++i) Om[i] = Real(0.5) * h * K1[i];
+        for (int i = 0; i < NG; ++i) Om[i] = Real(0.5) * h * K1[i];
         propagate(Om, y);
         Phys::accum_row(acc, bm.w, tv.row(2, tj), y);
         return;
       }
-      Real K2[NC], yn[NC], ye[NC], e[NC];
-      Phys::K(tv.row(2, tj), bm, bs.vac, bs.scr[2], K2);
+      Real K2[NG], yn[NC], ye[NC], e[NC];
+      Phys::K(tv.row(2, tj), bm, K2);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) { yn[i] = y[i]; ye[i] = y[i]; Om[i] = h * K2[i]; }
+      for (int i = 0; i < NC; ++i) { yn[i] = y[i]; ye[i] = y[i]; }
+#pragma unroll
+      for (int i = 0; i < NG; ++i) Om[i] = h * K2[i];
       propagate(Om, yn);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) Om[i] = h * K1[i];
+      for (int i = 0; i < NG; ++i) Om[i] = h * K1[i];
       propagate(Om, ye);
 #pragma unroll
       for (int i = 0; i < NC; ++i) e[i] = yn[i] - ye[i];
@@ -1716,41 +1719,41 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
       for (int i = 0; i < NC; ++i) y[i] = yn[i];
       return;
     }
-    Real K1[NC], K2[NC], K3[NC], K4[NC], Om[NC];
-    Phys::K(tv.row(1, tj), bm, bs.vac, bs.scr[1], K1);
+    Real K1[NG], K2[NG], K3[NG], K4[NG], Om[NG];
+    Phys::K(tv.row(1, tj), bm, K1);
     if (kKind == kStagePass && kPass == 0) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) Om[i] = Real(0.5) * h * K1[i];
+      for (int i = 0; i < NG; ++i) Om[i] = Real(0.5) * h * K1[i];
       propagate(Om, y);
       Phys::accum_row(acc, bm.w, tv.row(2, tj), y);
       return;
     }
-    Phys::K(tv.row(2, tj), bm, bs.vac, bs.scr[2], K2);
+    Phys::K(tv.row(2, tj), bm, K2);
     if (kKind == kStagePass && kPass == 1) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) Om[i] = Real(0.5) * h * K2[i];
+      for (int i = 0; i < NG; ++i) Om[i] = Real(0.5) * h * K2[i];
       propagate(Om, y);
       Phys::accum_row(acc, bm.w, tv.row(3, tj), y);
       return;
     }
-    Phys::K(tv.row(3, tj), bm, bs.vac, bs.scr[3], K3);
+    Phys::K(tv.row(3, tj), bm, K3);
     if (kKind == kStagePass && kPass == 2) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) Om[i] = Real(0.5) * h * K1[i];
+      for (int i = 0; i < NG; ++i) Om[i] = Real(0.5) * h * K1[i];
       propagate(Om, y);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) Om[i] = h * K3[i] - Real(0.5) * h * K1[i];
+      for (int i = 0; i < NG; ++i) Om[i] = h * K3[i] - Real(0.5) * h * K1[i];
       propagate(Om, y);
       Phys::accum_row(acc, bm.w, tv.row(4, tj), y);
       return;
     }
-    Phys::K(tv.row(4, tj), bm, bs.vac, bs.scr[4], K4);
+    Phys::K(tv.row(4, tj), bm, K4);
 #pragma unroll
-    for (int i = 0; i < NC; ++i)
+    for (int i = 0; i < NG; ++i)
       Om[i] = h * (Real(0.25) * K1[i] + Real(1.0 / 6.0) * (K2[i] + K3[i]) - Real(1.0 / 12.0) * K4[i]);
     propagate(Om, y);
 #pragma unroll
-    for (int i = 0; i < NC; ++i)
+    for (int i = 0; i < NG; ++i)
       Om[i] = h * (Real(-1.0 / 12.0) * K1[i] + Real(1.0 / 6.0) * (K2[i] + K3[i]) + Real(0.25) * K4[i]);
     propagate(Om, y);
     if (mixed) Phys::purify(y);
@@ -2013,20 +2016,22 @@ __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int
 template <typename Real>
 __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int k, Real du,
                                           typename Phys3<Real>::Beam& bm) {
-  const Real o21 = et[k], o31 = et[ne + k];
-  bm.o21 = sigma ? -o21 : o21;
-  bm.o31 = sigma ? -o31 : o31;
-  bm.w = du * et[(2 + sigma) * ne + k];
+  constexpr int kVac = Phys3<Real>::kVac;
+#pragma unroll
+  for (int i = 0; i < kVac; ++i) {
+    const Real v = et[i * ne + k];
+    bm.v[i] = sigma ? -v : v;
+  }
+  bm.w = du * et[(kVac + sigma) * ne + k];
 }
 
-// Checked build: a beam's energy-table entries (rows 0 .. 2 of the two-flavour tables, 0 .. 3 of
-// the three-flavour ones), its row of the shared angle tables and (stored-stage bodies) its
+// Checked build: a beam's energy-table entries (all rows of its bin), its row of the shared angle tables and (stored-stage bodies) its
 // elements of the stage planes.  Always true without XFLAT_BOUNDS.
 template <class Body, int NC, typename Real>
 __device__ __forceinline__ bool beam_in_bounds(const KParams& p, const Real* et, int ne, int k, int tj,
                                                int n_jj, const Real* kst_beam) {
 #ifdef XFLAT_BOUNDS
-  constexpr int kERowMax = NC == 3 ? 2 : 3;
+  constexpr int kERowMax = (NC == 3 ? Phys2<Real>::kERows : Phys3<Real>::kERows) - 1;
   bool ok = index_ok(p, tj >= 0 && tj < n_jj, 12, tj) && index_ok(p, k >= 0 && k < ne, 10, k) &&
             span_ok(p, kSpanEtab, et + k, sizeof(Real), 10) &&
             span_ok(p, kSpanEtab, et + (size_t)kERowMax * ne + k, sizeof(Real), 11);
@@ -2185,13 +2190,9 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       bs.hB2[i] = pk(fb, fb);
       bs.hE2[i] = pk(fe, fe);
     }
-    // launch-invariant part (vacuum matrices, tolerances, angle tables): a single-piece block
+    // launch-invariant part (tolerances, angle tables): a single-piece block
     // loads it once per launch
     if (!(single && bs.keep)) {
-      if (threadIdx.x < 6) {
-        bs.vac[threadIdx.x] = (Real)ic.M21[threadIdx.x];
-        bs.vac[6 + threadIdx.x] = (Real)ic.M31[threadIdx.x];
-      }
       if (threadIdx.x == 0) {
         bs.rtol = (Real)ic.rtol;
         bs.atol = (Real)ic.atol;
@@ -2221,8 +2222,6 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       if constexpr (Phys::NM == 12) C.n_phi = (int)ic.n_phi;
       else C.geom = ic.geom;
     } else {
-#pragma unroll
-      for (int i = 0; i < 6; ++i) { C.M21[i] = ic.M21[i]; C.M31[i] = ic.M31[i]; }
       C.geom = ic.geom;
     }
     // table rows: every needed stage, or (incremental) only the newest and the formed stage

@@ -55,7 +55,6 @@ struct InstConst {
   int32_t matter;
   int32_t adaptive;
   double B[3];              // 2 flavours: unit vacuum vector (sin 2th, 0, -cos 2th)
-  double M21[6], M31[6];    // 3 flavours: U diag(0,1,0) U^T, U diag(0,0,1) U^T (00,11,22,01,02,12)
   double rtol, atol, h_min, h_max;
 };
 
