@@ -35,7 +35,7 @@ L2_BYTES = 129 * 1024 * 1024
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
 STEP_TRAFFIC = {"bytes_per_launch": 51212800 + 173520640, "steps_per_launch": 8,
-                "code_sha256": "384a7fc295b4893c6b375e919685cf6890297471778ed692739cffb47e9a3cb5"}
+                "code_sha256": "4dfec4f99421bd9f1ffd37d47f21ea5db689157f765b3cbbf63738ee153468c8"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a

@@ -18,7 +18,7 @@
 // also move their stage planes.  The exponential integrators (commutator-free Lie RK4, the
 // exponential midpoint rule, the adaptive Lie RK4 with Richardson control) build every stage state
 // from y by exact propagators exp(-i Om) y exp(i Om) of Eq. U instead: a rotation of the Bloch
-// vector for two flavours, an eigen-decomposition of the 3 x 3 generator for three (propagate3).
+// vector for two flavours, a closed form of the 3 x 3 exponential for three (propagate3).
 //
 // Moments without cancellation.  With the measure of Eq. Hnu in u-bins, the nu-nu term of beam b is
 // mu(r) (J0 - cos(th_b) J1), J0 = sum w s / cos(th), J1 = sum w s.  Far from the neutrino sphere
@@ -1104,174 +1104,198 @@ __device__ __forceinline__ void rotate(const Real (&Om)[3], Real (&y)[3]) {
   y[2] += a * c2 + b * d2;
 }
 
-// Three flavours: one cyclic-Jacobi rotation of the Hermitian matrix A (real and imaginary parts)
-// in the plane (p, q), accumulated into V: a phase makes A_pq real, then the real symmetric 2 x 2
-// Schur rotation (Golub and Van Loan, Matrix Computations, Sec. 8.5.2) zeroes it.
-template <typename Real>
-__device__ __forceinline__ void jacobi3_rotate(Real (&ar)[3][3], Real (&ai)[3][3], Real (&vr)[3][3],
-                                               Real (&vi)[3][3], int p, int q) {
-  const Real br = ar[p][q], bi = ai[p][q];
-  const Real mag = hypot(br, bi);                      // no underflow of the squares: |exp(i phi)| = 1
-  // an entry below the rounding of the diagonal is dropped (also keeps converged entries, which
-  // fall towards the underflow range sweep after sweep, from ever entering the phase)
-  const Real tiny = sizeof(Real) == 8 ? Real(8.673617379884035e-19) : Real(9.313225746154785e-10);   // 2^-60, 2^-30
-  if (!(mag > tiny * (fabs(ar[p][p]) + fabs(ar[q][q])))) {
-    ar[p][q] = ar[q][p] = ai[p][q] = ai[q][p] = Real(0);
-    return;
-  }
-  const Real er = br / mag, ei = bi / mag;             // exp(i phi) of A_pq
-  // A <- D^dagger A D, V <- V D with D = diag(1, exp(-i phi)) in the plane: A_pq becomes |A_pq|
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const Real xr = ar[k][q], xi = ai[k][q];
-    ar[k][q] = xr * er + xi * ei;
-    ai[k][q] = xi * er - xr * ei;
-    const Real wr = vr[k][q], wi = vi[k][q];
-    vr[k][q] = wr * er + wi * ei;
-    vi[k][q] = wi * er - wr * ei;
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const Real xr = ar[q][k], xi = ai[q][k];
-    ar[q][k] = xr * er - xi * ei;
-    ai[q][k] = xi * er + xr * ei;
-  }
-  // real rotation J = [[c, s], [-s, c]] in the plane: A <- J^T A J, V <- V J
-  const Real tau = (ar[q][q] - ar[p][p]) / (Real(2) * mag);
-  const Real at = fabs(tau);
-  const Real big = sizeof(Real) == 8 ? Real(1e150) : Real(1e18);
-  const Real t = at > big ? Real(0.5) / tau : copysign(Real(1), tau) / (at + sqrt(Real(1) + tau * tau));
-  const Real c = Real(1) / sqrt(Real(1) + t * t), sn = t * c;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    Real x = ar[k][p], y = ar[k][q];
-    ar[k][p] = c * x - sn * y;
-    ar[k][q] = sn * x + c * y;
-    x = ai[k][p];
-    y = ai[k][q];
-    ai[k][p] = c * x - sn * y;
-    ai[k][q] = sn * x + c * y;
-    x = vr[k][p];
-    y = vr[k][q];
-    vr[k][p] = c * x - sn * y;
-    vr[k][q] = sn * x + c * y;
-    x = vi[k][p];
-    y = vi[k][q];
-    vi[k][p] = c * x - sn * y;
-    vi[k][q] = sn * x + c * y;
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    Real x = ar[p][k], y = ar[q][k];
-    ar[p][k] = c * x - sn * y;
-    ar[q][k] = sn * x + c * y;
-    x = ai[p][k];
-    y = ai[q][k];
-    ai[p][k] = c * x - sn * y;
-    ai[q][k] = sn * x + c * y;
-  }
-  ar[p][q] = ar[q][p] = ai[p][q] = ai[q][p] = Real(0);
+// Helpers of propagate3 in the working precision.  expo: the largest biased exponent of the entries,
+// from their bits (integer pipe); pow2: the power of two of a biased exponent.
+__device__ __forceinline__ int expo_bits(float v) { return __float_as_int(v) & 0x7fffffff; }
+__device__ __forceinline__ int expo_bits(double v) { return __double2hiint(v) & 0x7fffffff; }
+template <typename Real> __device__ __forceinline__ Real pow2_biased(int e) {
+  if constexpr (sizeof(Real) == 4) return __int_as_float(e << 23);
+  else return __hiloint2double(e << 20, 0);
+}
+__device__ __forceinline__ void sincos_of(float x, float& s, float& c) { sincosf(x, &s, &c); }
+__device__ __forceinline__ void sincos_of(double x, double& s, double& c) { sincos(x, &s, &c); }
+// The root of largest modulus of l^3 - c1 l - c0 = 0 (three real roots, c1 > 0; it is at least
+// sqrt(c1) in modulus and the derivative there at least 2 c1, so Newton's iteration is well
+// conditioned).  Seed: with l = sqrt(c1) m the equation is m^3 - m = a, a = |c0| c1^-3/2 in
+// [0, 0.385], whose root a cubic in a gives to 5e-5.
+__device__ __forceinline__ float largest_root_seed(float c1, float c0) {
+  const float rn = rsqrtf(c1);
+  const float a = fminf(fabsf(c0) * rn * rn * rn, 0.3849002f);
+  float m = fmaf(fmaf(fmaf(0.1887236f, a, -0.3171565f), a, 0.4959911f), a, 1.0000473f);
+  m -= __fdividef(fmaf(m, fmaf(m, m, -1.0f), -a), fmaf(3.0f * m, m, -1.0f));
+  return copysignf(m * (c1 * rn), c0);
+}
+__device__ __forceinline__ float largest_root(float c1, float c0) {
+  const float m = largest_root_seed(c1, c0);
+  return m - __fdividef(fmaf(m, fmaf(m, m, -c1), -c0), fmaf(3.0f * m, m, -c1));
+}
+__device__ __forceinline__ double largest_root(double c1, double c0) {
+  // two corrections with the FP32 slope: each multiplies the error (1e-7 at first) by ~1e-7
+  const float c1f = (float)c1, mf = largest_root_seed(c1f, (float)c0);
+  const double inv = (double)__fdividef(1.0f, fmaf(3.0f * mf, mf, -c1f));
+  double m = (double)mf;
+  m = fma(-inv, fma(m, fma(m, m, -c1), -c0), m);
+  return fma(-inv, fma(m, fma(m, m, -c1), -c0), m);
+}
+// 1/sqrt(x) of an x of the order of one, and w, 1/w of w2 = w^2 >= 0 (w = 0 where w2 underflows):
+// Newton steps from the hardware's FP32 values (GB300's FP64 division and square root are long
+// dependent chains)
+__device__ __forceinline__ float rnorm1(float x) {
+  const float r = rsqrtf(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
+__device__ __forceinline__ double rnorm1(double x) {
+  double r = (double)rsqrtf((float)x);
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
+}
+__device__ __forceinline__ void root_pair(float w2, float& w, float& rw) {
+  w = sqrtf(w2);
+  rw = __fdividef(1.0f, w);
+}
+__device__ __forceinline__ void root_pair(double w2, double& w, double& rw) {
+  const float f = (float)w2;
+  if (!(f >= 1.0e-36f)) { w = w2 == w2 ? 0.0 : w2; rw = w; return; }   // far below the rounding of Q
+  double r = (double)rsqrtf(f);
+  r = fma(0.5 * r, fma(-w2 * r, r, 1.0), r);
+  rw = fma(0.5 * r, fma(-w2 * r, r, 1.0), r);
+  w = w2 * rw;
 }
 
 // Three flavours: y <- U y U^dagger with U = exp(-i Om) for Hermitian Om (8 reals: the 00 and 11
-// entries less the 22 entry, then real and imaginary parts of the 01, 02 and 12 entries), the propagator of Eq. U for a
-// 3 x 3 generator.  Om = V diag(l) V^dagger by cyclic Jacobi sweeps (a 3 x 3 Hermitian matrix
-// converges quadratically: to the working precision in four sweeps, five in FP64); in the
-// eigenbasis the entry (a, b) of V^dagger y V turns by exp(-i (l_a - l_b)), so U is never formed.
+// entries less the 22 entry, then real and imaginary parts of the 01, 02 and 12 entries), the
+// propagator of Eq. U for a 3 x 3 generator; a phase of U and a multiple of the unit matrix in Om
+// drop out.
+//
+// Closed form on the traceless Q = Om / s (s a power of two, largest entry in [1, 2)).  Its
+// characteristic polynomial is l^3 - c1 l - c0 (c1 = tr Q^2 / 2, c0 = det Q); m = 2u, the root of
+// largest modulus, is at least sqrt(3 c1)/2 away from the other two, -u + w and -u - w, so its
+// eigenvector v, a column of Q^2 + m Q + (m^2 - c1) = (3 m^2 - c1) v v^dagger (Cayley-Hamilton), is
+// well conditioned even when the other two nearly coincide (matter far above the vacuum
+// splittings).  On the complement of P = v v^dagger the generator is -u + C with the traceless
+// C = Q + u - 3u P, C^2 = w^2 (1 - P), hence
+//   U e^{-ius} = e^{-3ius} P + cos(ws) (1 - P) - i sin(ws)/w C.
+// w comes from the entries of C, not from c1 - 3u^2, whose cancellation would cost eps |Om|^2
+// instead of eps |Om| in the phases; and C is first projected onto the traceless matrices on the
+// complement of v, because the rounding of its entries (eps, where C itself is w) would otherwise
+// make U non-unitary by eps |Om|: that moves whole flavours, not only phases, and near the neutrino
+// sphere it throttled the adaptive step.  With it U is unitary to about ten roundings at any |Om|.
+// About 470 operations, against about 2200 instructions of a cyclic-Jacobi eigen-decomposition
+// (262,144 beams, mixed adaptive Lie RK4 on GB300, a call of 5 attempted steps: 5.08 ms with Jacobi
+// sweeps, 1.98 ms so; largest error against 64 bits over random Om of norms 1e-8 .. 1e4,
+// relative to max(1, |Om|): 0.2e-6 to 0.7e-6 against 1.3e-6 to 1.9e-6 in FP32, 1.5e-15 to 2.7e-15
+// against 3e-15 to 5e-15 in FP64).
 template <typename Real>
 __device__ __noinline__ void propagate3(const Real (&Om)[8], Real (&y)[9]) {
-  constexpr int kSweeps = sizeof(Real) == 8 ? 5 : 4;
-  Real ar[3][3] = {{Om[0], Om[2], Om[4]}, {Om[2], Om[1], Om[6]}, {Om[4], Om[6], 0}};
-  Real ai[3][3] = {{0, Om[3], Om[5]}, {-Om[3], 0, Om[7]}, {-Om[5], -Om[7], 0}};
-  Real vr[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
-  Real vi[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-#pragma unroll 1
-  for (int sw = 0; sw < kSweeps; ++sw) {
-    jacobi3_rotate(ar, ai, vr, vi, 0, 1);
-    jacobi3_rotate(ar, ai, vr, vi, 0, 2);
-    jacobi3_rotate(ar, ai, vr, vi, 1, 2);
+  Real xr = Om[2], xi = Om[3], yr = Om[4], yi = Om[5], zr = Om[6], zi = Om[7];
+  const Real t = (Om[0] + Om[1]) * Real(1.0 / 3.0);
+  Real q0 = Om[0] - t, q1 = Om[1] - t, q2 = -t;
+  constexpr int kMant = sizeof(Real) == 4 ? 23 : 20, kMaxE = sizeof(Real) == 4 ? 253 : 2045;
+  int eb = max(max(expo_bits(q0), expo_bits(q1)), expo_bits(q2));
+  eb = max(eb, max(max(expo_bits(xr), expo_bits(xi)), max(expo_bits(yr), expo_bits(yi))));
+  eb = max(eb, max(expo_bits(zr), expo_bits(zi)));
+  const int E = min(eb >> kMant, kMaxE);
+  if (E == 0) return;                                       // Om = 0 (or denormal)
+  const Real s = pow2_biased<Real>(E), inv = pow2_biased<Real>(kMaxE + 1 - E);
+  q0 *= inv; q1 *= inv; q2 *= inv;
+  xr *= inv; xi *= inv; yr *= inv; yi *= inv; zr *= inv; zi *= inv;
+  // M = Q^2 first, its entries 00, 11, 22, 01, 02, 12
+  const Real x2 = xr * xr + xi * xi, y2 = yr * yr + yi * yi, z2 = zr * zr + zi * zi;
+  Real m00 = q0 * q0 + (x2 + y2), m11 = q1 * q1 + (x2 + z2), m22 = q2 * q2 + (y2 + z2);
+  const Real xzr = xr * zr - xi * zi, xzi = xr * zi + xi * zr;         // x z
+  Real m01r = yr * zr + yi * zi - q2 * xr, m01i = yi * zr - yr * zi - q2 * xi;
+  Real m02r = xzr - q1 * yr, m02i = xzi - q1 * yi;
+  Real m12r = xr * yr + xi * yi - q0 * zr, m12i = xr * yi - xi * yr - q0 * zi;
+  const Real c1 = Real(0.5) * (m00 + m11 + m22);
+  const Real c0 = q0 * (q1 * q2 - z2) - q1 * y2 - q2 * x2 + Real(2) * (xzr * yr + xzi * yi);
+  const Real m = largest_root(c1, c0), u = Real(0.5) * m;
+  // M = (3 m^2 - c1) v v^dagger
+  const Real e = m * m - c1;
+  m00 += m * q0 + e; m11 += m * q1 + e; m22 += m * q2 + e;
+  m01r += m * xr; m01i += m * xi; m02r += m * yr; m02i += m * yi; m12r += m * zr; m12i += m * zi;
+  // v: the column of M with the largest diagonal entry, normalised
+  const bool b1 = m11 > m00 && m11 >= m22, b2 = !b1 && m22 > m00;
+  Real v0r = b1 ? m01r : b2 ? m02r : m00, v0i = b1 ? m01i : b2 ? m02i : Real(0);
+  Real v1r = b1 ? m11 : b2 ? m12r : m01r, v1i = b1 ? Real(0) : b2 ? m12i : -m01i;
+  Real v2r = b1 ? m12r : b2 ? m22 : m02r, v2i = b1 ? -m12i : b2 ? Real(0) : -m02i;
+  const Real rn = rnorm1((v0r * v0r + v0i * v0i) + (v1r * v1r + v1i * v1i) + (v2r * v2r + v2i * v2i));
+  v0r *= rn; v0i *= rn; v1r *= rn; v1i *= rn; v2r *= rn; v2i *= rn;
+  const Real p00 = v0r * v0r + v0i * v0i, p11 = v1r * v1r + v1i * v1i, p22 = v2r * v2r + v2i * v2i;
+  const Real p01r = v0r * v1r + v0i * v1i, p01i = v0i * v1r - v0r * v1i;
+  const Real p02r = v0r * v2r + v0i * v2i, p02i = v0i * v2r - v0r * v2i;
+  const Real p12r = v1r * v2r + v1i * v2i, p12i = v1i * v2r - v1r * v2i;
+  // C = Q + u - 3u P (in q0 .. zi), then its projection C - v h^dagger - h v^dagger - (tau/2)(1 - P)
+  // with r = C v, h = r - (v^dagger r / 2 + tau / 4) v and tau the trace left on the complement
+  const Real k = Real(3) * u;
+  q0 = (q0 + u) - k * p00; q1 = (q1 + u) - k * p11; q2 = (q2 + u) - k * p22;
+  xr -= k * p01r; xi -= k * p01i; yr -= k * p02r; yi -= k * p02i; zr -= k * p12r; zi -= k * p12i;
+  Real w2;
+  {
+    Real r0r = q0 * v0r + xr * v1r - xi * v1i + yr * v2r - yi * v2i;
+    Real r0i = q0 * v0i + xr * v1i + xi * v1r + yr * v2i + yi * v2r;
+    Real r1r = xr * v0r + xi * v0i + q1 * v1r + zr * v2r - zi * v2i;
+    Real r1i = xr * v0i - xi * v0r + q1 * v1i + zr * v2i + zi * v2r;
+    Real r2r = yr * v0r + yi * v0i + zr * v1r + zi * v1i + q2 * v2r;
+    Real r2i = yr * v0i - yi * v0r + zr * v1i - zi * v1r + q2 * v2i;
+    const Real rho = (v0r * r0r + v0i * r0i) + (v1r * r1r + v1i * r1i) + (v2r * r2r + v2i * r2i);
+    const Real tau = (q0 + q1 + q2) - rho;
+    const Real hh = Real(0.5) * rho + Real(0.25) * tau, ht = Real(0.5) * tau;
+    r0r -= hh * v0r; r0i -= hh * v0i; r1r -= hh * v1r; r1i -= hh * v1i; r2r -= hh * v2r; r2i -= hh * v2i;
+    q0 = (q0 - ht) - Real(2) * (v0r * r0r + v0i * r0i);
+    q1 = (q1 - ht) - Real(2) * (v1r * r1r + v1i * r1i);
+    q2 = (q2 - ht) - Real(2) * (v2r * r2r + v2i * r2i);
+    xr -= v0r * r1r + v0i * r1i + r0r * v1r + r0i * v1i;
+    xi -= v0i * r1r - v0r * r1i + r0i * v1r - r0r * v1i;
+    yr -= v0r * r2r + v0i * r2i + r0r * v2r + r0i * v2i;
+    yi -= v0i * r2r - v0r * r2i + r0i * v2r - r0r * v2i;
+    zr -= v1r * r2r + v1i * r2i + r1r * v2r + r1i * v2i;
+    zi -= v1i * r2r - v1r * r2i + r1i * v2r - r1r * v2i;
+    w2 = Real(0.5) * (q0 * q0 + q1 * q1 + q2 * q2) + (xr * xr + xi * xi) + (yr * yr + yi * yi) + (zr * zr + zi * zi);
   }
-  const Real yr[3][3] = {{y[0], y[3], y[5]}, {y[3], y[1], y[7]}, {y[5], y[7], y[2]}};
-  const Real yi[3][3] = {{0, y[4], y[6]}, {-y[4], 0, y[8]}, {-y[6], -y[8], 0}};
-  // T = Y V, W = V^dagger T
-  Real tr[3][3], ti[3][3], wr[3][3], wi[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Real sr = 0, si = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sr += yr[a][c] * vr[c][b] - yi[a][c] * vi[c][b];
-        si += yr[a][c] * vi[c][b] + yi[a][c] * vr[c][b];
-      }
-      tr[a][b] = sr;
-      ti[a][b] = si;
-    }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Real sr = 0, si = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sr += vr[c][a] * tr[c][b] + vi[c][a] * ti[c][b];
-        si += vr[c][a] * ti[c][b] - vi[c][a] * tr[c][b];
-      }
-      wr[a][b] = sr;
-      wi[a][b] = si;
-    }
-  // the phases of the off-diagonal entries in the eigenbasis (W stays Hermitian)
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a + 1; b < 3; ++b) {
-      Real sd, cd;
-      if (sizeof(Real) == 4) sincosf((float)(ar[a][a] - ar[b][b]), (float*)&sd, (float*)&cd);
-      else sincos((double)(ar[a][a] - ar[b][b]), (double*)&sd, (double*)&cd);
-      const Real xr = wr[a][b], xi = wi[a][b];
-      wr[a][b] = xr * cd + xi * sd;
-      wi[a][b] = xi * cd - xr * sd;
-      wr[b][a] = wr[a][b];
-      wi[b][a] = -wi[a][b];
-    }
-  // T = V W, Y = T V^dagger (upper triangle)
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Real sr = 0, si = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sr += vr[a][c] * wr[c][b] - vi[a][c] * wi[c][b];
-        si += vr[a][c] * wi[c][b] + vi[a][c] * wr[c][b];
-      }
-      tr[a][b] = sr;
-      ti[a][b] = si;
-    }
-  Real outr[3][3], outi[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a; b < 3; ++b) {
-      Real sr = 0, si = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sr += tr[a][c] * vr[b][c] + ti[a][c] * vi[b][c];
-        si += ti[a][c] * vr[b][c] - tr[a][c] * vi[b][c];
-      }
-      outr[a][b] = sr;
-      outi[a][b] = si;
-    }
-  y[0] = outr[0][0];
-  y[1] = outr[1][1];
-  y[2] = outr[2][2];
-  y[3] = outr[0][1];
-  y[4] = outi[0][1];
-  y[5] = outr[0][2];
-  y[6] = outi[0][2];
-  y[7] = outr[1][2];
-  y[8] = outi[1][2];
+  Real w, rw, sw, cw, s3, c3;
+  root_pair(w2, w, rw);
+  sincos_of(w * s, sw, cw);
+  sincos_of(k * s, s3, c3);
+  const Real g = w == Real(0) ? s : sw * rw;
+  const Real br = c3 - cw, bi = -s3;
+  // U = cw (1 - P) + e^{-3ius} P - i g C, entry by entry (on the diagonal 1 - P is the sum of the other
+  // two entries of P: nothing cancels where P is nearly a flavour)
+  const Real u00r = c3 * p00 + cw * (p11 + p22), u00i = bi * p00 - g * q0;
+  const Real u11r = c3 * p11 + cw * (p00 + p22), u11i = bi * p11 - g * q1;
+  const Real u22r = c3 * p22 + cw * (p00 + p11), u22i = bi * p22 - g * q2;
+  Real u01r, u01i, u10r, u10i, u02r, u02i, u20r, u20i, u12r, u12i, u21r, u21i;
+  auto pair = [&](Real pr, Real pi, Real qr, Real qi, Real& ur, Real& ui, Real& lr, Real& li) {
+    const Real a1 = br * pr, a2 = bi * pi - g * qi, b1 = bi * pr - g * qr, b2 = br * pi;
+    ur = a1 - a2; ui = b1 + b2;
+    lr = a1 + a2; li = b1 - b2;
+  };
+  pair(p01r, p01i, xr, xi, u01r, u01i, u10r, u10i);
+  pair(p02r, p02i, yr, yi, u02r, u02i, u20r, u20i);
+  pair(p12r, p12i, zr, zi, u12r, u12i, u21r, u21i);
+  // row a of T = U Y, then the entries (a, b >= a) of T U^dagger
+  const Real ar = y[3], ai = y[4], hr = y[5], hi = y[6], cr = y[7], ci = y[8];
+  auto row = [&](Real v0r, Real v0i, Real v1r, Real v1i, Real v2r, Real v2i, Real (&tr)[3], Real (&ti)[3]) {
+    tr[0] = v0r * y[0] + v1r * ar + v1i * ai + v2r * hr + v2i * hi;
+    ti[0] = v0i * y[0] + v1i * ar - v1r * ai + v2i * hr - v2r * hi;
+    tr[1] = v0r * ar - v0i * ai + v1r * y[1] + v2r * cr + v2i * ci;
+    ti[1] = v0i * ar + v0r * ai + v1i * y[1] + v2i * cr - v2r * ci;
+    tr[2] = v0r * hr - v0i * hi + v1r * cr - v1i * ci + v2r * y[2];
+    ti[2] = v0i * hr + v0r * hi + v1i * cr + v1r * ci + v2i * y[2];
+  };
+  Real tr[3], ti[3], n0, n1, n2, n3, n4, n5, n6, n7, n8;
+  row(u00r, u00i, u01r, u01i, u02r, u02i, tr, ti);
+  n0 = tr[0] * u00r + ti[0] * u00i + tr[1] * u01r + ti[1] * u01i + tr[2] * u02r + ti[2] * u02i;
+  n3 = tr[0] * u10r + ti[0] * u10i + tr[1] * u11r + ti[1] * u11i + tr[2] * u12r + ti[2] * u12i;
+  n4 = ti[0] * u10r - tr[0] * u10i + ti[1] * u11r - tr[1] * u11i + ti[2] * u12r - tr[2] * u12i;
+  n5 = tr[0] * u20r + ti[0] * u20i + tr[1] * u21r + ti[1] * u21i + tr[2] * u22r + ti[2] * u22i;
+  n6 = ti[0] * u20r - tr[0] * u20i + ti[1] * u21r - tr[1] * u21i + ti[2] * u22r - tr[2] * u22i;
+  row(u10r, u10i, u11r, u11i, u12r, u12i, tr, ti);
+  n1 = tr[0] * u10r + ti[0] * u10i + tr[1] * u11r + ti[1] * u11i + tr[2] * u12r + ti[2] * u12i;
+  n7 = tr[0] * u20r + ti[0] * u20i + tr[1] * u21r + ti[1] * u21i + tr[2] * u22r + ti[2] * u22i;
+  n8 = ti[0] * u20r - tr[0] * u20i + ti[1] * u21r - tr[1] * u21i + ti[2] * u22r - tr[2] * u22i;
+  row(u20r, u20i, u21r, u21i, u22r, u22i, tr, ti);
+  n2 = tr[0] * u20r + ti[0] * u20i + tr[1] * u21r + ti[1] * u21i + tr[2] * u22r + ti[2] * u22i;
+  y[0] = n0; y[1] = n1; y[2] = n2; y[3] = n3; y[4] = n4; y[5] = n5; y[6] = n6; y[7] = n7; y[8] = n8;
 }
 
 // The propagator of Eq. U over one step for the generator Om (step length and coefficients folded
