@@ -35,7 +35,7 @@ L2_BYTES = 129 * 1024 * 1024
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
 STEP_TRAFFIC = {"bytes_per_launch": 51212800 + 173520640, "steps_per_launch": 8,
-                "code_sha256": "4dfec4f99421bd9f1ffd37d47f21ea5db689157f765b3cbbf63738ee153468c8"}
+                "code_sha256": "3eacce7fcc6dddffc43c6157187ade2712a199c9e7ba44dde131ca46aa02e752"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a

@@ -146,7 +146,7 @@ typedef struct {
   uint64_t barrier_timeout_ns;/* limit of every device-wide wait (0 = 2 s)                         */
   uint32_t block_size;        /* threads per block: 128, 256 or 512 (0 = library default: 512 for
                                  the mixed two-flavour bulb kernels whose two state buffers fit
-                                 the L2, 256 otherwise)                                          */
+                                 the L2, 256 otherwise, fewer where a small problem fills fewer) */
   uint32_t blocks_per_sm;     /* resident blocks per SM for the persistent grid (0 = occupancy)    */
   uint32_t steps_per_launch;  /* radial steps per persistent launch in xflat_evolve (0 = 64)       */
   uint32_t geometry;          /* xflat_geometry (0 = the bulb model); SINGLE_ANGLE and HOMOGENEOUS

@@ -68,6 +68,7 @@ const double kSqrt2GFhc2 = std::sqrt(2.0) * kGF * kHbarcGevKm * kHbarcGevKm;
 
 constexpr uint32_t kMaxJJ = 128;          // combined angle bins per piece (shared-memory table rows)
 constexpr uint32_t kAlignBeams = 4;       // instance offsets and piece starts: 16-byte vectors
+constexpr uint64_t kMinBlockBeams = 128;  // fewest beams a block: two warps of two-beam vectors
 uint32_t max_jj_cap(int nf, size_t real_size, bool ext = false);
 
 struct HostInst {
@@ -502,11 +503,16 @@ void reset_dyn(xflat_t h, uint32_t i, double r0) {
 
 // Cut all instances into G slices and slices into pieces; blk[b]..blk[b+1] are block b's pieces.
 // Dynamic scheduling: blocks take pieces in list order from a counter.  The list holds first every
-// instance's leading beams in pieces of about kDynBig vector iterations per thread, then the last
-// kDynTailPct percent of every instance in pieces of kDynSmall iterations (each at most the table's
-// rows): the large pieces keep the per-piece set-up rare, the small ones at the end of the list let
-// the blocks finish a pass within a small piece of one another.
-constexpr uint32_t kDynBig = 64, kDynSmall = 8, kDynTailPct = 15;
+// instance's leading beams in large pieces, then the last kDynTailPct percent of every instance in
+// small ones (each at most the table's rows): the large pieces keep the per-piece set-up rare, the
+// small ones at the end of the list let the blocks finish a pass within a small piece of one
+// another.  A large piece is a third of a block's vector iterations of a pass, between 16 and 64 of
+// them, a small one a quarter of that, between 4 and 8 (GB300, mixed DP45, 8 steps: 17 instances, 48
+// iterations a block, 5.41 ms in pieces of 64 and 8, 5.23 ms in 16 and 4; 64 instances, 181
+// iterations, 15.8 ms in 64 and 8, 16.8 ms in 32 and 4).  Below kDynMinIters iterations a block's
+// static slice is better (3 instances, 8 iterations: 1.22 ms static, 1.62 to 1.81 ms in pieces; 4
+// instances: 1.84 and 1.74 ms).
+constexpr uint32_t kDynTailPct = 15, kDynMinIters = 10;
 void build_dynamic_pieces(xflat_t h) {
   h->pieces.clear();
   h->blk.assign(h->grid + 1, 0);
@@ -527,12 +533,16 @@ void build_dynamic_pieces(xflat_t h) {
       h->pieces.push_back(p);
     }
   };
+  uint64_t total = 0;
+  for (auto& I : h->inst) total += I.n_beams;
+  const uint32_t iters = (uint32_t)std::min<uint64_t>(total / ((uint64_t)h->grid * 2 * h->block), 1u << 20);
+  const uint32_t big = std::min(64u, std::max(16u, iters / 3)), small = std::min(8u, big / 4);
   std::vector<uint64_t> split(h->inst.size());
   for (uint32_t i = 0; i < h->inst.size(); ++i) {
     split[i] = ((uint64_t)h->inst[i].n_beams * (100 - kDynTailPct) / 100) / kAlignBeams * kAlignBeams;
-    cut(i, 0, split[i], kDynBig);
+    cut(i, 0, split[i], big);
   }
-  for (uint32_t i = 0; i < h->inst.size(); ++i) cut(i, split[i], h->inst[i].n_beams, kDynSmall);
+  for (uint32_t i = 0; i < h->inst.size(); ++i) cut(i, split[i], h->inst[i].n_beams, small);
 }
 
 void build_pieces(xflat_t h, int G) {
@@ -798,16 +808,35 @@ int setup_launch_shape(xflat_t h, const xflat_config& c) {
   CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, h->kernel, h->block, smax));
   if (occ < 1) return fail(h, XFLAT_ERR_CUDA, "kernel does not fit on an SM");
   if (c.blocks_per_sm) occ = std::min<int>(occ, (int)c.blocks_per_sm);
-  uint64_t T = 0;
-  for (auto& I : h->inst) T += I.n_pad;
-  if (h->shard) T = h->shard_hi - h->shard_lo;
-  int G = occ * h->sm_count;
-  // at least one vector of work per thread
-  const uint64_t per_block = (uint64_t)h->block * kAlignBeams;
-  G = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)G, (T + per_block - 1) / per_block));
-  h->grid = G;
-  h->dyn_sched = h->inst.size() > 1 && !h->shard;
-  build_pieces(h, G);
+  // Grid: every resident block, down to kMinBlockBeams beams a block.  A small problem is bound by the
+  // length of a pass on its busiest SM, so its beams go to many SMs (4096 beams, FP64, a call of 16
+  // RK4 or 8 Lie RK4 steps on GB300: 1318 and 1817 us with 1024 beams a block on 4 SMs, 1030 and 840
+  // us with 128 on 32; 64 or 32 beams a block are no faster).  Beam shards of one problem that
+  // together are smaller than one full grid keep the whole problem's blocks, so that they sum in the
+  // same order as the unsharded run where a shard boundary falls between blocks.
+  uint64_t T_all = 0;
+  for (auto& I : h->inst) T_all += I.n_pad;
+  const uint64_t T = h->shard ? h->shard_hi - h->shard_lo : T_all;
+  const uint64_t G_max = (uint64_t)occ * h->sm_count;
+  const auto ceil_div = [](uint64_t a, uint64_t b) { return (a + b - 1) / b; };
+  const uint64_t G_all = std::max<uint64_t>(1, std::min(G_max, ceil_div(T_all, kMinBlockBeams)));
+  uint64_t G = G_all;
+  if (h->shard) {
+    const uint64_t full = std::min(G_max, ceil_div(T, (uint64_t)h->block * kAlignBeams));
+    G = std::max({(uint64_t)1, full, (G_all * T + T_all / 2) / T_all});
+  }
+  // Block: no more warps than the block's beams fill (two beams a thread), at least two; idle warps
+  // would still take part in the FP64 reduction trees.  The mixed two-flavour bulb kernels keep
+  // their block (their reductions are integer and FP32).
+  if (!c.block_size && !mixed_2f) {
+    const uint64_t threads = ceil_div(ceil_div(T_all, G_all), 2);
+    h->block = (int)std::min<uint64_t>((uint64_t)h->block, std::max<uint64_t>(64, ceil_div(threads, 32) * 32));
+  }
+  h->grid = (int)G;
+  // Several instances: blocks take pieces from a counter once each has kDynMinIters vector iterations
+  // of work per pass (see build_dynamic_pieces).
+  h->dyn_sched = h->inst.size() > 1 && !h->shard && T >= G * 2 * (uint64_t)h->block * kDynMinIters;
+  build_pieces(h, h->grid);
   h->smem = smem_bytes(h->nf, h->real_size, h->max_jj, table_stages(h->integrator), h->block, h->extended);
   if (h->d_pieces) cudaFree(h->d_pieces);
   if (h->d_blk) cudaFree(h->d_blk);

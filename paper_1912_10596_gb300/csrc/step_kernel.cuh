@@ -2195,8 +2195,8 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       bs.scr[s][c] = (Real)v;
     }
     if (threadIdx.x < kMaxStages) bs.xs[threadIdx.x] = ldcg(&d->xs[threadIdx.x]);
-    if (threadIdx.x < kMaxStages * kMaxStages) {
-      const int i = threadIdx.x / kMaxStages, j = threadIdx.x % kMaxStages;
+    for (int t = threadIdx.x; t < kMaxStages * kMaxStages; t += blockDim.x) {
+      const int i = t / kMaxStages, j = t % kMaxStages;
       bs.hA[i][j] = (Real)(h * ((i >= 1 && j >= 1) ? Tab::a(i, j) : 0.0));
       const float fa = (float)bs.hA[i][j];
       bs.hA2[i][j] = pk(fa, fa);
