@@ -374,6 +374,10 @@ __global__ void k_flux_spectra(const Real* src, uint64_t stride, uint32_t ne, ui
 
 // rows of an instance's energy table: vacuum entries, then the weights of nu and nubar
 constexpr int energy_rows(int nf) { return nf == 2 ? Phys2<double>::kERows : Phys3<double>::kERows; }
+// values per energy bin of the device table in the working precision
+constexpr int energy_values(int nf, size_t real_size) {
+  return nf == 2 && real_size == 4 ? Phys2<float>::kERows : energy_rows(nf);
+}
 
 // ---- host helpers ------------------------------------------------------------------------------
 void build_tables(xflat_t h, HostInst& I, std::vector<double>& et, InstConst& ic) {
@@ -479,12 +483,19 @@ int upload_tables(xflat_t h, uint32_t i) {
     }
     const int S = B > 0 ? std::min(100, 51 - (int)std::ceil(std::log2(B))) : 50;
     h->ic[i].acc_unit = std::ldexp(1.0, -S);
-    std::vector<float> ef(n);
+    std::vector<float> ef((size_t)energy_values(h->nf, 4) * ne, 0.0f);
+    const bool by_bin = h->nf == 2;                   // two flavours: one padded entry a bin
+    float gmax = 0.0f;
     for (size_t t = 0; t < n; ++t) {
       const bool weight = t >= (size_t)wrow * ne && t < (size_t)(wrow + 2) * ne;
-      ef[t] = (float)(weight ? std::ldexp(et[t], S) : et[t]);
+      const float v = (float)(weight ? std::ldexp(et[t], S) : et[t]);
+      ef[by_bin ? (t % ne) * 4 + t / ne : t] = v;
+      if (weight) gmax = std::max(gmax, std::fabs(v));
     }
-    CUDA_TRY(h, cudaMemcpy((float*)h->d_etab + I.e_off, ef.data(), n * 4, cudaMemcpyHostToDevice));
+    double dumax = 0.0;
+    for (double v : I.du) dumax = std::max(dumax, std::fabs(v));
+    h->ic[i].wmax = (float)dumax * gmax;
+    CUDA_TRY(h, cudaMemcpy((float*)h->d_etab + I.e_off, ef.data(), ef.size() * 4, cudaMemcpyHostToDevice));
   }
   CUDA_TRY(h, cudaMemcpy(h->d_u + I.a_off, I.u.data(), I.u.size() * 8, cudaMemcpyHostToDevice));
   CUDA_TRY(h, cudaMemcpy(h->d_du + I.a_off, I.du.data(), I.du.size() * 8, cudaMemcpyHostToDevice));
@@ -588,8 +599,8 @@ void build_pieces(xflat_t h, int G) {
 // Values per (stage, angle bin) table row of the step kernel (Phys2<float>::KT, Phys2<double>::KT,
 // Phys3::KT), and the cap on angle bins per piece that bounds the table's shared memory.
 int table_row_values(int nf, size_t real_size, bool ext = false) {
-  if (ext) return real_size == 4 ? 18 : 10;
-  return nf == 2 ? (real_size == 4 ? 24 : 8) : Phys3<double>::KT;
+  if (ext) return real_size == 4 ? Phys2E<float>::KT : Phys2E<double>::KT;
+  return nf == 2 ? (real_size == 4 ? Phys2<float>::KT : Phys2<double>::KT) : Phys3<double>::KT;
 }
 // combined angle rows per piece: bounded by the shared-memory table ([stage slots][rows][row values]);
 // the extended model has ten times the rows per beam, so its rows are kept narrow and a block's
@@ -990,7 +1001,7 @@ int create_impl(const xflat_config* cfgs, uint32_t n, xflat_t* out) {
     I.off = off;
     off += I.n_pad;
     I.e_off = eoff;
-    eoff += energy_rows(h->nf) * I.cfg.n_energy;
+    eoff += energy_values(h->nf, h->real_size) * I.cfg.n_energy;
     I.a_off = aoff;
     aoff += na_tot;
     // combined angle bins a = j n_phi + p: u_j and du_j / n_phi (the azimuthal measure dphi / 2 pi)
@@ -1750,7 +1761,7 @@ int xflat_shard_partials(xflat_t h, int64_t* words) {
     for (int cp = 0; cp < kAccCopies; ++cp) {
       const unsigned long long* w = acc.data() + ((size_t)cp * kNMMax + c) * 2;
       if (h->real_size == 4) t += (unsigned __int128)(__int128)(long long)w[0];   // one signed word
-      else t += ((unsigned __int128)w[1] << 64) | (unsigned __int128)w[0];
+      else t += (unsigned __int128)((__int128)(long long)w[1] * (1ll << 52) + (long long)w[0]);   // see fx_add
     }
     words[2 * c] = (int64_t)(unsigned long long)t;
     words[2 * c + 1] = (int64_t)(unsigned long long)(t >> 64);
@@ -1771,8 +1782,15 @@ int xflat_shard_set_totals(xflat_t h, const int64_t* words) {
   constexpr int kWords = kAccCopies * kNMMax * 2;
   std::vector<unsigned long long> acc(kWords, 0ull);    // the total in copy 0, the other copies 0
   for (int c = 0; c < nm; ++c) {
-    acc[(size_t)c * 2] = (unsigned long long)words[2 * c];
-    acc[(size_t)c * 2 + 1] = h->real_size == 4 ? 0ull : (unsigned long long)words[2 * c + 1];
+    const __int128 t = (__int128)(((unsigned __int128)(unsigned long long)words[2 * c + 1] << 64) |
+                                  (unsigned long long)words[2 * c]);
+    if (h->real_size == 4) {
+      acc[(size_t)c * 2] = (unsigned long long)words[2 * c];
+    } else {
+      // the two signed words of fx_add: the total's low 52 bits and the rest
+      acc[(size_t)c * 2] = (unsigned long long)t & ((1ull << 52) - 1);
+      acc[(size_t)c * 2 + 1] = (unsigned long long)(long long)(t >> 52);
+    }
     if (h->real_size == 4) {
       // a mixed accumulator is one signed 64-bit word: the total must fit it
       const long long lo = words[2 * c], hi = words[2 * c + 1];

@@ -30,12 +30,11 @@
 // Reduction.  FP64 path: each thread accumulates its beams' contributions in double, each block
 // reduces them with a fixed shuffle/shared-memory tree in double and adds its partial to the
 // instance accumulator as a 128-bit fixed-point integer (exact to 2^-64).  Mixed path: each beam's
-// contribution is formed in FP32 (per-beam algebra) and summed per thread without rounding loss as
-// an unevaluated (hi, lo) pair (TwoSum); at the end of the pass the pair goes to integers in units
-// of the instance's 2^-S (the FP32 weights carry that power-of-two scale), and the warp shuffle
-// trees, the sum over warps and the grid sum are integer additions.  So the moments are the
-// FP64-accurate sums of the FP32 contributions, with no FP64 instruction per beam (GB300's FP64
-// pipe is ~1/68 of its FP32 rate).  Integer addition is associative, so either grid-level sum is
+// contribution (an FP32 weight times an FP32 state) is summed per thread without rounding loss as an
+// unevaluated (hi, lo) pair (MomAcc<float>); at the end of the pass the pair goes to integers in units
+// of the instance's 2^-S (the FP32 weights carry that power-of-two scale), and the sums over lanes,
+// warps and the grid are integer additions.  So the moments are FP64-accurate sums, with no FP64
+// instruction per beam (GB300's FP64 pipe is ~1/68 of its FP32 rate).  Integer addition is associative, so either grid-level sum is
 // identical whatever order the blocks arrive in.  Every block derives a stage's constants
 // mu(r_s) D, mu(r_s) J1, lambda(r_s) from the integer sums; the last block to arrive at a step's
 // final barrier runs the step-size controller in double.
@@ -209,26 +208,34 @@ __device__ __forceinline__ void geometry_f(double u, double x, float& q, float& 
 
 // --------------------------------------------------------------------------------------------
 // Per-thread moment accumulators.  FP64 kernels add each beam's contribution w s by FMA into a
-// double.  Mixed kernels form each contribution w s in FP32 (per-beam algebra) and sum the
-// contributions without rounding loss: a component's running sum is the unevaluated pair hi + lo,
-// and TwoSum (Knuth, TAOCP vol. 2, 4.2.2) splits hi + c into the rounded sum and its exact
-// rounding error, which lo collects (lo's own roundings stay near 2^-48 of the sum, as in a
-// double accumulator).  At the end of a pass each thread's pair goes exactly to integers
-// (f32_to_fix) and every further sum is an integer addition.  The FP32 weights carry a
-// per-instance power-of-two scale (InstConst::acc_unit = 2^-S) so that the integers are in units
-// of 2^-S; no FP64 instruction is issued per beam (GB300's FP64 pipe is ~1/68 of its FP32 rate).
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float c) {
-  const float s = __fadd_rn(hi, c);
-  const float bv = __fsub_rn(s, hi);
-  const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bv)), __fsub_rn(c, bv));
+// double.  Mixed kernels sum the contributions of FP32 weights and states as an unevaluated pair
+// hi + lo without rounding loss, four operations a contribution:
+//   s = fma(w, y, hi),  z = hi - s,  lo += fma(w, y, z),  hi = s.
+// hi starts at a bias 1.5 2^m with 2^(m-1) at least the sum of the contributions' magnitudes, so it
+// stays in one binade: z is exact (both are multiples of the same 2^(m-23)), fma(w, y, z) is the part
+// of the exact product that hi did not take, rounded near 2^(m-48), and lo's own roundings lie there
+// too -- as in a double accumulator, and the product itself is not rounded first.  (TwoSum on the
+// rounded product takes eight operations and needs no bias.)  At the end of a pass hi is an integer
+// count of 2^(m-23) read off its bits (biased_fix) and every further sum is an integer addition.  The
+// FP32 weights carry a per-instance power-of-two scale (InstConst::acc_unit = 2^-S) so that the
+// integers are in units of 2^-S; no FP64 instruction is issued per beam (GB300's FP64 pipe is ~1/68
+// of its FP32 rate).  Components come in groups with a bias each (D, J1, and Jc, Js): their weights
+// differ by the geometry factor, which far from R is far below one.
+__device__ __forceinline__ void biased_add(float& hi, float& lo, float w, float y) {
+  const float s = __fmaf_rn(w, y, hi);
+  const float z = __fsub_rn(hi, s);
+  lo = __fadd_rn(lo, __fmaf_rn(w, y, z));
   hi = s;
-  lo = __fadd_rn(lo, err);
+}
+// The bias for contributions whose magnitudes sum to at most P: 1.5 2^m, 2^(m-2) <= P < 2^(m-1).
+__device__ __forceinline__ float sum_bias(float P) {
+  return __int_as_float((((__float_as_int(P) >> 23) + 2) << 23) | 0x400000);
 }
 
 template <typename Real, int NM> struct MomAcc;
 template <int NM> struct MomAcc<double, NM> {
   double v[NM];
-  __device__ __forceinline__ void zero() {
+  __device__ __forceinline__ void start(const float*, int) {
 #pragma unroll
     for (int i = 0; i < NM; ++i) v[i] = 0.0;
   }
@@ -236,11 +243,12 @@ template <int NM> struct MomAcc<double, NM> {
 };
 template <int NM> struct MomAcc<float, NM> {
   float hi[NM], lo[NM];
-  __device__ __forceinline__ void zero() {
+  // bias: one per group of nc components
+  __device__ __forceinline__ void start(const float* bias, int nc) {
 #pragma unroll
-    for (int i = 0; i < NM; ++i) { hi[i] = 0.0f; lo[i] = 0.0f; }
+    for (int i = 0; i < NM; ++i) { hi[i] = bias[i / nc]; lo[i] = 0.0f; }
   }
-  __device__ __forceinline__ void add(int i, float w, float y) { two_sum_acc(hi[i], lo[i], __fmul_rn(w, y)); }
+  __device__ __forceinline__ void add(int i, float w, float y) { biased_add(hi[i], lo[i], w, y); }
 };
 
 // A float that holds a count of 2^-S units (possibly with a fraction) as the nearest int64 (halves
@@ -259,6 +267,31 @@ __device__ __forceinline__ long long f32_to_fix(float v, int& ovf) {
 }
 constexpr long long kFixLimit = 1ll << 52;               // largest block partial accepted
 
+// The sum collected by N biased accumulators (hi starting at bias, lo) in units of 2^-S: hi's distance
+// from the bias off its bits, lo rounded.  A hi that left its binade (a state far above unit length) or
+// a lo past 32 bits takes the general conversion.
+template <int N>
+__device__ __forceinline__ long long biased_fix(const float (&hi)[N], float lo, float bias, int& ovf) {
+  const int bb = __float_as_int(bias), sh = (bb >> 23) - 127 - 23;
+  bool plain = fabsf(lo) < 2.0e9f;
+  int k = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int b = __float_as_int(hi[i]);
+    plain = plain && ((b ^ bb) >> 23) == 0;
+    k += b - bb;
+  }
+  if (plain) {
+    const int down = min(max(-sh, 0), 62);
+    const long long v = ((long long)k << max(sh, 0)) + (down ? 1ll << (down - 1) : 0ll);
+    return (v >> down) + (long long)__float2int_rn(lo);
+  }
+  long long v = f32_to_fix(lo, ovf);
+#pragma unroll
+  for (int i = 0; i < N; ++i) v += f32_to_fix(__fsub_rn(hi[i], bias), ovf);
+  return v;
+}
+
 // --------------------------------------------------------------------------------------------
 // Physics policies.  "Real" is the working precision of the per-beam algebra.
 //
@@ -268,65 +301,70 @@ constexpr long long kFixLimit = 1ll << 52;               // largest block partia
 // eta = +1 / -1 for nu / nubar, B = (sin 2 theta_v, 0, -cos 2 theta_v): this is
 // d(rho)/dr = -i [H, rho] / cos(th) of Eq. eom with H = (1/2) h.sigma.
 //
-// Per (stage, angle bin) table row: t1 = 1/cos - 1, q = 1/cos, q Bx, q Bz, G0x, G0y, G0z with
-// G0 = q (lambda z + mu D + (1 - cos) mu J1), so that K = eta omega (q Bx, 0, q Bz) + G0, followed
-// (FP32 only) by the negated q Bx, q Bz, G0.  FP64 rows hold the 7 values (KT = 8).  FP32 rows hold
-// 12 values each stored twice (KT = 24): a 64-bit load then yields a packed f32x2 operand for the
-// two beams a thread processes together (both share the angle bin), see PairRK.
+// A table row belongs to one (stage, angle bin): a geometry part, t1 = 1/cos - 1, q = 1/cos, t2 (see
+// Geo), q Bx, q Bz, known from the step's radii alone (fill_geo), and a coupling part G0 = q (lambda z +
+// mu D + t2 mu J1), known once the stage's moments are (fill_cpl), so that K = eta omega (q Bx, 0, q Bz)
+// + G0.  FP32 rows are in the order and the signs in which PairRK needs the components of K, one
+// 128-bit and one 32-bit load a stage; those of the commutator integrators are K times the step size.
 template <typename Real>
 struct Phys2 {
   static constexpr bool kF32 = sizeof(Real) == 4;
   static constexpr bool kPairable = kF32;       // FP32 passes run beam pairs (PairRK)
-  static constexpr bool kNegated = kF32;        // FP32 rows carry -G0_y (saves a multiply per stage)
-  static constexpr int NC = 3, NG = 3, NM = kNM2, NSC = kNSC2, KT = kF32 ? 24 : 8;
-  static constexpr int kERows = 3;              // energy table: omega_k, weights of nu and nubar
-  enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6,
-               vNQBX = 7, vNQBZ = 8, vNG0X = 9, vNG0Y = 10, vNG0Z = 11 };
+  static constexpr int NC = 3, NG = 3, NM = kNM2, NSC = kNSC2, KT = 8;
+  static constexpr int kERows = kF32 ? 4 : 3;   // energy table: omega_k, weights of nu and nubar (FP32: by bin, padded)
+  enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6, vT2 = 7 };   // FP64
+  enum : int { oNQBX = 0, oNG0X = 1, oQBZ = 2, oG0Z = 3, oG0Y = 4, oT1 = 5, oT2 = 6, oQ = 7 };                 // FP32
   struct Consts { double B[3]; int geom; };
   struct Beam { Real eo; Real w; };   // eta * omega_k, signed weight du_j * g_{sigma,k}
 
-  __device__ static inline Real val(const Real* t, int v) { return kF32 ? t[2 * v] : t[v]; }
-  __device__ static inline void put(Real* t, int v, Real x) {
-    if (kF32) { t[2 * v] = x; t[2 * v + 1] = x; } else { t[v] = x; }
-  }
-  __device__ static inline Real t1(const Real* t) { return val(t, vT1); }
+  __device__ static inline Real t1(const Real* t) { return kF32 ? t[oT1] : t[vT1]; }
 
-  // sc: mu D (3), mu J1 (3), lambda
-  __device__ static inline void fill(Real* t, const Geo& g, const double* sc, const Consts& C) {
-    put(t, vT1, (Real)g.t1);
-    put(t, vQ, (Real)g.q);
-    put(t, vQBX, (Real)(g.q * C.B[0]));
-    put(t, vQBZ, (Real)(g.q * C.B[2]));
-    put(t, vG0X, (Real)(g.q * (sc[0] + g.t2 * sc[3])));
-    put(t, vG0Y, (Real)(g.q * (sc[1] + g.t2 * sc[4])));
-    put(t, vG0Z, (Real)(g.q * (sc[6] + sc[2] + g.t2 * sc[5])));
-    if (!kF32) t[7] = 0;
+  // hs: factor of the K entries (the step size, or 1)
+  __device__ static inline void fill_geo(Real* t, double u, double x, const Consts& C, int, Real hs) {
+    if constexpr (kF32) {
+      float q, t1v, t2;
+      geometry_f(u, x, q, t1v, t2, C.geom);
+      const float hq = hs * q;
+      t[oNQBX] = -(hq * (float)C.B[0]);
+      t[oQBZ] = hq * (float)C.B[2];
+      t[oT1] = t1v;
+      t[oT2] = t2;
+      t[oQ] = hq;
+    } else {
+      const Geo g = geometry(u, x, C.geom);
+      t[vT1] = g.t1;
+      t[vQ] = g.q;
+      t[vT2] = g.t2;
+      t[vQBX] = g.q * C.B[0];
+      t[vQBZ] = g.q * C.B[2];
+    }
   }
-  __device__ static inline void fill_f(Real* t, float q, float t1v, float t2, const float* scf,
-                                       const Consts& C) {
-    const float qbx = q * (float)C.B[0], qbz = q * (float)C.B[2];
-    const float gx = q * (scf[0] + t2 * scf[3]);
-    const float gy = q * (scf[1] + t2 * scf[4]);
-    const float gz = q * (scf[6] + scf[2] + t2 * scf[5]);
-    put(t, vT1, t1v);
-    put(t, vQ, q);
-    put(t, vQBX, qbx);
-    put(t, vQBZ, qbz);
-    put(t, vG0X, gx);
-    put(t, vG0Y, gy);
-    put(t, vG0Z, gz);
-    if (kF32) {
-      put(t, vNQBX, -qbx);
-      put(t, vNQBZ, -qbz);
-      put(t, vNG0X, -gx);
-      put(t, vNG0Y, -gy);
-      put(t, vNG0Z, -gz);
+  // sc: mu D (3), mu J1 (3), lambda
+  __device__ static inline void fill_cpl(Real* t, const Real* sc) {
+    const Real q = kF32 ? t[oQ] : t[vQ], t2 = kF32 ? t[oT2] : t[vT2];
+    const Real gx = q * (sc[0] + t2 * sc[3]);
+    const Real gy = q * (sc[1] + t2 * sc[4]);
+    const Real gz = q * (sc[6] + sc[2] + t2 * sc[5]);
+    if constexpr (kF32) {
+      t[oNG0X] = -gx;
+      t[oG0Z] = gz;
+      t[oG0Y] = gy;
+    } else {
+      t[vG0X] = gx;
+      t[vG0Y] = gy;
+      t[vG0Z] = gz;
     }
   }
   __device__ static inline void K(const Real* t, const Beam& bm, Real (&Kv)[3]) {
-    Kv[0] = bm.eo * val(t, vQBX) + val(t, vG0X);
-    Kv[1] = val(t, vG0Y);
-    Kv[2] = bm.eo * val(t, vQBZ) + val(t, vG0Z);
+    if constexpr (kF32) {
+      Kv[0] = -(bm.eo * t[oNQBX] + t[oNG0X]);
+      Kv[1] = t[oG0Y];
+      Kv[2] = bm.eo * t[oQBZ] + t[oG0Z];
+    } else {
+      Kv[0] = bm.eo * t[vQBX] + t[vG0X];
+      Kv[1] = t[vG0Y];
+      Kv[2] = bm.eo * t[vQBZ] + t[vG0Z];
+    }
   }
   __device__ static inline void f(const Real (&Kv)[3], const Real (&y)[3], Real (&k)[3]) {
     k[0] = Kv[1] * y[2] - Kv[2] * y[1];
@@ -335,25 +373,10 @@ struct Phys2 {
   }
   // moments D (weight w t1) and J1 (weight w)
   template <class Acc>
-  __device__ static inline void accum(Acc& acc, Real w, Real t1, const Real (&y)[3]) {
-    const Real wt = w * t1;
+  __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[3]) {
+    const Real wt = w * t1(row);
 #pragma unroll
     for (int i = 0; i < 3; ++i) { acc.add(i, wt, y[i]); acc.add(3 + i, w, y[i]); }
-  }
-  template <class Acc>
-  __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[3]) {
-    accum(acc, w, t1(row), y);
-  }
-  // table row of (stage with constants sc / scf and R^2/r^2 = x, angle bin at u)
-  __device__ static inline void fill_row(Real* row, double u, double x, const double* sc, const Real* scr,
-                                         const Consts& C, int, int) {
-    if constexpr (kF32) {
-      float q, t1v, t2;
-      geometry_f(u, x, q, t1v, t2, C.geom);
-      fill_f(row, q, t1v, t2, reinterpret_cast<const float*>(scr), C);
-    } else {
-      fill(row, geometry(u, x, C.geom), sc, C);
-    }
   }
   // Frobenius norm^2 of the traceless part of P = (1 + s.sigma)/2: |s|^2 / 2
   __device__ static inline Real tnorm2(const Real (&y)[3]) {
@@ -386,31 +409,41 @@ struct Phys2 {
 //
 // Commutators and propagators do not see a multiple of the unit matrix in K, so a generator is 8
 // reals (NG): K00 - K22, K11 - K22, then real and imaginary parts of K01, K02, K12.  The energy
-// table holds the 5 real vacuum entries of each bin (kVac) and a table row (KT = 10) the rest of the
+// table holds the 5 real vacuum entries of each bin (kVac) and a table row the rest of the
 // generator, G = q (lambda E_ee + mu D + (1 - cos) mu J1), so an assembled generator is one FMA for
 // each real entry, K = q v + G.  These kernels are bound by arithmetic (FP64: the two-lane pipe).
 template <typename Real>
 struct Phys3 {
   static constexpr bool kPairable = false;
-  static constexpr int NC = 9, NG = 8, NM = kNM3, NSC = kNSC3, KT = 10;
+  static constexpr int NC = 9, NG = 8, NM = kNM3, NSC = kNSC3, KT = 11;
   static constexpr int kVac = 5, kERows = kVac + 2;
-  enum : int { vT1 = 0, vQ = 1, vG = 2 };
+  enum : int { vT1 = 0, vQ = 1, vG = 2, vT2 = 10 };
   struct Consts { int geom; };
   struct Beam { Real v[kVac]; Real w; };
 
   __device__ static inline Real t1(const Real* t) { return t[vT1]; }
-  // entry i of the generator's matrix-independent part (sc: mu D (9), mu J1 (9), lambda)
-  template <typename T>
-  __device__ static inline T coupling(const T* sc, T t2, int i) { return sc[i] + t2 * sc[9 + i]; }
-  template <typename T>
-  __device__ static inline void fill(Real* t, T q, T t1v, T t2, const T* sc) {
-    const T g22 = coupling(sc, t2, 2);
-    t[vT1] = (Real)t1v;
-    t[vQ] = (Real)q;
-    t[vG + 0] = (Real)(q * (sc[18] + coupling(sc, t2, 0) - g22));
-    t[vG + 1] = (Real)(q * (coupling(sc, t2, 1) - g22));
+  __device__ static inline void fill_geo(Real* t, double u, double x, const Consts& C, int, Real hs) {
+    if constexpr (sizeof(Real) == 4) {
+      float q, t1v, t2;
+      geometry_f(u, x, q, t1v, t2, C.geom);
+      t[vT1] = t1v;
+      t[vQ] = hs * q;
+      t[vT2] = t2;
+    } else {
+      const Geo g = geometry(u, x, C.geom);
+      t[vT1] = g.t1;
+      t[vQ] = g.q;
+      t[vT2] = g.t2;
+    }
+  }
+  // sc: mu D (9), mu J1 (9), lambda
+  __device__ static inline void fill_cpl(Real* t, const Real* sc) {
+    const Real q = t[vQ], t2 = t[vT2];
+    const Real g22 = sc[2] + t2 * sc[11];
+    t[vG + 0] = q * (sc[18] + (sc[0] + t2 * sc[9]) - g22);
+    t[vG + 1] = q * (sc[1] + t2 * sc[10] - g22);
 #pragma unroll
-    for (int i = 2; i < NG; ++i) t[vG + i] = (Real)(q * coupling(sc, t2, i + 1));
+    for (int i = 2; i < NG; ++i) t[vG + i] = q * (sc[i + 1] + t2 * sc[i + 10]);
   }
   // the generator: v holds eta (omega21 M21 + omega31 M31) of the beam's energy bin (00 - 22,
   // 11 - 22, 01, 02, 12)
@@ -452,8 +485,8 @@ struct Phys3 {
     z[8] = e12 * zr - d12 * cr - xr * br - xi * bi + ar * yr + ai * yi;
   }
   template <class Acc>
-  __device__ static inline void accum(Acc& acc, Real w, Real t1, const Real (&y)[9]) {
-    const Real wt = w * t1;
+  __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[9]) {
+    const Real wt = w * t1(row);
 #pragma unroll
     for (int i = 0; i < 9; ++i) { acc.add(i, wt, y[i]); acc.add(9 + i, w, y[i]); }
   }
@@ -525,100 +558,93 @@ struct Phys3 {
     y[7] = outr[1][2];
     y[8] = outi[1][2];
   }
-  template <class Acc>
-  __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[NC]) {
-    accum(acc, w, t1(row), y);
-  }
-  __device__ static inline void fill_row(Real* row, double u, double x, const double* sc, const Real* scr,
-                                         const Consts& C, int, int) {
-    if constexpr (sizeof(Real) == 4) {
-      float q, t1v, t2;
-      geometry_f(u, x, q, t1v, t2, C.geom);
-      fill<float>(row, q, t1v, t2, scr);
-    } else {
-      const Geo g = geometry(u, x, C.geom);
-      fill<double>(row, g.q, g.t1, g.t2, sc);
-    }
-  }
 };
 // Two flavours, extended bulb model (Sec. 2, Eq. int-v and Eq. F): beams also carry an azimuthal
 // angle phi around the radial direction, the combined angle bin a = j n_phi + p holding u_j,
 // du_j / n_phi and phi_p = 2 pi (p + 1/2) / n_phi.  Besides D and J1 the potential needs
 //   Jc = sum_b w_b (sin th_b / cos th_b) cos phi_b s_b,   Js = the same with sin phi_b,
 // and K = [eta omega B + lambda z + mu (D + (1 - cos th) J1 - sin th (cos phi Jc + sin phi Js))] / cos th.
-// Table row: t1, q, q Bx, q Bz, G0 (3), (sin th / cos th) cos phi, (sin th / cos th) sin phi (FP64:
-// KT = 10; FP32: each value twice, KT = 18, so FP32 passes run beam pairs as for the bulb model).
+// Table rows as Phys2's, with the azimuthal moment weights (sin th / cos th) cos phi and
+// (sin th / cos th) sin phi.
 template <typename Real>
 struct Phys2E {
   static constexpr bool kF32 = sizeof(Real) == 4;
   static constexpr bool kPairable = kF32;       // FP32 passes run beam pairs (PairRK)
-  static constexpr bool kNegated = false;       // no negated copies: rows stay small (many rows)
-  static constexpr int NC = 3, NG = 3, NM = 12, NSC = 14, KT = kF32 ? 18 : 10;
+  static constexpr int NC = 3, NG = 3, NM = 12, NSC = 14, KT = kF32 ? 12 : 10;
   static constexpr int kERows = Phys2<Real>::kERows;
-  // t1, q, q Bx, q Bz, G0 (3), then the azimuthal moment weights (sin th / cos th) cos phi and
-  // (sin th / cos th) sin phi; FP32 rows store each value twice (one 64-bit load per packed operand)
-  enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6, vSCC = 7, vSCS = 8 };
+  enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6, vSCC = 7, vSCS = 8, vT2 = 9 };   // FP64
+  enum : int { oNQBX = 0, oNG0X = 1, oQBZ = 2, oG0Z = 3, oG0Y = 4, oT1 = 5, oT2 = 6, oQ = 7, oSCC = 8, oSCS = 9, oH = 10 };   // FP32
   struct Consts { double B[3]; int n_phi; };
   using Beam = typename Phys2<Real>::Beam;
 
-  __device__ static inline Real val(const Real* t, int v) { return kF32 ? t[2 * v] : t[v]; }
-  __device__ static inline void put(Real* t, int v, Real x) {
-    if (kF32) { t[2 * v] = x; t[2 * v + 1] = x; } else { t[v] = x; }
-  }
-  __device__ static inline Real t1(const Real* t) { return val(t, vT1); }
-  // sc: mu D (3), mu J1 (3), mu Jc (3), mu Js (3), lambda
-  __device__ static inline void fill_row(Real* t, double u, double x, const double* sc, const Real* scr,
-                                         const Consts& C, int a, int) {
+  __device__ static inline Real t1(const Real* t) { return kF32 ? t[oT1] : t[vT1]; }
+  __device__ static inline void fill_geo(Real* t, double u, double x, const Consts& C, int a, Real hs) {
     const int pidx = a % C.n_phi;
-    Real q, t1v, t2, so, sp, cp;
     if constexpr (kF32) {
       // FP32 rows in FP32 arithmetic (as Phys2's): the table holds floats anyway, and FP64 square
       // roots, divisions and sincospi per row would cost more than the row's beams on GB300
+      float q, t1v, t2, sp, cp;
       geometry_f(u, x, q, t1v, t2);
-      so = sqrtf((float)(u * x)) * q;                         // sin th / cos th, sin^2 th = u R^2 / r^2
+      const float so = sqrtf((float)(u * x)) * q;             // sin th / cos th, sin^2 th = u R^2 / r^2
       sincospif((2.0f * pidx + 1.0f) / C.n_phi, &sp, &cp);   // phi_p = 2 pi (p + 1/2) / n_phi
+      const float hq = hs * q;
+      t[oNQBX] = -(hq * (float)C.B[0]);
+      t[oQBZ] = hq * (float)C.B[2];
+      t[oT1] = t1v;
+      t[oSCC] = so * cp;
+      t[oSCS] = so * sp;
+      t[oT2] = t2;
+      t[oQ] = hq;
+      t[oH] = hs;
     } else {
       const Geo g = geometry(u, x);
-      q = g.q;
-      t1v = g.t1;
-      t2 = g.t2;
-      so = sqrt(u * x) * g.q;
+      const double so = sqrt(u * x) * g.q;
+      double sp, cp;
       sincospi((2.0 * pidx + 1.0) / C.n_phi, &sp, &cp);
+      t[vT1] = g.t1;
+      t[vQ] = g.q;
+      t[vT2] = g.t2;
+      t[vQBX] = g.q * C.B[0];
+      t[vQBZ] = g.q * C.B[2];
+      t[vSCC] = so * cp;
+      t[vSCS] = so * sp;
     }
-    Real G0[3];
+  }
+  // sc: mu D (3), mu J1 (3), mu Jc (3), mu Js (3), lambda
+  __device__ static inline void fill_cpl(Real* t, const Real* sc) {
+    const Real q = kF32 ? t[oQ] : t[vQ], t2 = kF32 ? t[oT2] : t[vT2];
+    const Real scc = kF32 ? t[oH] * t[oSCC] : t[vSCC], scs = kF32 ? t[oH] * t[oSCS] : t[vSCS];
+    Real g[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      if constexpr (kF32) {
-        const float ext = cp * scr[6 + i] + sp * scr[9 + i];
-        G0[i] = q * ((i == 2 ? scr[12] : 0.0f) + scr[i] + t2 * scr[3 + i]) - so * ext;
-      } else {
-        const double ext = cp * sc[6 + i] + sp * sc[9 + i];
-        G0[i] = q * ((i == 2 ? sc[12] : 0.0) + sc[i] + t2 * sc[3 + i]) - so * ext;
-      }
+    for (int i = 0; i < 3; ++i)
+      g[i] = q * ((i == 2 ? sc[12] : Real(0)) + sc[i] + t2 * sc[3 + i]) - (scc * sc[6 + i] + scs * sc[9 + i]);
+    if constexpr (kF32) {
+      t[oNG0X] = -g[0];
+      t[oG0Z] = g[2];
+      t[oG0Y] = g[1];
+    } else {
+      t[vG0X] = g[0];
+      t[vG0Y] = g[1];
+      t[vG0Z] = g[2];
     }
-    const Real qbx = q * (Real)C.B[0], qbz = q * (Real)C.B[2];
-    put(t, vT1, t1v);
-    put(t, vQ, q);
-    put(t, vQBX, qbx);
-    put(t, vQBZ, qbz);
-    put(t, vG0X, G0[0]);
-    put(t, vG0Y, G0[1]);
-    put(t, vG0Z, G0[2]);
-    put(t, vSCC, so * cp);
-    put(t, vSCS, so * sp);
-    if constexpr (!kF32) t[9] = 0;
   }
   __device__ static inline void K(const Real* t, const Beam& bm, Real (&Kv)[3]) {
-    Kv[0] = bm.eo * val(t, vQBX) + val(t, vG0X);
-    Kv[1] = val(t, vG0Y);
-    Kv[2] = bm.eo * val(t, vQBZ) + val(t, vG0Z);
+    if constexpr (kF32) {
+      Kv[0] = -(bm.eo * t[oNQBX] + t[oNG0X]);
+      Kv[1] = t[oG0Y];
+      Kv[2] = bm.eo * t[oQBZ] + t[oG0Z];
+    } else {
+      Kv[0] = bm.eo * t[vQBX] + t[vG0X];
+      Kv[1] = t[vG0Y];
+      Kv[2] = bm.eo * t[vQBZ] + t[vG0Z];
+    }
   }
   __device__ static inline void f(const Real (&Kv)[3], const Real (&y)[3], Real (&k)[3]) {
     Phys2<Real>::f(Kv, y, k);
   }
   template <class Acc>
   __device__ static inline void accum_row(Acc& acc, Real w, const Real* t, const Real (&y)[3]) {
-    const Real wt = w * val(t, vT1), wc = w * val(t, vSCC), ws = w * val(t, vSCS);
+    const Real wt = w * t1(t), wc = w * (kF32 ? t[oSCC] : t[vSCC]), ws = w * (kF32 ? t[oSCS] : t[vSCS]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       acc.add(i, wt, y[i]);
@@ -714,26 +740,15 @@ __device__ __forceinline__ bool index_ok(const KParams& p, bool ok, int site, lo
 #define XFLAT_INDEX_OK(p, cond, site, v) true
 #endif
 
-// Add x (|x| < 2^63) to a 128-bit fixed-point accumulator (acc2[0]: fraction in units of 2^-64,
-// acc2[1]: signed integer part), truncating |x| below 2^-64.  The split is done on |x|, where
-// |x| - floor(|x|) is exact, and the pair is negated as a 128-bit integer for x < 0 (x - floor(x)
-// itself would round for small negative x).
+// Add x (|x| < 2^51) to a fixed-point accumulator of two signed words, acc2[1] in units of 2^-12 and
+// acc2[0] in units of 2^-64, truncating |x| below 2^-64: x = hi 2^-12 + lo 2^-64 exactly, |lo| < 2^52, so
+// hundreds of blocks cannot overflow a word, no carry passes between them and neither addition waits
+// for the other's result.
 __device__ __forceinline__ void fx_add(unsigned long long* acc2, double x) {
-  const double ax = fabs(x);
-  const double hi_d = floor(ax);
-  const unsigned long long lo_a = (unsigned long long)((ax - hi_d) * 18446744073709551616.0);
-  const long long hi_a = (long long)hi_d;
-  const bool neg = x < 0.0;
-  const unsigned long long lo = neg ? 0ull - lo_a : lo_a;
-  const long long hi = neg ? -hi_a - (lo_a != 0ull ? 1ll : 0ll) : hi_a;
-  const unsigned long long old = atomicAdd(&acc2[0], lo);
-  const unsigned long long carry = (old + lo < old) ? 1ull : 0ull;
-  atomicAdd(&acc2[1], (unsigned long long)hi + carry);
-}
-
-__device__ __forceinline__ double fx_read(const unsigned long long* acc2) {
-  const long long hi = (long long)acc2[1];
-  return (double)hi + (double)acc2[0] * 5.421010862427522e-20;   // 2^-64 (words already loaded)
+  const double hi_d = trunc(x * 4096.0);
+  const long long lo = (long long)((x * 4096.0 - hi_d) * 4503599627370496.0);        // exact difference, 2^52
+  atomicAdd(&acc2[0], (unsigned long long)lo);
+  atomicAdd(&acc2[1], (unsigned long long)(long long)hi_d);
 }
 
 template <class Tab>
@@ -808,14 +823,16 @@ __device__ __forceinline__ double acc_component(const unsigned long long* acc_sl
     for (int cp = 0; cp < kAccCopies; ++cp) sum += (long long)__ldcg(acc_slot + ((size_t)cp * kNMMax + c) * 2);
     return (double)sum * unit;                                   // 2^-S of the instance
   } else {
-    unsigned __int128 sum = 0;
+    long long hi = 0, lo = 0;
 #pragma unroll
     for (int cp = 0; cp < kAccCopies; ++cp) {
       const unsigned long long* w = acc_slot + ((size_t)cp * kNMMax + c) * 2;
-      sum += ((unsigned __int128)__ldcg(w + 1) << 64) | (unsigned __int128)__ldcg(w);
+      const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(w));
+      lo += (long long)v.x;
+      hi += (long long)v.y;
     }
-    return (double)(long long)(unsigned long long)(sum >> 64) +
-           (double)(unsigned long long)sum * 5.421010862427522e-20;    // 2^-64
+    const __int128 sum = ((__int128)hi << 52) + lo;                    // units of 2^-64
+    return (double)(long long)(sum >> 64) + (double)(unsigned long long)sum * 5.421010862427522e-20;
   }
 }
 
@@ -830,6 +847,100 @@ struct GeoHandoff {
 __device__ __forceinline__ GeoHandoff& geo_handoff() {
   __shared__ GeoHandoff g;
   return g;
+}
+
+// Sum of N values over a warp, the N results spread over its lanes: at each halving of the lane
+// distance a lane keeps one half of the values and hands the other half to its partner, so N = 6 takes 8
+// additions a lane instead of the 30 of six shuffle trees (18: 20 instead of 90; on GB300's two-lane
+// FP64 pipe every one costs the SM 16 cycles a warp).  Returns the sum of component *idx; *valid in the
+// one lane that reports it.
+template <int N, int O, typename T>
+__device__ __forceinline__ T reduce_scatter(T (&v)[N], int lane, int& idx, int& left, bool& valid) {
+  if constexpr (O == 0) {
+    valid = valid && left >= 1;
+    return v[0];
+  } else if constexpr (N == 1) {
+    T w[1] = {v[0] + __shfl_xor_sync(0xffffffffu, v[0], O)};
+    valid = valid && (lane & O) == 0;
+    return reduce_scatter<1, O / 2, T>(w, lane, idx, left, valid);
+  } else {
+    constexpr int H = (N + 1) / 2;
+    const bool up = (lane & O) != 0;
+    T w[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const T lo = v[i], hi = i + H < N ? v[i + H < N ? i + H : 0] : T(0);
+      w[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
+    }
+    idx += up ? H : 0;
+    left = up ? left - H : min(left, H);
+    return reduce_scatter<H, O / 2, T>(w, lane, idx, left, valid);
+  }
+}
+
+// Block sums of the threads' moment partials v (double, or integers of the instance's unit in the
+// mixed kernels) into one copy of the instance's accumulators: reduce-scatter in each warp, one
+// shared-memory row a warp, a half-warp tree a component over up to 16 warps, and one fixed-point
+// addition a component.  In a fixed order, so the result depends on the block decomposition only.
+// ovf: a thread's partial left the integer range (mixed).  A sum that is not finite or out of range
+// rejects an adaptive trial step (reject) and is fatal for a fixed step.
+template <int NM, typename T>
+__device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsigned long long* acc_copy,
+                                            unsigned long long* errmax, int* nonfinite, bool reject) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int idx = 0, left = NM;
+  bool valid = true;
+  const T s = reduce_scatter<NM, 16, T>(v, lane, idx, left, valid);
+  if (valid) red[warp * NM + idx] = s;
+  int any_ovf = 0;
+  if constexpr (sizeof(T) == 8 && T(0.5) == T(0)) any_ovf = __syncthreads_or(ovf);     // integers
+  else __syncthreads();
+  for (int t = threadIdx.x; t < NM * 16; t += blockDim.x) {
+    const int c = t >> 4, w = t & 15;
+    T x = w < nw ? red[w * NM + c] : T(0);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (w) continue;
+    bool ok;
+    if constexpr (T(0.5) == T(0)) {
+      ok = !any_ovf && x < kFixLimit && x > -kFixLimit;
+      if (ok) atomicAdd(acc_copy + 2 * c, (unsigned long long)x);
+    } else {
+      ok = fabs(x) <= 1.7e308;
+      if (ok) fx_add(acc_copy + 2 * c, x);
+    }
+    if (!ok) {
+      if (reject) atomicMax(errmax, 0x7ff0000000000000ull);
+      else atomicExch(nonfinite, 1);
+    }
+  }
+}
+
+// FP64 kernels share one copy of it over their passes (noinline): inlined, its code was out of the
+// instruction cache at every pass.
+template <int NM>
+__device__ __noinline__ void reduce_moments_shared(double (&v)[NM], double* red, unsigned long long* acc_copy,
+                                                   unsigned long long* errmax, int* nonfinite, bool reject) {
+  reduce_moments<NM, double>(v, 0, red, acc_copy, errmax, nonfinite, reject);
+}
+
+// The block's largest squared error ratio (FP32; infinity where not finite) and non-finite flag.
+__device__ __forceinline__ void reduce_error(float em, int bad, float* red, unsigned long long* errmax, int* nonfinite) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) em = fmaxf(em, __shfl_xor_sync(0xffffffffu, em, o));
+  if (lane == 0) red[warp] = em;
+  const int any_bad = __syncthreads_or(bad);
+  if (warp == 0) {
+    float m = lane < nw ? red[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+      if (any_bad) atomicExch(nonfinite, 1);
+      // the beams gave squared error ratios
+      atomicMax(errmax, (unsigned long long)__double_as_longlong(sqrt((double)m)));
+    }
+  }
 }
 
 template <class Phys, class Tab, typename Real>
@@ -1309,17 +1420,13 @@ __device__ __forceinline__ void propagate(const Real (&Om)[8], Real (&y)[9]) { p
 // Per-block shared state of the piece being processed.
 template <typename Real, class Phys>
 struct BlockShared {
-  double scd[kMaxStages][Phys::NSC];   // stage constants (double)
   double xs[kMaxStages];               // R^2 / r_s^2
-  unsigned long long hA2[kMaxStages][kMaxStages];   // packed (h a_ij, h a_ij) for the FP32 pair path
-  unsigned long long hB2[kMaxStages];
-  unsigned long long hE2[kMaxStages];
+  int t1max[kMaxStages];               // FP32 kernels: bits of the largest t1 of the piece's rows of a stage
   Real scr[kMaxStages][Phys::NSC];     // stage constants in working precision
-  Real hA[kMaxStages][kMaxStages];
+  Real hA[kMaxStages][kMaxStages];     // tableau coefficients times h (scaled_rows: the coefficients)
   Real hB[kMaxStages];
   Real hE[kMaxStages];
   Real rtol, atol;
-  double fx[kNMMax];
   int active;
   int parity;
   int flag;
@@ -1787,11 +1894,13 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
 
 // ----------------------------------------------------------------------------------------------
 // FP32 two-flavour beams in pairs with packed f32x2 arithmetic (Blackwell fma/mul.rn.f32x2).
-// A thread's two beams are consecutive energy bins of one angle bin, so every table value and step
-// coefficient is shared: it is stored duplicated and loaded as one 64-bit operand, while the
-// per-beam values (state, eta omega, weight) are packed once per pair.  Each packed instruction
-// does the work of two scalar ones, in the same order, so a pair gives the same bits as two
-// scalar beams would with contraction to FMA.
+// A thread's two beams are consecutive energy bins of one angle bin, so every table value is shared.
+// What bounds these passes (GB300, 4M beams, DP45): with the table values and step coefficients stored
+// twice, as packed operands, each pass moved about 110 128-byte wavefronts of shared memory a pair of
+// warps, and that, not the FMA pipe (45 % busy) or issue (45 %), set the time; scalar rows of h K with
+// compile-time coefficients, and moment sums of four operations a contribution instead of eight, took a
+// call of 12 steps from 3.19 to 2.70 ms (64 instances, 28M beams, 8 steps: 16.0 to 13.9 ms; 10
+// azimuthal bins, 4M beams, 8 steps: 3.07 to 2.51 ms).
 using F2 = unsigned long long;
 __device__ __forceinline__ F2 pk(float a, float b) {
   F2 r;
@@ -1821,14 +1930,12 @@ __device__ __forceinline__ F2 sub2(F2 a, F2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// two_sum_acc on a pair (each half one beam): hi + c split into the rounded sum and its exact
-// rounding error, collected in lo.
-__device__ __forceinline__ void two_sum_acc2(F2& hi, F2& lo, F2 c) {
-  const F2 s = add2(hi, c);
-  const F2 bv = sub2(s, hi);
-  const F2 err = add2(sub2(hi, sub2(s, bv)), sub2(c, bv));
+// biased_add on a pair (each half one beam)
+__device__ __forceinline__ void biased_add2(F2& hi, F2& lo, F2 w, F2 y) {
+  const F2 s = fma2(w, y, hi);
+  const F2 z = sub2(hi, s);
+  lo = add2(lo, fma2(w, y, z));
   hi = s;
-  lo = add2(lo, err);
 }
 // Moment accumulators of a thread's beam pairs: component i is the unevaluated sum hi[i] + lo[i].
 template <int NM>
@@ -1840,7 +1947,7 @@ struct PairAcc {
 template <int NM>
 struct PairHalfAcc {
   PairAcc<NM>& a;
-  __device__ __forceinline__ void add(int i, float w, float y) { two_sum_acc2(a.hi[i], a.lo[i], pk(__fmul_rn(w, y), 0.0f)); }
+  __device__ __forceinline__ void add(int i, float w, float y) { biased_add2(a.hi[i], a.lo[i], pk(w, 0.0f), pk(y, 0.0f)); }
 };
 
 template <class P, class Tab, int kPass, int kKind>
@@ -1850,40 +1957,46 @@ struct PairRK {
   static constexpr int kChain =
       kKind == kInitPass ? 0 : (kKind == kFinalPass ? Tab::S - (Tab::kAdaptive ? 1 : 0) : kPass + 1);
 
-  // K and -K of stage row R (packed values) for the pair's eta omega; -K_x and -K_z by one packed
-  // multiply by (-1, -1) each, -K_y = -G0_y from the row
-  __device__ static inline void Kpair(const F2* R, F2 eo, F2 (&K)[3], F2 (&nK)[3]) {
-    const F2 m1 = 0xbf800000bf800000ull;            // (-1.0f, -1.0f)
-    K[0] = fma2(eo, R[P::vQBX], R[P::vG0X]);
-    K[1] = R[P::vG0Y];
-    K[2] = fma2(eo, R[P::vQBZ], R[P::vG0Z]);
-    nK[0] = mul2(K[0], m1);
-    if constexpr (P::kNegated) nK[1] = R[P::vNG0Y];
-    else nK[1] = mul2(K[1], m1);
-    nK[2] = mul2(K[2], m1);
+  // h k = h K x Y of the row's stage.  The row's values are shared by the two beams and loaded once, as
+  // scalars (a value stored twice for a packed operand would cost the shared memory's 128 bytes a cycle
+  // twice over, which bound these kernels); the components of K that differ between the beams are made by
+  // two scalar FMAs straight into the halves of their operand.  Two components of k are kept with their
+  // signs reversed, (-k0, k1, -k2): then K enters as -K0, K2 and both signs of K1 only.
+  __device__ static inline void deriv(const float* R, float e0, float e1, const F2 (&Y)[3], F2 (&k)[3]) {
+    const float4 a = *reinterpret_cast<const float4*>(R);
+    const float g = R[P::oG0Y];
+    const F2 nK0 = pk(fmaf(e0, a.x, a.y), fmaf(e1, a.x, a.y)), K2 = pk(fmaf(e0, a.z, a.w), fmaf(e1, a.z, a.w));
+    const F2 K1 = pk(g, g), nK1 = pk(-g, -g);
+    k[0] = fma2(K2, Y[1], mul2(nK1, Y[2]));
+    k[1] = fma2(K2, Y[0], mul2(nK0, Y[2]));
+    k[2] = fma2(nK0, Y[1], mul2(K1, Y[0]));
   }
-  // k = K x Y as K1 Y2 - K2 Y1, ... with the products of -K added by FMA
-  __device__ static inline void cross(const F2 (&K)[3], const F2 (&nK)[3], const F2 (&Y)[3], F2 (&k)[3]) {
-    k[0] = fma2(K[1], Y[2], mul2(nK[2], Y[1]));
-    k[1] = fma2(K[2], Y[0], mul2(nK[0], Y[2]));
-    k[2] = fma2(K[0], Y[1], mul2(nK[1], Y[0]));
+  // Y + c k for k as deriv leaves it
+  __device__ static inline void axpy(double cd, const F2 (&k)[3], F2 (&Y)[3]) {
+    const float c = (float)cd;
+    const F2 cp = pk(c, c), cn = pk(-c, -c);
+    Y[0] = fma2(cn, k[0], Y[0]);
+    Y[1] = fma2(cp, k[1], Y[1]);
+    Y[2] = fma2(cn, k[2], Y[2]);
   }
   // moments of the pair's states with the weights of row R: D (w t1), J1 (w) and, extended model,
   // Jc (w (sin th / cos th) cos phi), Js (w (sin th / cos th) sin phi)
-  // (contributions formed in FP32, summed without loss: see MomAcc<float>)
-  __device__ static inline void accum(PairAcc<NM>& acc, F2 w, const F2* R, const F2 (&y)[3]) {
-    const F2 wt = mul2(w, R[P::vT1]);
+  // (summed without loss: see MomAcc<float>)
+  __device__ static inline void accum(PairAcc<NM>& acc, float w0, float w1, const float* R, const F2 (&y)[3]) {
+    const float t1 = R[P::oT1];
+    const F2 w = pk(w0, w1), wt = pk(w0 * t1, w1 * t1);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      two_sum_acc2(acc.hi[i], acc.lo[i], mul2(wt, y[i]));
-      two_sum_acc2(acc.hi[3 + i], acc.lo[3 + i], mul2(w, y[i]));
+      biased_add2(acc.hi[i], acc.lo[i], wt, y[i]);
+      biased_add2(acc.hi[3 + i], acc.lo[3 + i], w, y[i]);
     }
     if constexpr (NM == 12) {
-      const F2 wc = mul2(w, R[P::vSCC]), ws = mul2(w, R[P::vSCS]);
+      const float sc = R[P::oSCC], ss = R[P::oSCS];
+      const F2 wc = pk(w0 * sc, w1 * sc), ws = pk(w0 * ss, w1 * ss);
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        two_sum_acc2(acc.hi[6 + i], acc.lo[6 + i], mul2(wc, y[i]));
-        two_sum_acc2(acc.hi[9 + i], acc.lo[9 + i], mul2(ws, y[i]));
+        biased_add2(acc.hi[6 + i], acc.lo[6 + i], wc, y[i]);
+        biased_add2(acc.hi[9 + i], acc.lo[9 + i], ws, y[i]);
       }
     }
   }
@@ -1905,11 +2018,11 @@ struct PairRK {
     for (int i = 0; i < 3; ++i) y[i] = mul2(y[i], inv);
   }
 
-  // rows: table rows of this pair's angle bin, stage s at rows + s * rstride (in F2 units);
-  // y, ep as in PassBody::beam
+  // e0, e1, w0, w1: eta omega and weights of the two beams; rows: table rows of their angle bin, stage s
+  // at rows + s * rstride; y as in PassBody::beam
   template <class BS>
-  __device__ static inline void run(const BS& bs, F2 eo, F2 w, const F2* rows, int rstride, F2 (&y)[3],
-                                    F2 (&ep)[4], PairAcc<NM>& acc, float& emax, int& bad) {
+  __device__ static inline void run(const BS& bs, float e0, float e1, float w0, float w1, const float* rows, int rstride,
+                                    F2 (&y)[3], PairAcc<NM>& acc, float& emax, int& bad) {
     F2 k[Tab::S + 1][3];
     // adaptive final pass: y5 and the error accumulate as soon as each stage derivative exists
     // (same order of operations as summing after the chain), so the derivatives die early
@@ -1921,29 +2034,19 @@ struct PairRK {
       F2 Y[3] = {y[0], y[1], y[2]};
 #pragma unroll
       for (int m = 1; m < l; ++m)
-        if (Tab::a(l, m) != 0.0) {
-          const F2 ha = bs.hA2[l][m];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) Y[i] = fma2(ha, k[m][i], Y[i]);
-        }
-      F2 K[3], nK[3];
-      Kpair(rows + l * rstride, eo, K, nK);
-      cross(K, nK, Y, k[l]);
+        if (Tab::a(l, m) != 0.0) axpy(Tab::a(l, m), k[m], Y);
+      deriv(rows + l * rstride, e0, e1, Y, k[l]);
       if (kFinalAdaptive) {
-        if (Tab::b(l) != 0.0) {
-          const F2 hb = bs.hB2[l];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) yn[i] = fma2(hb, k[l][i], yn[i]);
-        }
-        if (Tab::e(l) != 0.0) {
-          const F2 he = bs.hE2[l];
+        if (Tab::b(l) != 0.0) axpy(Tab::b(l), k[l], yn);
+        if (Tab::e(l) != 0.0) {            // the error's components carry the signs of k
+          const F2 he = pk((float)Tab::e(l), (float)Tab::e(l));
 #pragma unroll
           for (int i = 0; i < 3; ++i) e[i] = fma2(he, k[l][i], e[i]);
         }
       }
     }
     if (kKind == kInitPass) {
-      accum(acc, w, rows + rstride * 1, y);
+      accum(acc, w0, w1, rows + rstride * 1, y);
       return;
     }
     if (kKind == kStagePass) {
@@ -1951,13 +2054,9 @@ struct PairRK {
       F2 Y[3] = {y[0], y[1], y[2]};
 #pragma unroll
       for (int m = 1; m < I; ++m)
-        if (Tab::a(I, m) != 0.0) {
-          const F2 ha = bs.hA2[I][m];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) Y[i] = fma2(ha, k[m][i], Y[i]);
-        }
+        if (Tab::a(I, m) != 0.0) axpy(Tab::a(I, m), k[m], Y);
       if (Tab::kAdaptive && I == Tab::S) normalise(Y);
-      accum(acc, w, rows + rstride * I, Y);
+      accum(acc, w0, w1, rows + rstride * I, Y);
       return;
     }
     if (Tab::kAdaptive) {
@@ -1979,11 +2078,9 @@ struct PairRK {
 #pragma unroll
         for (int i = 0; i < 3; ++i) yn[i] = mul2(yn[i], inv);
       }
-      F2 K[3], nK[3];
-      Kpair(rows + Tab::S * rstride, eo, K, nK);
-      cross(K, nK, yn, k[Tab::S]);
+      deriv(rows + Tab::S * rstride, e0, e1, yn, k[Tab::S]);
       if (Tab::e(Tab::S) != 0.0) {
-        const F2 he = bs.hE2[Tab::S];
+        const F2 he = pk((float)Tab::e(Tab::S), (float)Tab::e(Tab::S));
 #pragma unroll
         for (int i = 0; i < 3; ++i) e[i] = fma2(he, k[Tab::S][i], e[i]);
       }
@@ -2012,18 +2109,14 @@ struct PairRK {
     // final pass of a fixed-step tableau
 #pragma unroll
     for (int m = 1; m <= kChain; ++m)
-      if (Tab::b(m) != 0.0) {
-        const F2 hb = bs.hB2[m];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) yn[i] = fma2(hb, k[m][i], yn[i]);
-      }
+      if (Tab::b(m) != 0.0) axpy(Tab::b(m), k[m], yn);
     float a0[3], a1[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) upk(yn[i], a0[i], a1[i]);
     const bool ok0 = 0.5f * (a0[0] * a0[0] + a0[1] * a0[1] + a0[2] * a0[2]) <= 3.0e38f;
     const bool ok1 = 0.5f * (a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2]) <= 3.0e38f;
     if (ok0 && ok1) normalise(yn);
-    accum(acc, w, rows + rstride * Tab::S, yn);
+    accum(acc, w0, w1, rows + rstride * Tab::S, yn);
 #pragma unroll
     for (int i = 0; i < 3; ++i) y[i] = yn[i];
   }
@@ -2033,9 +2126,16 @@ struct PairRK {
 template <typename Real>
 __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int k, Real du,
                                           typename Phys2<Real>::Beam& bm) {
-  const Real om = et[k];
-  bm.eo = sigma ? -om : om;
-  bm.w = du * et[(1 + sigma) * ne + k];
+  if constexpr (sizeof(Real) == 4) {
+    // one 128-bit entry a bin: omega, weights of nu and nubar, pad
+    const float4 v = *reinterpret_cast<const float4*>(et + 4 * (size_t)k);
+    bm.eo = sigma ? -v.x : v.x;
+    bm.w = du * (sigma ? v.z : v.y);
+  } else {
+    const Real om = et[k];
+    bm.eo = sigma ? -om : om;
+    bm.w = du * et[(1 + sigma) * ne + k];
+  }
 }
 template <typename Real>
 __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int k, Real du,
@@ -2055,10 +2155,12 @@ template <class Body, int NC, typename Real>
 __device__ __forceinline__ bool beam_in_bounds(const KParams& p, const Real* et, int ne, int k, int tj,
                                                int n_jj, const Real* kst_beam) {
 #ifdef XFLAT_BOUNDS
-  constexpr int kERowMax = (NC == 3 ? Phys2<Real>::kERows : Phys3<Real>::kERows) - 1;
+  constexpr int kERowMax = (NC == 3 ? Phys2<double>::kERows : Phys3<Real>::kERows) - 1;
   bool ok = index_ok(p, tj >= 0 && tj < n_jj, 12, tj) && index_ok(p, k >= 0 && k < ne, 10, k) &&
-            span_ok(p, kSpanEtab, et + k, sizeof(Real), 10) &&
-            span_ok(p, kSpanEtab, et + (size_t)kERowMax * ne + k, sizeof(Real), 11);
+            (NC == 3 && sizeof(Real) == 4
+                 ? span_ok(p, kSpanEtab, et + 4 * (size_t)k, 16, 10)
+                 : span_ok(p, kSpanEtab, et + k, sizeof(Real), 10) &&
+                       span_ok(p, kSpanEtab, et + (size_t)kERowMax * ne + k, sizeof(Real), 11));
   if constexpr (Body::kStore)
     ok = ok && span_ok(p, kSpanKst, kst_beam, sizeof(Real), 8) &&
          span_ok(p, kSpanKst, kst_beam + ((size_t)(Body::kYPlanes + 1) * NC - 1) * p.plane_stride,
@@ -2069,6 +2171,17 @@ __device__ __forceinline__ bool beam_in_bounds(const KParams& p, const Real* et,
 #endif
 }
 
+// Dynamic shared memory: reduction scratch, the table rows, the angle weights, the angle positions
+// (8-byte aligned) and the state rings.
+template <typename Real>
+__device__ __forceinline__ Real* table_smem(unsigned char* dyn_smem) {
+  return reinterpret_cast<Real*>(dyn_smem + 32 * kNMMax * sizeof(double));
+}
+template <typename Real>
+__device__ __forceinline__ double* angle_smem(Real* after_weights) {
+  return reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(after_weights) + 7) & ~uintptr_t(7));
+}
+
 // Stages whose table rows a pass reads (bit s set: row s needed).
 template <class Tab, int kPass, int kKind>
 __device__ __forceinline__ unsigned stages_needed() {
@@ -2077,19 +2190,152 @@ __device__ __forceinline__ unsigned stages_needed() {
   return ((1u << (kPass + 3)) - 1u) & ~1u;                                      // 1..kPass+2
 }
 
+// FP32 commutator kernels tabulate h K instead of K, so that the tableau's coefficients are compile-time
+// constants of their pass bodies (shared memory's bandwidth bounds them, see PairRK::deriv).
+template <typename Real, bool kCF>
+__host__ __device__ constexpr bool scaled_rows() { return sizeof(Real) == 4 && !kCF; }
+
+// Set-up of a piece for a pass: flags, step size, coefficients, stage constants and the table rows.
+// newest: the stage whose moments the previous pass reduced (0: none of this step); every block derives
+// its constants mu m (and lambda) from the accumulators itself (integer sums: the same bits everywhere),
+// so that barrier needs no serial section, and the block holding the instance's first beams records
+// them for later passes and the host.  need: stages whose rows the pass reads.  single: the block's only
+// piece, whose set-up stays in shared memory for the whole step: pass 0 fills the geometry of every
+// stage's rows, and after it (incremental) only the newest stage's couplings are still to come.
+// One copy of this code serves every pass of a kernel (instruction cache).
+template <class Phys, class Tab, typename Real, bool kCF>
+__device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phys>& bs, unsigned char* dyn_smem, int pi,
+                                         int newest, unsigned need, bool incremental, bool single) {
+  constexpr int kTS = Tab::S + 1;                                    // table stage slots 0..S
+  Real* tab = table_smem<Real>(dyn_smem);                            // [kTS][max_jj][KT]
+  Real* dut = tab + (size_t)kTS * p.max_jj * Phys::KT;               // [max_jj]
+  double* ut = angle_smem(dut + p.max_jj);                           // [max_jj]
+  const Piece pc = p.pieces[pi];
+  const InstConst& ic = p.ic[pc.inst];
+  const InstDyn* d = p.dyn + pc.inst;
+  const int n_jj = pc.n_jj;
+  // constant c of the newest stage
+  auto newest_constant = [&](int c) {
+    const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)newest * kAccCopies * kNMMax * 2;
+    InstDyn* dw = p.dyn + pc.inst;
+    double v = 0.0;
+    if (c < Phys::NM) {
+      const double m = acc_component<Real>(accs, c, ic.acc_unit);
+      v = ldcg(&d->mus[newest]) * m;
+      if (pc.start == ic.rec_start) dw->mom[newest][c] = m;
+    } else if (c == Phys::NM) {
+      v = ldcg(&d->lams[newest]);
+    }
+    if (pc.start == ic.rec_start && c <= Phys::NM) dw->sc[newest][c] = v;
+    return v;
+  };
+  __syncthreads();
+  if (incremental) {
+    if (threadIdx.x < Phys::NSC) bs.scr[newest][threadIdx.x] = (Real)newest_constant(threadIdx.x);
+    __syncthreads();
+    for (int tj = threadIdx.x; tj < n_jj; tj += blockDim.x)
+      Phys::fill_cpl(tab + ((size_t)newest * n_jj + tj) * Phys::KT, bs.scr[newest]);
+    __syncthreads();
+    return;
+  }
+  // one parallel load phase (every load issued before any of them is used, so the phase costs one L2
+  // round trip)
+  if (threadIdx.x == 0) {
+    const int dn = ldcg(&d->done), st = ldcg(&d->status), par = ldcg(&d->parity);
+    bs.active = (dn == 0 && st == 0) ? 1 : 0;
+    bs.parity = par;
+  }
+  const double h = Tab::kAdaptive ? ldcg(&d->h) : ldcg(&d->h_fixed);
+  for (int t = threadIdx.x; t < kTS * Phys::NSC; t += blockDim.x) {
+    const int s = t / Phys::NSC, c = t % Phys::NSC;
+    double v = 0.0;
+    if (s == newest) v = newest_constant(c);
+    else if ((need >> s) & 1u) v = ldcg(&d->sc[s][c]);
+    bs.scr[s][c] = (Real)v;
+  }
+  if (threadIdx.x < kMaxStages) {
+    bs.xs[threadIdx.x] = ldcg(&d->xs[threadIdx.x]);
+    bs.t1max[threadIdx.x] = 0;
+  }
+  if constexpr (kCF) {
+    if (threadIdx.x == 0) bs.hB[0] = (Real)h;
+  } else {
+    // the non-zero coefficients of the tableau, one a thread: (i, j) of a, then b_j, then e_j
+    constexpr int kA = Tab::S + 1, kCoef = kA * kA + 2 * kA;
+    for (int t = threadIdx.x; t < kCoef; t += blockDim.x) {
+      double v = 0.0;
+#pragma unroll
+      for (int i = 1; i < kA; ++i)
+#pragma unroll
+        for (int j = 1; j < kA; ++j)
+          if (Tab::a(i, j) != 0.0) v = t == i * kA + j ? Tab::a(i, j) : v;
+#pragma unroll
+      for (int j = 1; j < kA; ++j) {
+        if (Tab::b(j) != 0.0) v = t == kA * kA + j ? Tab::b(j) : v;
+        if (Tab::e(j) != 0.0) v = t == kA * kA + kA + j ? Tab::e(j) : v;
+      }
+      const Real hv = (Real)(scaled_rows<Real, kCF>() ? v : h * v);
+      if (t < kA * kA) bs.hA[t / kA][t % kA] = hv;
+      else if (t < kA * kA + kA) bs.hB[t - kA * kA] = hv;
+      else bs.hE[t - kA * kA - kA] = hv;
+    }
+  }
+  // launch-invariant part (tolerances, angle tables): a single-piece block loads it once per launch
+  if (!(single && bs.keep)) {
+    if (threadIdx.x == 0) {
+      bs.rtol = (Real)ic.rtol;
+      bs.atol = (Real)ic.atol;
+    }
+    for (int t = threadIdx.x; t < n_jj; t += blockDim.x) {
+      const int jj = pc.jj_lo + t;
+      const int j = jj >= (int)ic.n_angle ? jj - (int)ic.n_angle : jj;
+      if (!(XFLAT_INDEX_OK(p, j >= 0 && j < (int)ic.n_angle, 15, jj) &&
+            XFLAT_SPAN_OK(p, kSpanDu, p.du_tab + ic.a_off + j, sizeof(double), 16) &&
+            XFLAT_SPAN_OK(p, kSpanU, p.u_tab + ic.a_off + j, sizeof(double), 16))) {
+        dut[t] = Real(0);
+        ut[t] = 0.0;
+        continue;
+      }
+      dut[t] = (Real)p.du_tab[ic.a_off + j];
+      ut[t] = p.u_tab[ic.a_off + j];
+    }
+  }
+  __syncthreads();
+  if (single && threadIdx.x == 0) bs.keep = 1;       // read after later barriers only
+  if (!bs.active) return;
+  typename Phys::Consts C;
+  if constexpr (Phys::NC == 3) {
+    C.B[0] = ic.B[0]; C.B[1] = ic.B[1]; C.B[2] = ic.B[2];
+    if constexpr (Phys::NM == 12) C.n_phi = (int)ic.n_phi;
+    else C.geom = ic.geom;
+  } else {
+    C.geom = ic.geom;
+  }
+  const unsigned geo = single && !p.shard_mode ? ((1u << kTS) - 1u) & ~1u : need;
+  for (int t = threadIdx.x; t < kTS * n_jj; t += blockDim.x) {
+    const int s = t / n_jj, tj = t % n_jj;
+    if (!((geo >> s) & 1u)) continue;
+    Real* row = tab + ((size_t)s * n_jj + tj) * Phys::KT;
+    const int jj = (int)pc.jj_lo + tj;
+    const int a = jj >= (int)ic.n_angle ? jj - (int)ic.n_angle : jj;     // angle bin of its species
+    Phys::fill_geo(row, ut[tj], bs.xs[s], C, a, scaled_rows<Real, kCF>() ? (Real)h : Real(1));
+    if constexpr (sizeof(Real) == 4) atomicMax(&bs.t1max[s], __float_as_int(Phys::t1(row)));   // t1 >= 0
+    if ((need >> s) & 1u) Phys::fill_cpl(row, bs.scr[s]);
+  }
+  __syncthreads();
+}
+
 // One pass over all pieces of this block.
 template <class Phys, class Tab, typename Real, bool kCF, int kPass, int kKind>
 __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned char* dyn_smem) {
   constexpr int NC = Phys::NC, NM = Phys::NM, VN = Vec16<Real>::N;
   using Body = PassBody<Phys, Tab, Real, kCF, kPass, kKind>;
-  double* red = reinterpret_cast<double*>(dyn_smem);                 // 32 * NM doubles
+  double* red = reinterpret_cast<double*>(dyn_smem);                 // 32 * kNMMax doubles
   constexpr int kTS = Tab::S + 1;                                    // table stage slots 0..S
-  Real* tab = reinterpret_cast<Real*>(red + 32 * kNMMax);            // [kTS][max_jj][KT]
+  Real* tab = table_smem<Real>(dyn_smem);                            // [kTS][max_jj][KT]
   Real* dut = tab + (size_t)kTS * p.max_jj * Phys::KT;               // [max_jj]
-  double* ut = reinterpret_cast<double*>(                            // [max_jj], 8-byte aligned
-      (reinterpret_cast<uintptr_t>(dut + p.max_jj) + 7) & ~uintptr_t(7));
   float* ring = reinterpret_cast<float*>(                            // [slots][NC][threads][2], 16-byte aligned
-      (reinterpret_cast<uintptr_t>(ut + p.max_jj) + 15) & ~uintptr_t(15));
+      (reinterpret_cast<uintptr_t>(angle_smem(dut + p.max_jj) + p.max_jj) + 15) & ~uintptr_t(15));
   const bool mixed = sizeof(Real) == 4;
   const int slot = kKind == kInitPass ? 1 : (kKind == kStagePass ? kPass + 2 : 0);
   // Clear accumulator slots nobody reads any more (block 0, while the other blocks already work).
@@ -2116,9 +2362,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
   constexpr int kNewest = (kKind != kInitPass && kPass >= 1) ? kPass + 1 : 0;
   const bool dyn = p.dyn_sched != 0;
   const int b0 = dyn ? 0 : p.blk_piece[blockIdx.x], b1 = dyn ? 0 : p.blk_piece[blockIdx.x + 1];
-  // A block with a single piece keeps its set-up in shared memory for the whole step: after pass
-  // 0 only the newest stage's constants and the table rows of the newest and the formed stage
-  // change (flags, step size, coefficients, radii, angle tables and older rows stay valid).
+  // a block with a single piece keeps its set-up in shared memory for the whole step (setup_piece)
   const bool single = !dyn && b1 - b0 == 1;
   const bool incremental = single && kNewest >= 1 && !p.shard_mode;
   for (int it = 0;; ++it) {
@@ -2138,127 +2382,9 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
                                (uint64_t)pc.start + pc.len <= p.ic[pc.inst].n_beams, 14, pi))
       continue;
     const InstConst& ic = p.ic[pc.inst];
-    const InstDyn* d = p.dyn + pc.inst;
-    __syncthreads();
-    if (incremental) {
-      if (threadIdx.x < Phys::NSC) {
-        const int c = threadIdx.x;
-        double v = 0.0;
-        const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst +
-                                         (size_t)kNewest * kAccCopies * kNMMax * 2;
-        InstDyn* dw = p.dyn + pc.inst;
-        if (c < Phys::NM) {
-          const double m = acc_component<Real>(accs, c, ic.acc_unit);
-          v = ldcg(&d->mus[kNewest]) * m;
-          if (pc.start == ic.rec_start) dw->mom[kNewest][c] = m;
-        } else if (c == Phys::NM) {
-          v = ldcg(&d->lams[kNewest]);
-        }
-        if (pc.start == ic.rec_start && c <= Phys::NM) dw->sc[kNewest][c] = v;
-        bs.scd[kNewest][c] = v;
-        bs.scr[kNewest][c] = (Real)v;
-      }
-      __syncthreads();
-    }
-    if (!incremental) {
-    // one parallel load phase: flags, step size, stage constants, radii, angle weights (every
-    // load issued before any of them is used, so the phase costs one L2 round trip)
-    if (threadIdx.x == 0) {
-      const int dn = ldcg(&d->done), st = ldcg(&d->status), par = ldcg(&d->parity);
-      bs.active = (dn == 0 && st == 0) ? 1 : 0;
-      bs.parity = par;
-    }
-    const double h = Tab::kAdaptive ? ldcg(&d->h) : ldcg(&d->h_fixed);
-    for (int t = threadIdx.x; t < kTS * Phys::NSC; t += blockDim.x) {
-      const int s = t / Phys::NSC, c = t % Phys::NSC;
-      double v = 0.0;
-      if (s == kNewest) {
-        // the stage reduced by the previous pass: every block derives its constants mu m (and
-        // lambda) from the accumulators itself (integer sums: the same bits everywhere), so that
-        // barrier needs no serial section; the block holding the instance's first beams records
-        // the moments and constants for later passes and the host
-        const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst +
-                                         (size_t)s * kAccCopies * kNMMax * 2;
-        InstDyn* dw = p.dyn + pc.inst;
-        if (c < Phys::NM) {
-          const double m = acc_component<Real>(accs, c, ic.acc_unit);
-          v = ldcg(&d->mus[s]) * m;
-          if (pc.start == ic.rec_start) dw->mom[s][c] = m;
-        } else if (c == Phys::NM) {
-          v = ldcg(&d->lams[s]);
-        }
-        if (pc.start == ic.rec_start && c <= Phys::NM) dw->sc[s][c] = v;
-      } else if ((need >> s) & 1u) {
-        v = ldcg(&d->sc[s][c]);
-      }
-      bs.scd[s][c] = v;
-      bs.scr[s][c] = (Real)v;
-    }
-    if (threadIdx.x < kMaxStages) bs.xs[threadIdx.x] = ldcg(&d->xs[threadIdx.x]);
-    for (int t = threadIdx.x; t < kMaxStages * kMaxStages; t += blockDim.x) {
-      const int i = t / kMaxStages, j = t % kMaxStages;
-      bs.hA[i][j] = (Real)(h * ((i >= 1 && j >= 1) ? Tab::a(i, j) : 0.0));
-      const float fa = (float)bs.hA[i][j];
-      bs.hA2[i][j] = pk(fa, fa);
-    }
-    if (threadIdx.x < kMaxStages) {
-      const int i = threadIdx.x;
-      if (kCF) {
-        bs.hB[i] = (Real)h;
-        bs.hE[i] = 0;
-      } else {
-        bs.hB[i] = (Real)(h * (i >= 1 ? Tab::b(i) : 0.0));
-        bs.hE[i] = (Real)(h * (i >= 1 ? Tab::e(i) : 0.0));
-      }
-      const float fb = (float)bs.hB[i], fe = (float)bs.hE[i];
-      bs.hB2[i] = pk(fb, fb);
-      bs.hE2[i] = pk(fe, fe);
-    }
-    // launch-invariant part (tolerances, angle tables): a single-piece block
-    // loads it once per launch
-    if (!(single && bs.keep)) {
-      if (threadIdx.x == 0) {
-        bs.rtol = (Real)ic.rtol;
-        bs.atol = (Real)ic.atol;
-      }
-      for (int t = threadIdx.x; t < (int)pc.n_jj; t += blockDim.x) {
-        const int jj = pc.jj_lo + t;
-        const int j = jj >= (int)ic.n_angle ? jj - (int)ic.n_angle : jj;
-        if (!(XFLAT_INDEX_OK(p, j >= 0 && j < (int)ic.n_angle, 15, jj) &&
-              XFLAT_SPAN_OK(p, kSpanDu, p.du_tab + ic.a_off + j, sizeof(double), 16) &&
-              XFLAT_SPAN_OK(p, kSpanU, p.u_tab + ic.a_off + j, sizeof(double), 16))) {
-          dut[t] = Real(0);
-          ut[t] = 0.0;
-          continue;
-        }
-        dut[t] = (Real)p.du_tab[ic.a_off + j];
-        ut[t] = p.u_tab[ic.a_off + j];
-      }
-    }
-    __syncthreads();
-    if (single && threadIdx.x == 0) bs.keep = 1;     // read after later barriers only
-    }
-    const int n_jj = pc.n_jj;
+    setup_piece<Phys, Tab, Real, kCF>(p, bs, dyn_smem, pi, kNewest, need, incremental, single);
     if (!bs.active) continue;
-    typename Phys::Consts C;
-    if constexpr (Phys::NC == 3) {
-      C.B[0] = ic.B[0]; C.B[1] = ic.B[1]; C.B[2] = ic.B[2];
-      if constexpr (Phys::NM == 12) C.n_phi = (int)ic.n_phi;
-      else C.geom = ic.geom;
-    } else {
-      C.geom = ic.geom;
-    }
-    // table rows: every needed stage, or (incremental) only the newest and the formed stage
-    const unsigned fill = incremental ? (need & (3u << kNewest)) : need;
-    for (int t = threadIdx.x; t < kTS * n_jj; t += blockDim.x) {
-      const int s = t / n_jj, tj = t % n_jj;
-      if (!((fill >> s) & 1u)) continue;
-      Real* row = tab + ((size_t)s * n_jj + tj) * Phys::KT;
-      const int jj = (int)pc.jj_lo + tj;
-      const int a = jj >= (int)ic.n_angle ? jj - (int)ic.n_angle : jj;     // angle bin of its species
-      Phys::fill_row(row, ut[tj], bs.xs[s], bs.scd[s], bs.scr[s], C, a, 0);
-    }
-    __syncthreads();
+    const int n_jj = pc.n_jj;
     const TabView<Real, Phys> tv{tab, n_jj};
     const Real* et = reinterpret_cast<const Real*>(p.etab) + ic.e_off;
     const Real* yin = reinterpret_cast<const Real*>(bs.parity ? p.planeB : p.planeA) + ic.beam_off;
@@ -2271,15 +2397,32 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     Real* kst = Body::kStore ? reinterpret_cast<Real*>(p.kst) + ic.beam_off : nullptr;
     const Real* ysrc = kSplitLoad ? yout : yin;
     const int ne = (int)ic.n_energy, na = (int)ic.n_angle;
+    // biases of the mixed sums: a thread adds at most 2 (its + 1) contributions of |w| <= wmax (times the
+    // geometry factor), |Y| <= 2, to an accumulator
+    auto biases = [&](float (&bias)[NM / NC]) {
+      if constexpr (sizeof(Real) == 4) {
+        constexpr int kMomRow = kKind == kInitPass ? 1 : (kKind == kStagePass ? kPass + 2 : Tab::S);
+        const float t1m = __int_as_float(bs.t1max[kMomRow]);
+        const float P = 4.0f * (float)(pc.len / (VN * blockDim.x) + 2u) * ic.wmax;
+        bias[0] = sum_bias(P * t1m);
+        bias[1] = sum_bias(P);
+        if constexpr (NM / NC == 4) bias[2] = bias[3] = sum_bias(P * sqrtf(t1m * (t1m + 2.0f)));   // tan th
+      }
+    };
+    float bias[NM / NC];
+    biases(bias);
     MomAcc<Real, NM> acc;
-    acc.zero();
+    acc.start(bias, NC);
     Real emax = 0;
     int bad = 0;
     // FP32 two-flavour RK passes run beam pairs on packed f32x2 arithmetic (PairRK)
     constexpr bool kPair = Phys::kPairable && !kCF;
     PairAcc<NM> acc2;
 #pragma unroll
-    for (int i = 0; i < NM; ++i) { acc2.hi[i] = 0ull; acc2.lo[i] = 0ull; }
+    for (int i = 0; i < NM; ++i) {
+      if constexpr (kPair) acc2.hi[i] = pk(bias[i / NC], bias[i / NC]);
+      acc2.lo[i] = 0ull;
+    }
     float emax2 = 0.0f;
     const uint32_t end = pc.start + pc.len;
     const uint32_t vstep = VN * blockDim.x;
@@ -2359,22 +2502,13 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
           typename Phys2<float>::Beam b0, b1;
           load_beam<float>(et, ne, sigma, k, dut[tj], b0);
           load_beam<float>(et, ne, sigma, k + 1, dut[tj], b1);
-          F2 y2[3], ep2[4];
+          F2 y2[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) y2[c] = pk(ys[c][0], ys[c][1]);
-          if constexpr (kSplitLoad) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) ep2[c] = pk(ep[c][0], ep[c][1]);
-          }
-          const F2* rows = reinterpret_cast<const F2*>(tab) + (size_t)tj * (Phys::KT / 2);
-          PairRK<Phys, Tab, kPass, kKind>::run(bs, pk(b0.eo, b1.eo), pk(b0.w, b1.w), rows,
-                                         n_jj * (Phys::KT / 2), y2, ep2, acc2, emax2, bad);
+          PairRK<Phys, Tab, kPass, kKind>::run(bs, b0.eo, b1.eo, b0.w, b1.w, tab + (size_t)tj * Phys::KT, n_jj * Phys::KT, y2,
+                                               acc2, emax2, bad);
 #pragma unroll
           for (int c = 0; c < 3; ++c) upk(y2[c], ys[c][0], ys[c][1]);
-          if constexpr (kSplitStore) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) upk(ep2[c], ep[c][0], ep[c][1]);
-          }
         }
       }
       if (!paired) {
@@ -2435,69 +2569,37 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     constexpr bool kErrMax = kKind == kFinalPass && Tab::kAdaptive;
     constexpr bool kMoments = kKind != kFinalPass || Tab::kFinalMoments;
     constexpr bool kRejectOverflow = Tab::kAdaptive;
+    unsigned long long* acc_copy = p.acc + (size_t)pc.inst * kAccWordsPerInst +
+                                   ((size_t)slot * kAccCopies + blockIdx.x % kAccCopies) * kNMMax * 2;
     if constexpr (sizeof(Real) == 4) {
       // mixed precision: each thread's (hi, lo) partial sums go to integers of the instance's
-      // acc_unit; the warp shuffle trees, the sum over warps and the accumulator atomics are
-      // integer additions (exact, order-free).  A thread or block partial of 2^52 units or more
-      // (only a runaway or non-finite state reaches it) rejects an adaptive trial step and is
-      // fatal for a fixed step.  The error maximum is a max (exact); the square root of the
-      // block's maximum is taken in double.
-      const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-      float* redf = reinterpret_cast<float*>(red);
-      if constexpr (kErrMax) {
-        float em = (emax <= 3.0e38f) ? (float)emax : INFINITY;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) em = fmaxf(em, __shfl_down_sync(0xffffffffu, em, o));
-        if (lane == 0) redf[warp] = em;
-        const int any_bad = __syncthreads_or(bad);
-        if (threadIdx.x == 0) {
-          float m = 0.0f;
-          for (int w = 0; w < nw; ++w) m = fmaxf(m, redf[w]);
-          if (any_bad) atomicExch(&p.nonfinite[pc.inst], 1);
-          // the beams gave squared error ratios
-          atomicMax(&p.errmax[pc.inst], (unsigned long long)__double_as_longlong(sqrt((double)m)));
-        }
-      }
+      // acc_unit, and every further sum is an integer addition (exact, order-free).  A thread or block
+      // partial of 2^52 units or more (only a runaway or non-finite state reaches it) rejects an
+      // adaptive trial step and is fatal for a fixed step.  The error maximum is a max (exact); the
+      // square root of the block's maximum is taken in double.
+      if constexpr (kErrMax)
+        reduce_error((emax <= 3.0e38f) ? (float)emax : INFINITY, bad, reinterpret_cast<float*>(red), &p.errmax[pc.inst],
+                     &p.nonfinite[pc.inst]);
       if constexpr (kMoments) {
         if constexpr (kErrMax) __syncthreads();              // the scratch is reused
-        long long* redl = reinterpret_cast<long long*>(red);  // [warp][NM]
         int ovf = 0;
+        long long v[NM];
+        float bias[NM / NC];                                 // again, not held over the loop
+        biases(bias);
 #pragma unroll
         for (int i = 0; i < NM; ++i) {
-          // the thread's partial (pair halves and scalar accumulator joined by TwoSum), then a warp
-          // shuffle tree on the (hi, lo) pairs, each step a TwoSum with the error added to lo
-          // (lo's FP32 additions round near 2^-48 of the partial), and lane 0 turns the warp's
-          // pair into integers of 2^-S units
-          float hi, lo;
           if constexpr (kPair) {
-            float b, lb;
-            upk(acc2.hi[i], hi, b);
-            upk(acc2.lo[i], lo, lb);
-            two_sum_acc(hi, lo, b);
-            lo = __fadd_rn(lo, lb);
+            float h[2], l0, l1;
+            upk(acc2.hi[i], h[0], h[1]);
+            upk(acc2.lo[i], l0, l1);
+            v[i] = biased_fix<2>(h, __fadd_rn(l0, l1), bias[i / NC], ovf);
           } else {
-            hi = acc.hi[i];
-            lo = acc.lo[i];
-          }
-          long long v = f32_to_fix(hi, ovf) + f32_to_fix(lo, ovf);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-          if (lane == 0) redl[warp * NM + i] = v;
-        }
-        const int any_ovf = __syncthreads_or(ovf);
-        if (threadIdx.x < NM) {
-          long long v = 0;
-          for (int w = 0; w < nw; ++w) v += redl[w * NM + threadIdx.x];
-          unsigned long long* a = p.acc + (size_t)pc.inst * kAccWordsPerInst +
-                                  (((size_t)slot * kAccCopies + blockIdx.x % kAccCopies) * kNMMax + threadIdx.x) * 2;
-          if (!any_ovf && v < kFixLimit && v > -kFixLimit) {
-            atomicAdd(a, (unsigned long long)v);
-          } else if (kRejectOverflow) {
-            atomicMax(&p.errmax[pc.inst], 0x7ff0000000000000ull);   // overflowing trial step
-          } else {
-            atomicExch(&p.nonfinite[pc.inst], 1);
+            const float h[1] = {acc.hi[i]};
+            v[i] = biased_fix<1>(h, acc.lo[i], bias[i / NC], ovf);
           }
         }
+        reduce_moments<NM, long long>(v, ovf, reinterpret_cast<long long*>(red), acc_copy, &p.errmax[pc.inst],
+                                      &p.nonfinite[pc.inst], kRejectOverflow);
       }
     } else {
       if constexpr (kErrMax) {
@@ -2511,28 +2613,11 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
         }
       }
       if constexpr (kMoments) {
-        double v[NM];
+        if constexpr (kErrMax) __syncthreads();              // the scratch is reused
+        double v[NM];                                        // a copy: the accumulators stay in registers
 #pragma unroll
         for (int i = 0; i < NM; ++i) v[i] = acc.v[i];
-        block_sum<NM>(v, red);
-        if (threadIdx.x == 0) {
-          bool fin = true;
-#pragma unroll
-          for (int i = 0; i < NM; ++i) { bs.fx[i] = v[i]; fin = fin && (fabs(v[i]) <= 1.7e308); }
-          bs.flag = fin ? 1 : 0;
-          if (!fin) {
-            if (kRejectOverflow)
-              atomicMax(&p.errmax[pc.inst], 0x7ff0000000000000ull);
-            else
-              atomicExch(&p.nonfinite[pc.inst], 1);
-          }
-        }
-        __syncthreads();
-        if (bs.flag && threadIdx.x < NM) {
-          unsigned long long* a = p.acc + (size_t)pc.inst * kAccWordsPerInst +
-                                  (((size_t)slot * kAccCopies + blockIdx.x % kAccCopies) * kNMMax + threadIdx.x) * 2;
-          fx_add(a, bs.fx[threadIdx.x]);
-        }
+        reduce_moments_shared<NM>(v, red, acc_copy, &p.errmax[pc.inst], &p.nonfinite[pc.inst], kRejectOverflow);
       }
     }
   }
@@ -2622,7 +2707,7 @@ __device__ __forceinline__ void one_pass(const KParams& p, BlockShared<Real, Phy
 // then finish together instead of the older block's warps finishing first), and the launch shape
 // is chosen by measurement (the autotuner in paper_1912_10596_gb300/autotune.py).
 template <class Phys, class Tab, typename Real, bool kCF, int kMinB, int kThreads = 256>
-__global__ void __launch_bounds__(kThreads, kMinB) step_kernel(KParams p) {
+__global__ void __launch_bounds__(kThreads, kMinB) step_kernel(const __grid_constant__ KParams p) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   __shared__ BlockShared<Real, Phys> bs;
   if (threadIdx.x == 0) {

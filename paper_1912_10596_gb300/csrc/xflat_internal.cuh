@@ -45,6 +45,7 @@ struct InstConst {
   double mu_coef;           // mu(r) = mu_coef / r^2, includes the weight scale wscale
   double wscale;            // physical per-bin number luminosity of a unit table weight (1/s)
   double acc_unit;          // mixed kernels: value of one unit of the fixed-point moment sums (2^-S)
+  float wmax, pad_wmax;     // mixed kernels: largest weight |du_j g_k| of a beam, in those units
   double lam_coef, power, lam_const, r_ref;   // lambda(r) = lam_coef (r_ref / r)^power
   const double* mtab;       // matter table: [mt_n][3] (r_i, lambda_i, exponent p_i of the interval
   int32_t mt_n;             // after r_i: lambda = lambda_i (r/r_i)^p_i), device memory, or null
