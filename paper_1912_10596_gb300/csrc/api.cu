@@ -68,7 +68,7 @@ const double kSqrt2GFhc2 = std::sqrt(2.0) * kGF * kHbarcGevKm * kHbarcGevKm;
 
 constexpr uint32_t kMaxJJ = 128;          // combined angle bins per piece (shared-memory table rows)
 constexpr uint32_t kAlignBeams = 4;       // instance offsets and piece starts: 16-byte vectors
-constexpr uint64_t kMinBlockBeams = 128;  // fewest beams a block: two warps of two-beam vectors
+constexpr uint64_t kMinBlockBeams = 128;  // fewest beams a block
 uint32_t max_jj_cap(int nf, size_t real_size, bool ext = false);
 
 struct HostInst {
@@ -94,7 +94,7 @@ struct xflat_s {
   int device = 0, sm_count = 0;
   // device memory
   void* planes = nullptr;                  // [2][nc][stride] Real
-  void* escr = nullptr;                    // DP45: error partial + scale planes [nc + 1][stride] Real
+  void* escr = nullptr;                    // FP64 DP45: error partial planes [nc][stride] Real
   void* kst = nullptr;                     // FP64 RK4 / DP45: stage derivatives + one stage state [n + 1][nc][stride] Real
   uint64_t stride = 0;
   InstConst* d_ic = nullptr;
@@ -512,6 +512,11 @@ void reset_dyn(xflat_t h, uint32_t i, double r0) {
   d.done = 1;
 }
 
+// consecutive beams a thread of the step kernel takes at once
+uint64_t beams_per_thread(xflat_t h) { return h->nf == 2 && h->real_size == 4 ? 2 : 1; }
+static_assert(vec_beams<Phys2<float>, float>() == 2 && vec_beams<Phys2E<float>, float>() == 2 &&
+              vec_beams<Phys3<float>, float>() == 1 && vec_beams<Phys2<double>, double>() == 1);
+
 // Cut all instances into G slices and slices into pieces; blk[b]..blk[b+1] are block b's pieces.
 // Dynamic scheduling: blocks take pieces in list order from a counter.  The list holds first every
 // instance's leading beams in large pieces, then the last kDynTailPct percent of every instance in
@@ -532,7 +537,7 @@ void build_dynamic_pieces(xflat_t h) {
     const HostInst& I = h->inst[i];
     const uint32_t ne = I.cfg.n_energy;
     const uint64_t rows_cap = std::max<uint64_t>(kAlignBeams, ((uint64_t)(max_jj_cap(h->nf, h->real_size, h->extended) - 1) * ne) / kAlignBeams * kAlignBeams);
-    const uint64_t len = std::min<uint64_t>((uint64_t)iters * 2 * h->block, rows_cap);
+    const uint64_t len = std::min<uint64_t>((uint64_t)iters * beams_per_thread(h) * h->block, rows_cap) / kAlignBeams * kAlignBeams;
     for (uint64_t a = a0; a < a1; a += len) {
       Piece p{};
       p.inst = (int)i;
@@ -546,7 +551,7 @@ void build_dynamic_pieces(xflat_t h) {
   };
   uint64_t total = 0;
   for (auto& I : h->inst) total += I.n_beams;
-  const uint32_t iters = (uint32_t)std::min<uint64_t>(total / ((uint64_t)h->grid * 2 * h->block), 1u << 20);
+  const uint32_t iters = (uint32_t)std::min<uint64_t>(total / ((uint64_t)h->grid * beams_per_thread(h) * h->block), 1u << 20);
   const uint32_t big = std::min(64u, std::max(16u, iters / 3)), small = std::min(8u, big / 4);
   std::vector<uint64_t> split(h->inst.size());
   for (uint32_t i = 0; i < h->inst.size(); ++i) {
@@ -836,17 +841,17 @@ int setup_launch_shape(xflat_t h, const xflat_config& c) {
     const uint64_t full = std::min(G_max, ceil_div(T, (uint64_t)h->block * kAlignBeams));
     G = std::max({(uint64_t)1, full, (G_all * T + T_all / 2) / T_all});
   }
-  // Block: no more warps than the block's beams fill (two beams a thread), at least two; idle warps
-  // would still take part in the FP64 reduction trees.  The mixed two-flavour bulb kernels keep
+  // Block: no more warps than the block's beams fill, at least two; idle warps would still take part in
+  // the FP64 reductions.  The mixed two-flavour bulb kernels keep
   // their block (their reductions are integer and FP32).
   if (!c.block_size && !mixed_2f) {
-    const uint64_t threads = ceil_div(ceil_div(T_all, G_all), 2);
+    const uint64_t threads = ceil_div(ceil_div(T_all, G_all), beams_per_thread(h));
     h->block = (int)std::min<uint64_t>((uint64_t)h->block, std::max<uint64_t>(64, ceil_div(threads, 32) * 32));
   }
   h->grid = (int)G;
   // Several instances: blocks take pieces from a counter once each has kDynMinIters vector iterations
   // of work per pass (see build_dynamic_pieces).
-  h->dyn_sched = h->inst.size() > 1 && !h->shard && T >= G * 2 * (uint64_t)h->block * kDynMinIters;
+  h->dyn_sched = h->inst.size() > 1 && !h->shard && T >= G * beams_per_thread(h) * (uint64_t)h->block * kDynMinIters;
   build_pieces(h, h->grid);
   h->smem = smem_bytes(h->nf, h->real_size, h->max_jj, table_stages(h->integrator), h->block, h->extended);
   if (h->d_pieces) cudaFree(h->d_pieces);
@@ -1020,9 +1025,9 @@ int create_impl(const xflat_config* cfgs, uint32_t n, xflat_t* out) {
   h->etab_bytes = (size_t)eoff * h->real_size;
   h->angle_bytes = sizeof(double) * aoff;
   if (dev_alloc(&h->planes, plane_bytes) != cudaSuccess) return bail(XFLAT_ERR_NOMEM);
-  // FP64 DP45: error partial (nc planes) and error scale (one plane) of the step in flight
+  // FP64 DP45: error partial of the step in flight
   if (h->integrator == XFLAT_DP45 && h->real_size == 8) {
-    h->escr_bytes = (size_t)(h->nc + 1) * h->stride * h->real_size;
+    h->escr_bytes = (size_t)h->nc * h->stride * h->real_size;
     if (dev_alloc(&h->escr, h->escr_bytes) != cudaSuccess) return bail(XFLAT_ERR_NOMEM);
   }
   // FP64 RK4 / DP45: the stage derivatives a step stores (k_1..k_3 of RK4, k_1..k_5 of DP45, whose

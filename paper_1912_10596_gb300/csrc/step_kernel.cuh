@@ -233,15 +233,18 @@ __device__ __forceinline__ float sum_bias(float P) {
 }
 
 template <typename Real, int NM> struct MomAcc;
+// FP64: within an angle row all weights share their angle factors, so a thread sums g_k s (row, 3 or 9
+// FMAs a beam) and multiplies the row's sum by du, du t1, ... when it leaves the row (Phys::flush_row).
 template <int NM> struct MomAcc<double, NM> {
-  double v[NM];
-  __device__ __forceinline__ void start(const float*, int) {
+  static constexpr bool kRows = true;
+  double v[NM], r[NM];                                 // r: as many as a state has components are used
+  __device__ __forceinline__ void start(const float*, int nc) {
 #pragma unroll
-    for (int i = 0; i < NM; ++i) v[i] = 0.0;
+    for (int i = 0; i < NM; ++i) { v[i] = 0.0; if (i < nc) r[i] = 0.0; }
   }
-  __device__ __forceinline__ void add(int i, double w, double y) { v[i] = fma(w, y, v[i]); }
 };
 template <int NM> struct MomAcc<float, NM> {
+  static constexpr bool kRows = false;
   float hi[NM], lo[NM];
   // bias: one per group of nc components
   __device__ __forceinline__ void start(const float* bias, int nc) {
@@ -315,7 +318,8 @@ struct Phys2 {
   enum : int { vT1 = 0, vQ = 1, vQBX = 2, vQBZ = 3, vG0X = 4, vG0Y = 5, vG0Z = 6, vT2 = 7 };   // FP64
   enum : int { oNQBX = 0, oNG0X = 1, oQBZ = 2, oG0Z = 3, oG0Y = 4, oT1 = 5, oT2 = 6, oQ = 7 };                 // FP32
   struct Consts { double B[3]; int geom; };
-  struct Beam { Real eo; Real w; };   // eta * omega_k, signed weight du_j * g_{sigma,k}
+  struct Beam { Real eo; Real w; };   // eta * omega_k, signed weight du_j * g_{sigma,k} (FP64: g alone)
+  template <typename R> using With = Phys2<R>;
 
   __device__ static inline Real t1(const Real* t) { return kF32 ? t[oT1] : t[vT1]; }
 
@@ -371,12 +375,27 @@ struct Phys2 {
     k[1] = Kv[2] * y[0] - Kv[0] * y[2];
     k[2] = Kv[0] * y[1] - Kv[1] * y[0];
   }
-  // moments D (weight w t1) and J1 (weight w)
+  // moments D (weight w t1) and J1 (weight w); row sums: w is g_k alone
   template <class Acc>
   __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[3]) {
-    const Real wt = w * t1(row);
+    if constexpr (Acc::kRows) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { acc.add(i, wt, y[i]); acc.add(3 + i, w, y[i]); }
+      for (int i = 0; i < 3; ++i) acc.r[i] = fma(w, y[i], acc.r[i]);
+    } else {
+      const Real wt = w * t1(row);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) { acc.add(i, wt, y[i]); acc.add(3 + i, w, y[i]); }
+    }
+  }
+  template <class Acc>
+  __device__ static inline void flush_row(Acc& acc, Real du, const Real* row) {
+    const Real dt = du * t1(row);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      acc.v[i] = fma(dt, acc.r[i], acc.v[i]);
+      acc.v[3 + i] = fma(du, acc.r[i], acc.v[3 + i]);
+      acc.r[i] = 0;
+    }
   }
   // Frobenius norm^2 of the traceless part of P = (1 + s.sigma)/2: |s|^2 / 2
   __device__ static inline Real tnorm2(const Real (&y)[3]) {
@@ -420,6 +439,7 @@ struct Phys3 {
   enum : int { vT1 = 0, vQ = 1, vG = 2, vT2 = 10 };
   struct Consts { int geom; };
   struct Beam { Real v[kVac]; Real w; };
+  template <typename R> using With = Phys3<R>;
 
   __device__ static inline Real t1(const Real* t) { return t[vT1]; }
   __device__ static inline void fill_geo(Real* t, double u, double x, const Consts& C, int, Real hs) {
@@ -486,9 +506,24 @@ struct Phys3 {
   }
   template <class Acc>
   __device__ static inline void accum_row(Acc& acc, Real w, const Real* row, const Real (&y)[9]) {
-    const Real wt = w * t1(row);
+    if constexpr (Acc::kRows) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) { acc.add(i, wt, y[i]); acc.add(9 + i, w, y[i]); }
+      for (int i = 0; i < 9; ++i) acc.r[i] = fma(w, y[i], acc.r[i]);
+    } else {
+      const Real wt = w * t1(row);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) { acc.add(i, wt, y[i]); acc.add(9 + i, w, y[i]); }
+    }
+  }
+  template <class Acc>
+  __device__ static inline void flush_row(Acc& acc, Real du, const Real* row) {
+    const Real dt = du * t1(row);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      acc.v[i] = fma(dt, acc.r[i], acc.v[i]);
+      acc.v[9 + i] = fma(du, acc.r[i], acc.v[9 + i]);
+      acc.r[i] = 0;
+    }
   }
   // ||P - tr(P)/3||_F^2 with off-diagonal entries counted twice
   __device__ static inline Real tnorm2(const Real (&y)[9]) {
@@ -576,6 +611,7 @@ struct Phys2E {
   enum : int { oNQBX = 0, oNG0X = 1, oQBZ = 2, oG0Z = 3, oG0Y = 4, oT1 = 5, oT2 = 6, oQ = 7, oSCC = 8, oSCS = 9, oH = 10 };   // FP32
   struct Consts { double B[3]; int n_phi; };
   using Beam = typename Phys2<Real>::Beam;
+  template <typename R> using With = Phys2E<R>;
 
   __device__ static inline Real t1(const Real* t) { return kF32 ? t[oT1] : t[vT1]; }
   __device__ static inline void fill_geo(Real* t, double u, double x, const Consts& C, int a, Real hs) {
@@ -644,13 +680,28 @@ struct Phys2E {
   }
   template <class Acc>
   __device__ static inline void accum_row(Acc& acc, Real w, const Real* t, const Real (&y)[3]) {
-    const Real wt = w * t1(t), wc = w * (kF32 ? t[oSCC] : t[vSCC]), ws = w * (kF32 ? t[oSCS] : t[vSCS]);
+    if constexpr (Acc::kRows) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) acc.r[i] = fma(w, y[i], acc.r[i]);
+    } else {
+      const Real wt = w * t1(t), wc = w * t[oSCC], ws = w * t[oSCS];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc.add(i, wt, y[i]);
+        acc.add(3 + i, w, y[i]);
+        acc.add(6 + i, wc, y[i]);
+        acc.add(9 + i, ws, y[i]);
+      }
+    }
+  }
+  template <class Acc>
+  __device__ static inline void flush_row(Acc& acc, Real du, const Real* t) {
+    const Real f[4] = {du * t1(t), du, du * t[vSCC], du * t[vSCS]};
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      acc.add(i, wt, y[i]);
-      acc.add(3 + i, w, y[i]);
-      acc.add(6 + i, wc, y[i]);
-      acc.add(9 + i, ws, y[i]);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) acc.v[3 * g + i] = fma(f[g], acc.r[i], acc.v[3 * g + i]);
+      acc.r[i] = 0;
     }
   }
   __device__ static inline Real tnorm2(const Real (&y)[3]) { return Phys2<Real>::tnorm2(y); }
@@ -673,7 +724,7 @@ struct KParams {
   int* nonfinite;                // [n_inst]
   void* planeA;
   void* planeB;
-  void* escr;                    // adaptive tableaus: error partial and scale planes [NC + 1][plane_stride]
+  void* escr;                    // FP64 DP45: error partial planes [NC][plane_stride]
   void* kst;                     // FP64 RK4 / DP45: stage derivatives k_1..k_n, then one stage state [n + 1][NC][plane_stride]
   uint64_t plane_stride;         // elements between component planes
   const void* etab;              // energy tables, Real, per instance at e_off: [n_tab][n_energy]
@@ -1146,44 +1197,41 @@ __device__ __forceinline__ void cp_async_wait_pending() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Per-thread state vectors: two consecutive beams per load (float2 / double2), so the loaded and
-// the prefetched vectors fit the register budget; a warp still reads 256 or 512 contiguous bytes
-// per plane.
-template <typename Real> struct Vec16;
-template <> struct Vec16<float> { using T = float2; static constexpr int N = 2; };
-template <> struct Vec16<double> { using T = double2; static constexpr int N = 2; };
+// Consecutive beams a thread takes at once: two in the FP32 two-flavour kernels (packed pairs), one in
+// the others (their pass bodies are long, a second copy for the second beam only fills the instruction
+// cache, and FP64 stage planes are then read and written in full 256-byte rows).
+template <class Phys, typename Real>
+__host__ __device__ constexpr int vec_beams() { return Phys::NC == 3 && sizeof(Real) == 4 ? 2 : 1; }
 
-template <typename Real>
-__device__ __forceinline__ void vload(const Real* p, Real (&v)[Vec16<Real>::N]) {
-  const typename Vec16<Real>::T t = __ldcg(reinterpret_cast<const typename Vec16<Real>::T*>(p));
-  const Real* a = reinterpret_cast<const Real*>(&t);
-#pragma unroll
-  for (int i = 0; i < Vec16<Real>::N; ++i) v[i] = a[i];
+template <typename Real, int N>
+__device__ __forceinline__ void vload(const Real* p, Real (&v)[N]) {
+  if constexpr (N == 1) {
+    v[0] = __ldcg(p);
+  } else {
+    const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+    v[0] = t.x;
+    v[1] = t.y;
+  }
 }
-template <typename Real>
-__device__ __forceinline__ void vstore(Real* p, const Real (&v)[Vec16<Real>::N]) {
-  typename Vec16<Real>::T t;
-  Real* a = reinterpret_cast<Real*>(&t);
-#pragma unroll
-  for (int i = 0; i < Vec16<Real>::N; ++i) a[i] = v[i];
-  __stcg(reinterpret_cast<typename Vec16<Real>::T*>(p), t);
+template <typename Real, int N>
+__device__ __forceinline__ void vstore(Real* p, const Real (&v)[N]) {
+  if constexpr (N == 1) __stcg(p, v[0]);
+  else __stcg(reinterpret_cast<float2*>(p), make_float2(v[0], v[1]));
 }
 
 // Plane accesses of the pass body, checked in the checked build (site: where, for the record).
-template <typename Real>
-__device__ __forceinline__ void vload_at(const KParams& p, int span, const Real* ptr,
-                                         Real (&v)[Vec16<Real>::N], int site) {
-  if (XFLAT_SPAN_OK(p, span, ptr, sizeof(typename Vec16<Real>::T), site)) {
+template <typename Real, int N>
+__device__ __forceinline__ void vload_at(const KParams& p, int span, const Real* ptr, Real (&v)[N], int site) {
+  if (XFLAT_SPAN_OK(p, span, ptr, N * sizeof(Real), site)) {
     vload(ptr, v);
   } else {
 #pragma unroll
-    for (int i = 0; i < Vec16<Real>::N; ++i) v[i] = Real(0);
+    for (int i = 0; i < N; ++i) v[i] = Real(0);
   }
 }
-template <typename Real>
-__device__ __forceinline__ void vstore_at(const KParams& p, int span, Real* ptr,
-                                          const Real (&v)[Vec16<Real>::N], int site) {
-  if (XFLAT_SPAN_OK(p, span, ptr, sizeof(typename Vec16<Real>::T), site)) vstore(ptr, v);
+template <typename Real, int N>
+__device__ __forceinline__ void vstore_at(const KParams& p, int span, Real* ptr, const Real (&v)[N], int site) {
+  if (XFLAT_SPAN_OK(p, span, ptr, N * sizeof(Real), site)) vstore(ptr, v);
 }
 
 // Rotation of y about Om by |Om| (right-handed): y + a Om x y + b Om x (Om x y), the Bloch form of
@@ -1427,6 +1475,8 @@ struct BlockShared {
   Real hB[kMaxStages];
   Real hE[kMaxStages];
   Real rtol, atol;
+  float rtol_f, atol_f, inv_tol;       // FP64 error filter: tolerances times inv_tol = 1 / (rtol + atol)
+  int emax_f;                          // bits of the largest squared error ratio found in the piece so far (rounded down)
   int active;
   int parity;
   int flag;
@@ -1446,12 +1496,22 @@ struct TabView {
   }
 };
 
+// The FP32 value of a double's leading 21 bits (truncated), from its high word on the integer pipe;
+// zero below 2^-126, infinite or not a number from 2^128 on.
+__device__ __forceinline__ float lead_f32(double x) {
+  const int h = __double2hiint(x), e = ((h >> 20) & 0x7ff) - 896;
+  const int m = (h & 0xfffff) << 3;
+  const int bits = e <= 0 ? 0 : e >= 255 ? (0x7f800000 | ((h & 0x7ff00000) == 0x7ff00000 ? m : 0)) : (e << 23) | m;
+  return __int_as_float(bits | (h & 0x80000000));
+}
+__device__ __forceinline__ float lead_f32(float x) { return x; }
+
 // What a pass does (compile time).
 enum PassKind : int { kStagePass = 0, kFinalPass = 1, kInitPass = 2 };
 
 // Adaptive FP64 kernels split the last two passes of a step: the pass forming Y_S (= y5, first
-// same as last) also stores y5, the error partial sum over stages 1..S-1 and the error scale, and
-// the final pass only adds k_S -- the stage chain costs FP64 instructions on GB300's narrow FP64
+// same as last) also stores y5 and the error partial sum over stages 1..S-1, and the final pass only
+// adds k_S -- the stage chain costs FP64 instructions on GB300's narrow FP64
 // pipe.  FP32 kernels rebuild the chain in the final pass instead: their state, y5 and those
 // partials together exceed the L2, and the extra DRAM traffic costs more than the FP32 chain.
 template <class Tab, typename Real>
@@ -1500,14 +1560,14 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
   static constexpr bool kStoreY = kStore && kKind == kStagePass && !(kSplit && kPass + 2 == Tab::S);
   static constexpr int kYPlanes = stored_stage_count<Tab, Real>();
   // y: the step's state.  Split final pass: the pass forming Y_S replaces y by the new state
-  // y5 = Y_S and sets ep = (error partial sum over stages 1..S-1, atol + rtol max(|y|, |y5|)); the
-  // final pass gets y5 in y and that ep back.  kst: this beam's element of the stage-derivative
+  // y5 = Y_S and sets ep, the error partial sum over stages 1..S-1; the final pass gets y5 in y, that
+  // ep back, and the step's state in yo.  kst: this beam's element of the stage-derivative
   // planes (component i of k_l at kst[((l - 1) NC + i) kstride]), read and written by this thread
   // only.
   template <class BS, class Acc>
-  __device__ static inline void beam(const BS& bs, const typename Phys::Beam& bm,
+  __device__ static inline void beam(BS& bs, const typename Phys::Beam& bm,
                                      const TabView<Real, Phys>& tv, int tj, Real (&y)[NC],
-                                     Real (&ep)[NC + 1],
+                                     Real (&ep)[NC], const Real (&yo)[NC],
                                      Acc& acc, Real& emax, int& bad, bool mixed,
                                      Real* kst, size_t kstride) {
     Real k[Tab::S + 1][NC];
@@ -1556,8 +1616,7 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       }
       if (kSplit && I == Tab::S) {
         // first same as last: Y_S is the new state y5 (row S of A is b).  Its error partial sum
-        // over stages 1..S-1 and the error scale go with it, so the final pass needs only k_S.
-        if (!(Phys::tnorm2(y) <= rbig<Real>())) bad = 1;   // non-finite input state: fatal
+        // over stages 1..S-1 goes with it, so the final pass needs only k_S.
         if (mixed) Phys::normalise(Y);
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
@@ -1567,7 +1626,6 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
             if (Tab::e(m) != 0.0) v += bs.hE[m] * k[m][i];
           ep[i] = v;
         }
-        ep[NC] = bs.atol + bs.rtol * sqrt(fmax(Phys::tnorm2(y), Phys::tnorm2(Y)));
         Phys::accum_row(acc, bm.w, tv.row(I, tj), Y);
 #pragma unroll
         for (int i = 0; i < NC; ++i) y[i] = Y[i];
@@ -1617,23 +1675,36 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       return;
     }
     if (Tab::kAdaptive) {
-      // split final pass (y holds y5): k_S = f(y5) with the moments of y5, the embedded error,
-      // and the squared error ratio (its square root is taken once per block)
-      const bool ynok = Phys::tnorm2(y) <= rbig<Real>();
+      // split final pass (y holds y5): k_S = f(y5) with the moments of y5, the embedded error, and the
+      // squared error ratio (its square root is taken once per block).  Only the largest ratio counts:
+      // an FP32 estimate of it (components by their leading 21 bits, so within 2e-5) passes over every
+      // beam that cannot exceed the largest found so far in the block, so the FP64 norms, square root
+      // and division -- a fifth of a DP45 step's FP64 work -- are left for a few beams a block.
       Real Kv[Phys::NG], kS[NC], e[NC];
       Phys::K(tv.row(Tab::S, tj), bm, Kv);
       Phys::f(Kv, y, kS);
 #pragma unroll
+      for (int i = 0; i < NC; ++i) e[i] = ep[i] + bs.hE[Tab::S] * kS[i];
+      float ef[NC], yf[NC], of[NC];
+#pragma unroll
       for (int i = 0; i < NC; ++i) {
-        Real v = ep[i];
-        v += bs.hE[Tab::S] * kS[i];
-        e[i] = v;
+        ef[i] = lead_f32(e[i]) * bs.inv_tol;
+        yf[i] = lead_f32(y[i]);
+        of[i] = lead_f32(yo[i]);
       }
-      const Real den = ep[NC];
-      Real r2 = Phys::tnorm2(e) / (den * den);
-      // a trial step whose stages overflowed the working precision is rejected, not fatal
-      if (!(r2 <= rbig<Real>()) || !ynok) r2 = Real(INFINITY);
-      emax = fmax(emax, r2);
+      using P32 = typename Phys::template With<float>;
+      const float df = bs.atol_f + bs.rtol_f * sqrtf(fmaxf(P32::tnorm2(of), P32::tnorm2(yf)));
+      const float rf = __fdividef(P32::tnorm2(ef), df * df);
+      if (!(rf * 1.001f < __int_as_float(*(volatile int*)&bs.emax_f))) {       // also where rf is not a number
+        const Real no = Phys::tnorm2(yo), n5 = Phys::tnorm2(y);
+        if (!(no <= rbig<Real>())) bad = 1;                     // non-finite input state: fatal
+        const Real den = bs.atol + bs.rtol * sqrt(fmax(no, n5));
+        Real r2 = Phys::tnorm2(e) / (den * den);
+        // a trial step whose stages overflowed the working precision is rejected, not fatal
+        if (!(r2 <= rbig<Real>()) || !(n5 <= rbig<Real>())) r2 = Real(INFINITY);
+        emax = fmax(emax, r2);
+        atomicMax(&bs.emax_f, __float_as_int(__double2float_rd((double)fmin(r2, Real(3.0e38)))));
+      }
       return;
     }
     // final pass of a fixed-step tableau
@@ -1802,7 +1873,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
   template <class BS, class Acc>
   __device__ static inline void beam(const BS& bs, const typename Phys::Beam& bm,
                                      const TabView<Real, Phys>& tv, int tj, Real (&y)[NC],
-                                     Real (&)[NC + 1],
+                                     Real (&)[NC], const Real (&)[NC],
                                      Acc& acc, Real& emax, int& bad, bool mixed,
                                      Real*, size_t) {
     if (kKind == kInitPass) {
@@ -1946,6 +2017,7 @@ struct PairAcc {
 // accumulators, so those kernels keep one set of accumulator registers.
 template <int NM>
 struct PairHalfAcc {
+  static constexpr bool kRows = false;
   PairAcc<NM>& a;
   __device__ __forceinline__ void add(int i, float w, float y) { biased_add2(a.hi[i], a.lo[i], pk(w, 0.0f), pk(y, 0.0f)); }
 };
@@ -2134,7 +2206,7 @@ __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int
   } else {
     const Real om = et[k];
     bm.eo = sigma ? -om : om;
-    bm.w = du * et[(1 + sigma) * ne + k];
+    bm.w = et[(1 + sigma) * ne + k];                // row sums carry du
   }
 }
 template <typename Real>
@@ -2146,7 +2218,8 @@ __device__ __forceinline__ void load_beam(const Real* et, int ne, int sigma, int
     const Real v = et[i * ne + k];
     bm.v[i] = sigma ? -v : v;
   }
-  bm.w = du * et[(kVac + sigma) * ne + k];
+  const Real g = et[(kVac + sigma) * ne + k];
+  bm.w = sizeof(Real) == 4 ? du * g : g;             // FP64 row sums carry du
 }
 
 // Checked build: a beam's energy-table entries (all rows of its bin), its row of the shared angle tables and (stored-stage bodies) its
@@ -2230,6 +2303,7 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
     return v;
   };
   __syncthreads();
+  if (threadIdx.x == 0) bs.emax_f = 0;
   if (incremental) {
     if (threadIdx.x < Phys::NSC) bs.scr[newest][threadIdx.x] = (Real)newest_constant(threadIdx.x);
     __syncthreads();
@@ -2285,6 +2359,10 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
     if (threadIdx.x == 0) {
       bs.rtol = (Real)ic.rtol;
       bs.atol = (Real)ic.atol;
+      const double inv = fmin(1.0 / (ic.rtol + ic.atol), 1.0e30);      // keeps FP32 squares in range
+      bs.inv_tol = (float)inv;
+      bs.rtol_f = (float)(ic.rtol * inv);
+      bs.atol_f = (float)(ic.atol * inv);
     }
     for (int t = threadIdx.x; t < n_jj; t += blockDim.x) {
       const int jj = pc.jj_lo + t;
@@ -2328,7 +2406,7 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
 // One pass over all pieces of this block.
 template <class Phys, class Tab, typename Real, bool kCF, int kPass, int kKind>
 __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned char* dyn_smem) {
-  constexpr int NC = Phys::NC, NM = Phys::NM, VN = Vec16<Real>::N;
+  constexpr int NC = Phys::NC, NM = Phys::NM, VN = vec_beams<Phys, Real>();
   using Body = PassBody<Phys, Tab, Real, kCF, kPass, kKind>;
   double* red = reinterpret_cast<double*>(dyn_smem);                 // 32 * kNMMax doubles
   constexpr int kTS = Tab::S + 1;                                    // table stage slots 0..S
@@ -2390,7 +2468,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     const Real* yin = reinterpret_cast<const Real*>(bs.parity ? p.planeB : p.planeA) + ic.beam_off;
     Real* yout = reinterpret_cast<Real*>(bs.parity ? p.planeA : p.planeB) + ic.beam_off;
     // split final pass (see split_final): the pass forming Y_S stores y5 (into the output planes),
-    // the error partial and the error scale; the final pass reads those instead of the chain
+    // and the error partial; the final pass reads those instead of the chain
     constexpr bool kSplitStore = split_final<Tab, Real>() && kKind == kStagePass && kPass + 2 == Tab::S;
     constexpr bool kSplitLoad = split_final<Tab, Real>() && kKind == kFinalPass;
     Real* escr = reinterpret_cast<Real*>(p.escr) + ic.beam_off;
@@ -2401,8 +2479,8 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     // geometry factor), |Y| <= 2, to an accumulator
     auto biases = [&](float (&bias)[NM / NC]) {
       if constexpr (sizeof(Real) == 4) {
-        constexpr int kMomRow = kKind == kInitPass ? 1 : (kKind == kStagePass ? kPass + 2 : Tab::S);
-        const float t1m = __int_as_float(bs.t1max[kMomRow]);
+        constexpr int kRow = kKind == kInitPass ? 1 : (kKind == kStagePass ? kPass + 2 : Tab::S);
+        const float t1m = __int_as_float(bs.t1max[kRow]);
         const float P = 4.0f * (float)(pc.len / (VN * blockDim.x) + 2u) * ic.wmax;
         bias[0] = sum_bias(P * t1m);
         bias[1] = sum_bias(P);
@@ -2424,8 +2502,16 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       acc2.lo[i] = 0ull;
     }
     float emax2 = 0.0f;
-    const uint32_t end = pc.start + pc.len;
-    const uint32_t vstep = VN * blockDim.x;
+    // Which beams a thread takes: FP32 passes stride the block over the piece; FP64 passes give each
+    // warp a contiguous run of it, so that a thread stays in one angle row for many beams (row sums).
+    constexpr bool kRows = MomAcc<Real, NM>::kRows;
+    constexpr bool kMoments = kKind != kFinalPass || Tab::kFinalMoments;
+    constexpr int kMomRow = kKind == kInitPass ? 1 : (kKind == kStagePass ? kPass + 2 : Tab::S);
+    const uint32_t run = kRows ? (pc.len + VN * blockDim.x - 1) / (VN * blockDim.x) * (32u * VN) : 0u;
+    const uint32_t first = pc.start + (kRows ? (threadIdx.x >> 5) * run + VN * (threadIdx.x & 31) : VN * threadIdx.x);
+    const uint32_t end = kRows ? min(pc.start + pc.len, pc.start + ((threadIdx.x >> 5) + 1) * run) : pc.start + pc.len;
+    const uint32_t vstep = kRows ? 32u * VN : VN * blockDim.x;
+    int row_cur = -1;                                  // row sums: the row being summed
     // FP32 two-flavour bulb passes: the state comes through the thread's ring, kStateRingDepth vectors
     // ahead (see state_ring).  Other two-flavour passes: the next vector's state is loaded into
     // registers while this one is processed.  Either way the L2/HBM latency of the stream overlaps
@@ -2433,9 +2519,9 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     constexpr bool kRingLoad = state_ring<Phys, Real>();
     constexpr bool kPrefetch = NC == 3 && !kRingLoad;
     Real nxt[NC][VN];
-    if (kPrefetch && pc.start + VN * threadIdx.x < end) {
+    if (kPrefetch && first < end) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) vload_at(p, kSpanPlanes, ysrc + (size_t)c * p.plane_stride + pc.start + VN * threadIdx.x, nxt[c], 1);
+      for (int c = 0; c < NC; ++c) vload_at(p, kSpanPlanes, ysrc + (size_t)c * p.plane_stride + first, nxt[c], 1);
     }
     constexpr int ring_d = kStateRingDepth;
     constexpr uint32_t ring_slots = (uint32_t)ring_d + 1u;
@@ -2455,9 +2541,9 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       q_fill = q_fill + 1u == ring_slots ? 0u : q_fill + 1u;
     };
     if constexpr (kRingLoad) {
-      for (int j = 0; j < ring_d; ++j) ring_fill(pc.start + VN * threadIdx.x + (uint32_t)j * vstep);
+      for (int j = 0; j < ring_d; ++j) ring_fill(first + (uint32_t)j * vstep);
     }
-    for (uint32_t l0 = pc.start + VN * threadIdx.x; l0 < end; l0 += vstep) {
+    for (uint32_t l0 = first; l0 < end; l0 += vstep) {
       Real ys[NC][VN];
       if constexpr (kRingLoad) {
         // the slot filled now is the one read in the previous iteration (kStateRingDepth + 1 slots)
@@ -2483,10 +2569,13 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
 #pragma unroll
         for (int c = 0; c < NC; ++c) vload_at(p, kSpanPlanes, ysrc + (size_t)c * p.plane_stride + l0, ys[c], 3);
       }
-      Real ep[NC + 1][VN];
+      Real ep[NC][VN], yo[NC][VN];
       if constexpr (kSplitLoad) {
 #pragma unroll
-        for (int c = 0; c <= NC; ++c) vload_at(p, kSpanEscr, escr + (size_t)c * p.plane_stride + l0, ep[c], 4);
+        for (int c = 0; c < NC; ++c) {
+          vload_at(p, kSpanEscr, escr + (size_t)c * p.plane_stride + l0, ep[c], 4);
+          vload_at(p, kSpanPlanes, yin + (size_t)c * p.plane_stride + l0, yo[c], 17);
+        }
       }
       int jj = (int)fast_div(l0, ic.div_magic);
       int k = (int)l0 - jj * ne;
@@ -2521,25 +2610,31 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
             const int tj = jj - (int)pc.jj_lo;
             typename Phys::Beam bm;
             load_beam<Real>(et, ne, sigma, k, dut[tj], bm);
-            Real y[NC], ev[NC + 1];
+            if constexpr (kRows && kMoments) {
+              if (tj != row_cur) {
+                if (row_cur >= 0) Phys::flush_row(acc, dut[row_cur], tv.row(kMomRow, row_cur));
+                row_cur = tj;
+              }
+            }
+            Real y[NC], ev[NC], ov[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) y[c] = ys[c][v];
             if constexpr (kSplitLoad) {
 #pragma unroll
-              for (int c = 0; c <= NC; ++c) ev[c] = ep[c][v];
+              for (int c = 0; c < NC; ++c) { ev[c] = ep[c][v]; ov[c] = yo[c][v]; }
             }
             if constexpr (kPair) {
               PairHalfAcc<NM> hacc{acc2};
-              Body::beam(bs, bm, tv, tj, y, ev, hacc, emax, bad, mixed, nullptr, p.plane_stride);
+              Body::beam(bs, bm, tv, tj, y, ev, ov, hacc, emax, bad, mixed, nullptr, p.plane_stride);
             } else {
-              Body::beam(bs, bm, tv, tj, y, ev, acc, emax, bad, mixed, Body::kStore ? kst + l0 + v : nullptr,
+              Body::beam(bs, bm, tv, tj, y, ev, ov, acc, emax, bad, mixed, Body::kStore ? kst + l0 + v : nullptr,
                          p.plane_stride);
             }
 #pragma unroll
             for (int c = 0; c < NC; ++c) ys[c][v] = y[c];
             if constexpr (kSplitStore) {
 #pragma unroll
-              for (int c = 0; c <= NC; ++c) ep[c][v] = ev[c];
+              for (int c = 0; c < NC; ++c) ep[c][v] = ev[c];
             }
           }
           if (++k == ne) { k = 0; ++jj; }
@@ -2553,21 +2648,18 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
 #pragma unroll
         for (int c = 0; c < NC; ++c) vstore_at(p, kSpanPlanes, yout + (size_t)c * p.plane_stride + l0, ys[c], 6);
 #pragma unroll
-        for (int c = 0; c <= NC; ++c) vstore_at(p, kSpanEscr, escr + (size_t)c * p.plane_stride + l0, ep[c], 7);
+        for (int c = 0; c < NC; ++c) vstore_at(p, kSpanEscr, escr + (size_t)c * p.plane_stride + l0, ep[c], 7);
       }
     }
     if constexpr (kRingLoad) cp_async_wait_pending<0>();  // nothing in flight into the ring after the piece
     if constexpr (kPair) emax = fmax(emax, (Real)emax2);
-    // the pass forming Y_S also checked the step's input state (non-finite: fatal)
-    if constexpr (kSplitStore) {
-      const int any_bad = __syncthreads_or(bad);
-      if (any_bad && threadIdx.x == 0) atomicExch(&p.nonfinite[pc.inst], 1);
+    if constexpr (kRows && kMoments) {
+      if (row_cur >= 0) Phys::flush_row(acc, dut[row_cur], tv.row(kMomRow, row_cur));
     }
     // reduce this piece into the instance accumulators: the error maximum (final pass of an
     // adaptive tableau) and the moments (every pass but a final one without moments); a
     // non-finite moment rejects an adaptive trial step and is fatal for a fixed step
     constexpr bool kErrMax = kKind == kFinalPass && Tab::kAdaptive;
-    constexpr bool kMoments = kKind != kFinalPass || Tab::kFinalMoments;
     constexpr bool kRejectOverflow = Tab::kAdaptive;
     unsigned long long* acc_copy = p.acc + (size_t)pc.inst * kAccWordsPerInst +
                                    ((size_t)slot * kAccCopies + blockIdx.x % kAccCopies) * kNMMax * 2;
@@ -2603,13 +2695,18 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
       }
     } else {
       if constexpr (kErrMax) {
-        const double em = (emax <= rbig<Real>()) ? (double)emax : __longlong_as_double(0x7ff0000000000000ll);
+        // the maximum over the bits of non-negative doubles (integer pipe)
+        long long em = __double_as_longlong((emax <= rbig<Real>()) ? (double)emax : (double)INFINITY);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+        long long* redl = reinterpret_cast<long long*>(red);
+        if ((threadIdx.x & 31) == 0) redl[threadIdx.x >> 5] = em;
         const int any_bad = __syncthreads_or(bad);
-        const double bmax = block_max(em, red);
         if (threadIdx.x == 0) {
+          for (int w = 1; w < (int)(blockDim.x >> 5); ++w) em = max(em, redl[w]);
           if (any_bad) atomicExch(&p.nonfinite[pc.inst], 1);
           // the beams gave squared error ratios
-          atomicMax(&p.errmax[pc.inst], (unsigned long long)__double_as_longlong(sqrt(bmax)));
+          atomicMax(&p.errmax[pc.inst], (unsigned long long)__double_as_longlong(sqrt(__longlong_as_double(em))));
         }
       }
       if constexpr (kMoments) {
