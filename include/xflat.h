@@ -69,7 +69,7 @@ enum xflat_integrator {
   XFLAT_DP45 = 1,             /* Dormand-Prince 5(4), FSAL, adaptive (error control below)        */
   XFLAT_LIE_RK4 = 2,          /* commutator-free Lie RK4 whose every update is an exact propagator
                                  exp(-i H dl) of Eq. U (two flavours: the closed form; three: by
-                                 the eigen-decomposition of the 3 x 3 generator), fixed step      */
+                                 the closed form of its 3 x 3 counterpart), fixed step            */
   XFLAT_EXP_MIDPOINT = 3,     /* exponential midpoint rule (Lie-group Runge-Kutta-Munthe-Kaas method
                                  with Runge's midpoint tableau; Sec. 3.4's exact propagator of Eq. U
                                  with a mid-point scheme): y' = exp(-i H(r+h/2, y_half) dl) applied

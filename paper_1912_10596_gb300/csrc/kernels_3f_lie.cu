@@ -1,6 +1,6 @@
 // Three-flavour step kernels of the exponential integrators (commutator-free Lie RK4, the
 // exponential midpoint rule and the adaptive Lie RK4 with Richardson control): FP64 and mixed, one
-// 256-thread block per SM.  The propagators are the eigen-decomposition form of Eq. U for 3 x 3
+// 256-thread block per SM.  The propagators are the closed form of Eq. U for 3 x 3
 // generators (propagate3).  A translation unit of its own, so that it compiles in parallel with
 // the others.
 #include "step_kernel.cuh"

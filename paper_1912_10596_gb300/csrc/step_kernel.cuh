@@ -1234,20 +1234,39 @@ __device__ __forceinline__ void vstore_at(const KParams& p, int span, Real* ptr,
   if (XFLAT_SPAN_OK(p, span, ptr, N * sizeof(Real), site)) vstore(ptr, v);
 }
 
+// sqrt(x) and 1/sqrt(x) to rounding for x in the normal FP32 range: Newton steps from the hardware's
+// FP32 reciprocal square root, no division (the library's FP64 square root and division are chains of
+// 673 and 429 cycles on GB300)
+__device__ __forceinline__ void sqrt_pair(float x, float& t, float& r) {
+  r = rsqrtf(x);
+  r = fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+  t = x * r;
+  t = fmaf(0.5f * r, fmaf(-t, t, x), t);
+}
+__device__ __forceinline__ void sqrt_pair(double x, double& t, double& r) {
+  r = (double)rsqrtf((float)x);
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  t = x * r;
+  t = fma(0.5 * r, fma(-t, t, x), t);
+}
+
 // Rotation of y about Om by |Om| (right-handed): y + a Om x y + b Om x (Om x y), the Bloch form of
-// y -> U y U^dagger with U = exp(-i Om.sigma/2), i.e. the propagator of Eq. U.
+// y -> U y U^dagger with U = exp(-i Om.sigma/2), i.e. the propagator of Eq. U; a = sin t / t and
+// b = (1 - cos t) / t^2 = (sin(t/2) / t)^2 2 from the half angle, without cancellation.
 template <typename Real>
 __device__ __forceinline__ void rotate(const Real (&Om)[3], Real (&y)[3]) {
   const Real t2 = Om[0] * Om[0] + Om[1] * Om[1] + Om[2] * Om[2];
   Real a, b;
   const Real eps = sizeof(Real) == 4 ? Real(1e-3) : Real(1e-5);
   if (t2 > eps * eps) {
-    const Real t = sqrt(t2);
-    Real sh, ch;
-    if (sizeof(Real) == 4) sincosf((float)(Real(0.5) * t), (float*)&sh, (float*)&ch);
-    else sincos((double)(Real(0.5) * t), (double*)&sh, (double*)&ch);
-    a = Real(2) * sh * ch / t;
-    b = Real(2) * sh * sh / t2;
+    Real t, r, sh, ch;
+    sqrt_pair(t2, t, r);
+    if constexpr (sizeof(Real) == 4) sincosf(0.5f * t, &sh, &ch);
+    else sincos(0.5 * t, &sh, &ch);
+    const Real sr = sh * r;
+    a = Real(2) * sr * ch;
+    b = Real(2) * sr * sr;
   } else {
     a = Real(1) - t2 * Real(1.0 / 6.0);
     b = Real(0.5) - t2 * Real(1.0 / 24.0);
@@ -1459,7 +1478,7 @@ __device__ __noinline__ void propagate3(const Real (&Om)[8], Real (&y)[9]) {
 
 // The propagator of Eq. U over one step for the generator Om (step length and coefficients folded
 // in): y <- exp(-i Om) y exp(i Om).  Two flavours: the rotation of the Bloch vector; three
-// flavours: by the eigen-decomposition of Om.
+// flavours: the closed form of propagate3.
 template <typename Real>
 __device__ __forceinline__ void propagate(const Real (&Om)[3], Real (&y)[3]) { rotate(Om, y); }
 template <typename Real>
@@ -1542,6 +1561,7 @@ struct PassBody;
 template <class Phys, class Tab, typename Real, int kPass, int kKind>
 struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
   static constexpr int NC = Phys::NC;
+  static constexpr bool kWriteOut = false, kReadOut = false, kReadBoth = false;
   static constexpr bool kSplit = split_final<Tab, Real>();
   // number of stage derivatives the pass needs before its stage state, rebuilt or (stored stages)
   // read back (split final pass: none, the pass forming Y_S left y5 and the error partial behind;
@@ -1731,6 +1751,17 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
   static constexpr int NC = Phys::NC;          // 3: Bloch vectors; 9: Hermitian 3 x 3 matrices
   static constexpr int NG = Phys::NG;          // reals of a generator: 3, or 8 (a 3 x 3 without its trace)
   static constexpr bool kStore = false;
+  // Stage states that later passes start from are kept in the output planes, which nobody reads before
+  // the final pass: the commutator-free scheme's Y2, from which Y4 follows by one more propagator, and
+  // (Richardson) the first half step's Y5 likewise for Y7, then its result y_a, from which slots 9 to 11
+  // and the second half step start.  An attempt takes 16 propagators a beam instead of the 26 that start
+  // from y every time (a rejected attempt leaves the output planes as scratch), for three more writes of
+  // a state that stays in the L2 (GB300: 4M beams mixed, 4 attempts, 3.18 -> 2.23 ms with rotate's
+  // division-free form; three flavours, 262,144 beams, 5 attempts, 1.92 -> 1.60 ms).
+  static constexpr int kSlot = kKind == kStagePass && !Tab::kEM2 ? kPass + 2 : 0;
+  static constexpr bool kWriteOut = kSlot == 2 || (Tab::kRichardson && (kSlot == 5 || kSlot == 8));
+  static constexpr bool kReadOut = kSlot == 4 || (Tab::kRichardson && (kSlot == 7 || kSlot >= 9));
+  static constexpr bool kReadBoth = kKind == kFinalPass && Tab::kRichardson;
   // rotation of y by d K (the propagator of Eq. U over the path length d for generator K)
   __device__ static inline void rot(Real (&y)[NC], const Real (&K)[NG], Real d) {
     Real Om[NG];
@@ -1738,10 +1769,9 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
     for (int i = 0; i < NG; ++i) Om[i] = d * K[i];
     propagate(Om, y);
   }
-  // the fourth stage state of a CF4 step of size hh from y with generators Ka (its first stage)
-  // and Kc (its third): exp(hh (Kc - Ka/2)) exp(hh/2 Ka) y
+  // the fourth stage state of a CF4 step of size hh from its second, y = exp(hh/2 Ka) y0, with generators
+  // Ka (its first stage) and Kc (its third): exp(hh (Kc - Ka/2)) y
   __device__ static inline void cf4_stage4(Real (&y)[NC], const Real (&Ka)[NG], const Real (&Kc)[NG], Real hh) {
-    rot(y, Ka, Real(0.5) * hh);
     Real D[NG];
 #pragma unroll
     for (int i = 0; i < NG; ++i) D[i] = Kc[i] - Real(0.5) * Ka[i];
@@ -1765,93 +1795,70 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
                                     int tj, int s, Real (&K)[NG]) {
     Phys::K(tv.row(s, tj), bm, K);
   }
-  // Richardson-controlled CF4 (TabCFR): pass p forms the stage state of slot p + 2 from y; the
-  // final pass forms both results, the error ratio and the moments of the kept result.
+  // Richardson-controlled CF4 (TabCFR): pass p forms the stage state of slot p + 2, from y or from the
+  // state kept in the output planes (kReadOut); the final pass (y the step's state, ya the first half
+  // step's result) forms both results, the error ratio and the moments of the kept result.
   template <class BS, class Acc>
   __device__ static inline void richardson(const BS& bs, const typename Phys::Beam& bm,
-                                           const TabView<Real, Phys>& tv, int tj, Real (&y)[NC], Acc& acc,
-                                           Real& emax, int& bad, bool mixed) {
+                                           const TabView<Real, Phys>& tv, int tj, Real (&y)[NC], const Real (&ya)[NC],
+                                           Acc& acc, Real& emax, int& bad, bool mixed) {
     const Real h = bs.hB[0], hh = Real(0.5) * h;
     constexpr int I = kKind == kFinalPass ? 0 : kPass + 2;   // slot formed by this pass
-    Real K1[NG];
-    gen(bs, bm, tv, tj, 1, K1);
-    if constexpr (I >= 2 && I <= 4) {
-      // full step: Y2 = exp(h/2 K1) y, Y3 = exp(h/2 K2) y, Y4 = exp(h (K3 - K1/2)) exp(h/2 K1) y
-      if constexpr (I == 2) {
-        rot(y, K1, hh);
-      } else if constexpr (I == 3) {
-        Real K2[NG];
-        gen(bs, bm, tv, tj, 2, K2);
-        rot(y, K2, hh);
-      } else {
-        Real K3[NG];
-        gen(bs, bm, tv, tj, 3, K3);
-        cf4_stage4(y, K1, K3, h);
-      }
-      Phys::accum_row(acc, bm.w, tv.row(I, tj), y);
-      return;
-    }
-    if constexpr (I >= 5 && I <= 7) {
-      // first half step: slots 5, 6, 7 as 2, 3, 4 with hh and generators K1, K5, K6
-      if constexpr (I == 5) {
-        rot(y, K1, Real(0.5) * hh);
-      } else if constexpr (I == 6) {
-        Real K5[NG];
-        gen(bs, bm, tv, tj, 5, K5);
-        rot(y, K5, Real(0.5) * hh);
-      } else {
-        Real K6[NG];
-        gen(bs, bm, tv, tj, 6, K6);
-        cf4_stage4(y, K1, K6, hh);
-      }
-      Phys::accum_row(acc, bm.w, tv.row(I, tj), y);
-      return;
-    }
-    // everything later starts from the first half step's result y_a (slot 8)
-    Real y0[NC];
-#pragma unroll
-    for (int i = 0; i < NC; ++i) y0[i] = y[i];
-    {
-      Real K5[NG], K6[NG], K7[NG];
+    if constexpr (I == 2 || I == 3) {
+      // full step: Y2 = exp(h/2 K1) y, Y3 = exp(h/2 K2) y
+      Real K[NG];
+      gen(bs, bm, tv, tj, I - 1, K);
+      rot(y, K, hh);
+    } else if constexpr (I == 5 || I == 6) {
+      // first half step: slots 5, 6 as 2, 3 with hh and generators K1, K5
+      Real K[NG];
+      gen(bs, bm, tv, tj, I == 5 ? 1 : 5, K);
+      rot(y, K, Real(0.5) * hh);
+    } else if constexpr (I == 4 || I == 7) {
+      // y holds Y2 (Y5): Y4 = exp(h (K3 - K1/2)) Y2, Y7 = exp(hh (K6 - K1/2)) Y5
+      Real K1[NG], K[NG];
+      gen(bs, bm, tv, tj, 1, K1);
+      gen(bs, bm, tv, tj, I - 1, K);
+      cf4_stage4(y, K1, K, I == 4 ? h : hh);
+    } else if constexpr (I == 8) {
+      // the first half step's result y_a
+      Real K1[NG], K5[NG], K6[NG], K7[NG];
+      gen(bs, bm, tv, tj, 1, K1);
       gen(bs, bm, tv, tj, 5, K5);
       gen(bs, bm, tv, tj, 6, K6);
       gen(bs, bm, tv, tj, 7, K7);
       cf4_final(y, K1, K5, K6, K7, hh);
+    } else if constexpr (I == 9 || I == 10) {
+      // second half step from y_a
+      Real K[NG];
+      gen(bs, bm, tv, tj, I - 1, K);
+      rot(y, K, Real(0.5) * hh);
+    } else if constexpr (I == 11) {
+      Real K8[NG], K10[NG];
+      gen(bs, bm, tv, tj, 8, K8);
+      gen(bs, bm, tv, tj, 10, K10);
+      rot(y, K8, Real(0.5) * hh);
+      cf4_stage4(y, K8, K10, hh);
     }
-    if constexpr (I == 8) {
-      Phys::accum_row(acc, bm.w, tv.row(8, tj), y);
-      return;
-    }
-    Real K8[NG];
-    gen(bs, bm, tv, tj, 8, K8);
-    if constexpr (I >= 9 && I <= 11) {
-      if constexpr (I == 9) {
-        rot(y, K8, Real(0.5) * hh);
-      } else if constexpr (I == 10) {
-        Real K9[NG];
-        gen(bs, bm, tv, tj, 9, K9);
-        rot(y, K9, Real(0.5) * hh);
-      } else {
-        Real K10[NG];
-        gen(bs, bm, tv, tj, 10, K10);
-        cf4_stage4(y, K8, K10, hh);
-      }
+    if constexpr (I >= 2) {
       Phys::accum_row(acc, bm.w, tv.row(I, tj), y);
       return;
     } else {
-      // final pass: y_b = the second half step from y_a, y_full = the full step from y0
+      // final pass: y_b = the second half step from y_a, y_full = the full step from y
+      Real yb[NC], yf[NC];
+#pragma unroll
+      for (int i = 0; i < NC; ++i) { yb[i] = ya[i]; yf[i] = y[i]; }
       {
-        Real K9[NG], K10[NG], K11[NG];
+        Real K8[NG], K9[NG], K10[NG], K11[NG];
+        gen(bs, bm, tv, tj, 8, K8);
         gen(bs, bm, tv, tj, 9, K9);
         gen(bs, bm, tv, tj, 10, K10);
         gen(bs, bm, tv, tj, 11, K11);
-        cf4_final(y, K8, K9, K10, K11, hh);
+        cf4_final(yb, K8, K9, K10, K11, hh);
       }
-      Real yf[NC];
-#pragma unroll
-      for (int i = 0; i < NC; ++i) yf[i] = y0[i];
       {
-        Real K2[NG], K3[NG], K4[NG];
+        Real K1[NG], K2[NG], K3[NG], K4[NG];
+        gen(bs, bm, tv, tj, 1, K1);
         gen(bs, bm, tv, tj, 2, K2);
         gen(bs, bm, tv, tj, 3, K3);
         gen(bs, bm, tv, tj, 4, K4);
@@ -1859,21 +1866,23 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
       }
       Real e[NC];
 #pragma unroll
-      for (int i = 0; i < NC; ++i) e[i] = (y[i] - yf[i]) * Real(1.0 / 15.0);
-      if (!(Phys::tnorm2(y0) <= rbig<Real>())) bad = 1;       // non-finite input state: fatal
-      const bool ynok = Phys::tnorm2(y) <= rbig<Real>();
-      const Real den = bs.atol + bs.rtol * sqrt(fmax(Phys::tnorm2(y0), Phys::tnorm2(y)));
+      for (int i = 0; i < NC; ++i) e[i] = (yb[i] - yf[i]) * Real(1.0 / 15.0);
+      if (!(Phys::tnorm2(y) <= rbig<Real>())) bad = 1;        // non-finite input state: fatal
+      const bool ynok = Phys::tnorm2(yb) <= rbig<Real>();
+      const Real den = bs.atol + bs.rtol * sqrt(fmax(Phys::tnorm2(y), Phys::tnorm2(yb)));
       Real r2 = Phys::tnorm2(e) / (den * den);
       if (!(r2 <= rbig<Real>()) || !ynok) r2 = Real(INFINITY);
       emax = fmax(emax, r2);
-      if (mixed && ynok) Phys::purify(y);
-      Phys::accum_row(acc, bm.w, tv.row(11, tj), y);
+      if (mixed && ynok) Phys::purify(yb);
+      Phys::accum_row(acc, bm.w, tv.row(11, tj), yb);
+#pragma unroll
+      for (int i = 0; i < NC; ++i) y[i] = yb[i];
     }
   }
   template <class BS, class Acc>
   __device__ static inline void beam(const BS& bs, const typename Phys::Beam& bm,
                                      const TabView<Real, Phys>& tv, int tj, Real (&y)[NC],
-                                     Real (&)[NC], const Real (&)[NC],
+                                     Real (&)[NC], const Real (&yo)[NC],
                                      Acc& acc, Real& emax, int& bad, bool mixed,
                                      Real*, size_t) {
     if (kKind == kInitPass) {
@@ -1882,7 +1891,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
     }
     const Real h = bs.hB[0];
     if constexpr (Tab::kRichardson) {
-      richardson(bs, bm, tv, tj, y, acc, emax, bad, mixed);
+      richardson(bs, bm, tv, tj, y, yo, acc, emax, bad, mixed);
       return;
     }
     if constexpr (Tab::kEM2) {
@@ -1940,12 +1949,7 @@ struct PassBody<Phys, Tab, Real, true, kPass, kKind> {
     }
     Phys::K(tv.row(3, tj), bm, K3);
     if (kKind == kStagePass && kPass == 2) {
-#pragma unroll
-      for (int i = 0; i < NG; ++i) Om[i] = Real(0.5) * h * K1[i];
-      propagate(Om, y);
-#pragma unroll
-      for (int i = 0; i < NG; ++i) Om[i] = h * K3[i] - Real(0.5) * h * K1[i];
-      propagate(Om, y);
+      cf4_stage4(y, K1, K3, h);                                // y holds Y2
       Phys::accum_row(acc, bm.w, tv.row(4, tj), y);
       return;
     }
@@ -2303,7 +2307,9 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
     return v;
   };
   __syncthreads();
-  if (threadIdx.x == 0) bs.emax_f = 0;
+  if constexpr (sizeof(Real) == 8) {
+    if (threadIdx.x == 0) bs.emax_f = 0;
+  }
   if (incremental) {
     if (threadIdx.x < Phys::NSC) bs.scr[newest][threadIdx.x] = (Real)newest_constant(threadIdx.x);
     __syncthreads();
@@ -2359,10 +2365,12 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
     if (threadIdx.x == 0) {
       bs.rtol = (Real)ic.rtol;
       bs.atol = (Real)ic.atol;
-      const double inv = fmin(1.0 / (ic.rtol + ic.atol), 1.0e30);      // keeps FP32 squares in range
-      bs.inv_tol = (float)inv;
-      bs.rtol_f = (float)(ic.rtol * inv);
-      bs.atol_f = (float)(ic.atol * inv);
+      if constexpr (sizeof(Real) == 8) {
+        const double inv = fmin(1.0 / (ic.rtol + ic.atol), 1.0e30);      // keeps FP32 squares in range
+        bs.inv_tol = (float)inv;
+        bs.rtol_f = (float)(ic.rtol * inv);
+        bs.atol_f = (float)(ic.atol * inv);
+      }
     }
     for (int t = threadIdx.x; t < n_jj; t += blockDim.x) {
       const int jj = pc.jj_lo + t;
@@ -2473,7 +2481,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     constexpr bool kSplitLoad = split_final<Tab, Real>() && kKind == kFinalPass;
     Real* escr = reinterpret_cast<Real*>(p.escr) + ic.beam_off;
     Real* kst = Body::kStore ? reinterpret_cast<Real*>(p.kst) + ic.beam_off : nullptr;
-    const Real* ysrc = kSplitLoad ? yout : yin;
+    const Real* ysrc = kSplitLoad || Body::kReadOut ? yout : yin;
     const int ne = (int)ic.n_energy, na = (int)ic.n_angle;
     // biases of the mixed sums: a thread adds at most 2 (its + 1) contributions of |w| <= wmax (times the
     // geometry factor), |Y| <= 2, to an accumulator
@@ -2577,6 +2585,10 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
           vload_at(p, kSpanPlanes, yin + (size_t)c * p.plane_stride + l0, yo[c], 17);
         }
       }
+      if constexpr (Body::kReadBoth) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) vload_at(p, kSpanPlanes, yout + (size_t)c * p.plane_stride + l0, yo[c], 17);
+      }
       int jj = (int)fast_div(l0, ic.div_magic);
       int k = (int)l0 - jj * ne;
       bool paired = false;
@@ -2619,7 +2631,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
             Real y[NC], ev[NC], ov[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) y[c] = ys[c][v];
-            if constexpr (kSplitLoad) {
+            if constexpr (kSplitLoad || Body::kReadBoth) {
 #pragma unroll
               for (int c = 0; c < NC; ++c) { ev[c] = ep[c][v]; ov[c] = yo[c][v]; }
             }
@@ -2640,7 +2652,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
           if (++k == ne) { k = 0; ++jj; }
         }
       }
-      if constexpr (kKind == kFinalPass && !kSplitLoad) {
+      if constexpr ((kKind == kFinalPass && !kSplitLoad) || Body::kWriteOut) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) vstore_at(p, kSpanPlanes, yout + (size_t)c * p.plane_stride + l0, ys[c], 5);
       }
