@@ -814,8 +814,12 @@ int setup_launch_shape(xflat_t h, const xflat_config& c) {
   const bool resident = state_bytes <= (uint64_t)l2_bytes;
   h->block = c.block_size ? (int)c.block_size : (mixed_2f && !c.blocks_per_sm && resident ? 512 : 256);
   const int want_bps = c.blocks_per_sm ? (int)c.blocks_per_sm : ((mixed_2f ? 512 : 768) / h->block);
-  h->kernel = step_kernel_ptr(h->nf, h->precision, h->integrator, h->block, want_bps * h->block >= 768 ? 3 : 2,
-                              h->extended);
+  uint64_t T_all = 0;
+  for (auto& I : h->inst) T_all += I.n_pad;
+  // FP64: the two-block kernels once a block of a one-block grid has eight beams a thread
+  const int bps = mixed_2f ? (want_bps * h->block >= 768 ? 3 : 2)
+                           : (T_all >= 8ull * h->block * h->sm_count && c.blocks_per_sm != 1 ? 2 : 1);
+  h->kernel = step_kernel_ptr(h->nf, h->precision, h->integrator, h->block, bps, h->extended);
   if (!h->kernel) return fail(h, XFLAT_ERR_UNSUPPORTED, "no kernel for this flavour/precision/integrator");
   const size_t smax = smem_bytes(h->nf, h->real_size, max_jj_cap(h->nf, h->real_size, h->extended),
                                  table_stages(h->integrator), h->block, h->extended);
@@ -830,8 +834,6 @@ int setup_launch_shape(xflat_t h, const xflat_config& c) {
   // us with 128 on 32; 64 or 32 beams a block are no faster).  Beam shards of one problem that
   // together are smaller than one full grid keep the whole problem's blocks, so that they sum in the
   // same order as the unsharded run where a shard boundary falls between blocks.
-  uint64_t T_all = 0;
-  for (auto& I : h->inst) T_all += I.n_pad;
   const uint64_t T = h->shard ? h->shard_hi - h->shard_lo : T_all;
   const uint64_t G_max = (uint64_t)occ * h->sm_count;
   const auto ceil_div = [](uint64_t a, uint64_t b) { return (a + b - 1) / b; };

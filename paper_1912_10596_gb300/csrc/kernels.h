@@ -4,7 +4,8 @@
 namespace xflat {
 struct KParams;
 // The __global__ step kernel for (n_flavor, precision, integrator) built for the requested block
-// size and resident blocks per SM (mixed two-flavour kernels: 256 x 2 or 3, or 512 x 1; all others:
+// size and resident blocks per SM (mixed two-flavour kernels: 256 x 2 or 3, or 512 x 1; FP64 RK4 and DP45:
+// up to 256 threads, one or two blocks; all others:
 // up to 256 threads, one block), or nullptr.
 const void* step_kernel_ptr(int n_flavor, int precision, int integrator, int block, int blocks_per_sm,
                             bool extended = false);

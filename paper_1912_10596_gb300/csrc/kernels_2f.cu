@@ -20,8 +20,15 @@ const void* step_kernel_ptr_2f(int precision, int integrator, int block, int blo
   if (integrator == kLieAdaptive) return step_kernel_ptr_lie(precision, block, blocks_per_sm);
   if (block > 256) return (precision == 1 && block == 512) ? mixed_2f<1, 512>(integrator) : nullptr;
   if (precision == 0) {
-    if (integrator == kRK4) return (const void*)&step_kernel<Phys2<double>, TabRK4, double, false, 1>;
-    if (integrator == kDP45) return (const void*)&step_kernel<Phys2<double>, TabDP45, double, false, 1>;
+    // stored stages: two blocks per SM (128 registers) hide the plane loads' latency where every SM has
+    // work for them (4M beams, DP45, 3 steps on GB300: 5.38 ms with one block, 5.09 ms with two); a small
+    // problem is faster without the tighter registers (4096 beams, 16 RK4 steps: 770 and 789 us)
+    if (integrator == kRK4)
+      return blocks_per_sm >= 2 ? (const void*)&step_kernel<Phys2<double>, TabRK4, double, false, 2>
+                                : (const void*)&step_kernel<Phys2<double>, TabRK4, double, false, 1>;
+    if (integrator == kDP45)
+      return blocks_per_sm >= 2 ? (const void*)&step_kernel<Phys2<double>, TabDP45, double, false, 2>
+                                : (const void*)&step_kernel<Phys2<double>, TabDP45, double, false, 1>;
     if (integrator == kLieRK4) return (const void*)&step_kernel<Phys2<double>, TabCF4, double, true, 1>;
     if (integrator == kExpMid) return (const void*)&step_kernel<Phys2<double>, TabEM2, double, true, 1>;
     return nullptr;
