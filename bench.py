@@ -34,14 +34,14 @@ L2_BYTES = 129 * 1024 * 1024
 # DRAM traffic of one timed launch of the step kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
-STEP_TRAFFIC = {"bytes_per_launch": 51321600 + 173744640, "steps_per_launch": 8,
+STEP_TRAFFIC = {"bytes_per_launch": 51251200 + 173570560, "steps_per_launch": 8,
                 "code_sha256": "f8f7c6198b00e64bbe60cdc671a5c71a19647465bee8ab6dce02a883b0b44d34"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a
 # longer launch issues a little less): with the step time and the sampled SM clock it gives the
 # kernel's place under its instruction-issue ceiling (4 warp instructions per clock per SM).
-STEP_INSTRUCTIONS = {"warp_inst_per_step": 112139706, "code_sha256": STEP_TRAFFIC["code_sha256"]}
+STEP_INSTRUCTIONS = {"warp_inst_per_step": 112215206, "code_sha256": STEP_TRAFFIC["code_sha256"]}
 
 
 def issue_roofline(ms_per_step, sm_mhz, n_sm):

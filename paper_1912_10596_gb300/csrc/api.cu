@@ -118,6 +118,7 @@ struct xflat_s {
   // host mirrors
   std::vector<InstConst> ic;
   std::vector<InstDyn> dyn;
+  bool dyn_current = false;                // dyn equals the device's copy (no step launch since the last transfer)
   std::vector<Piece> pieces;
   std::vector<int> blk;
   const void* kernel = nullptr;
@@ -449,12 +450,18 @@ int upload_inst(xflat_t h) {
   return XFLAT_OK;
 }
 int upload_dyn(xflat_t h) {
+  h->dyn_current = false;
   CUDA_TRY(h, cudaMemcpyAsync(h->d_dyn, h->dyn.data(), sizeof(InstDyn) * h->dyn.size(), cudaMemcpyHostToDevice, h->stream));
+  h->dyn_current = true;
   return XFLAT_OK;
 }
+// The dynamics change on the device only in step launches (launch, graph replays): between them the host
+// copy is the device's, and the round trip (a synchronisation, ~12 us) is left out.
 int download_dyn(xflat_t h) {
+  if (h->dyn_current) return XFLAT_OK;
   CUDA_TRY(h, cudaMemcpyAsync(h->dyn.data(), h->d_dyn, sizeof(InstDyn) * h->dyn.size(), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  h->dyn_current = true;
   return XFLAT_OK;
 }
 
@@ -686,6 +693,7 @@ int launch(xflat_t h, int n_steps, int init_only, cudaStream_t stream, int shard
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  h->dyn_current = false;
   CUDA_TRY(h, cudaLaunchKernelExC(&cfg, h->kernel, args));
   h->launches++;
   return XFLAT_OK;
@@ -748,13 +756,9 @@ int clear_sync_words(xflat_t h) {
   return XFLAT_OK;
 }
 
-int read_words(xflat_t h, int& status, int& all_done) {
-  CUDA_TRY(h, cudaMemcpyAsync(h->h_words, h->d_words, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  status = h->h_words[0];
-  all_done = h->h_words[1];
+// checked build: name the first access the kernel found outside its allocation
+int check_bounds_words(xflat_t h, int& status) {
 #ifdef XFLAT_BOUNDS
-  // checked build: name the first access the kernel found outside its allocation
   Barrier b{};
   CUDA_TRY(h, cudaMemcpy(&b, h->d_bar, sizeof(Barrier), cudaMemcpyDeviceToHost));
   if (b.bounds_site) {
@@ -763,7 +767,17 @@ int read_words(xflat_t h, int& status, int& all_done) {
                                        ", byte offset " + std::to_string(b.bounds_off));
   }
 #endif
+  (void)h;
+  (void)status;
   return XFLAT_OK;
+}
+
+int read_words(xflat_t h, int& status, int& all_done) {
+  CUDA_TRY(h, cudaMemcpyAsync(h->h_words, h->d_words, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  status = h->h_words[0];
+  all_done = h->h_words[1];
+  return check_bounds_words(h, status);
 }
 
 // Compute the moments of the current state of every instance (stage 1 constants).
@@ -888,6 +902,7 @@ void* cur_plane(xflat_t h, uint32_t i) {
 int prepare_targets(xflat_t h, const double* r1, bool& any, bool& changed) {
   int rc;
   if ((rc = download_dyn(h))) return rc;
+  h->dyn_current = false;                  // edited here; the caller uploads it, or the edits are void
   any = false;
   changed = !h->moments_valid;
   for (size_t i = 0; i < h->inst.size(); ++i) {
@@ -952,16 +967,17 @@ int do_evolve(xflat_t h, const double* r1, bool sync_loop, uint32_t max_steps, i
     h->advancing = true;
     return XFLAT_OK;
   }
-  for (;;) {
+  int st = 0, ad = 0;
+  do {
     if ((rc = launch(h, (int)h->steps_per_launch, 0))) return rc;
-    int st, ad;
-    if ((rc = read_words(h, st, ad))) return rc;
-    if (st || ad) break;
-  }
-  if ((rc = download_dyn(h))) return rc;
+    // the status words and the dynamics in one synchronisation
+    CUDA_TRY(h, cudaMemcpyAsync(h->h_words, h->d_words, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = download_dyn(h))) return rc;
+    st = h->h_words[0];
+    ad = h->h_words[1];
+    if ((rc = check_bounds_words(h, st))) return rc;
+  } while (!st && !ad);
   h->moments_valid = true;
-  int st, ad;
-  if ((rc = read_words(h, st, ad))) return rc;
   for (auto& d : h->dyn)
     if (d.status) return fail(h, d.status, std::string("device status: ") + xflat_status_string(d.status));
   if (st) return fail(h, st, std::string("device status: ") + xflat_status_string(st));
@@ -1248,6 +1264,7 @@ int xflat_reset(xflat_t h, double r0_km) {
   if (!h) return XFLAT_ERR_INVAL;
   if (!is_fin(r0_km)) return fail(h, XFLAT_ERR_INVAL, "r0 not finite");
   int rc;
+  h->dyn_current = false;                  // edited here, uploaded below
   for (size_t i = 0; i < h->inst.size(); ++i) {
     if (r0_km < h->inst[i].cfg.R_km) return fail(h, XFLAT_ERR_INVAL, "r0 below R");
     reset_dyn(h, (uint32_t)i, r0_km);
@@ -1297,6 +1314,7 @@ int xflat_advance_graph(xflat_t h, uint32_t n_launches, uint32_t max_steps, int*
   if (!h->graph_exec || h->graph_launches != n_launches || h->graph_steps != max_steps)
     if ((rc = capture_graph(h, n_launches, max_steps))) return rc;
   if (done_out) *done_out = h->h_words[1];
+  h->dyn_current = false;
   CUDA_TRY(h, cudaGraphLaunch(h->graph_exec, h->stream));
   h->launches += n_launches;
   return XFLAT_OK;
