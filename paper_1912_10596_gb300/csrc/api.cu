@@ -251,37 +251,59 @@ __global__ void k_initial_state(Real* planes, uint64_t stride, uint64_t n_total,
     }
 }
 
-// native (Real, internal convention) -> double dst in the requested layout
+// native (Real, internal convention) -> double dst, NATIVE layout
 template <typename Real>
-__global__ void k_export(const Real* src, uint64_t stride, uint32_t n, uint32_t n_nu, int nf, int layout,
-                         double* dst) {
+__global__ void k_export(const Real* src, uint64_t stride, uint32_t n, int nc, double* dst) {
   const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= n) return;
-  const bool bar = b >= n_nu;
+  for (int c = 0; c < nc; ++c) dst[(uint64_t)c * n + b] = (double)src[(uint64_t)c * stride + b];
+}
+
+// ... MATRIX layout: one complex entry (16 bytes) a thread, so that a warp writes 512 contiguous bytes; the
+// planes' values are shared by the NF^2 threads of a beam through the L1.  (One beam a thread, GB300, 4M
+// beams: its stores of 8 bytes, 64 bytes apart, wrote every 128-byte line in 16 pieces; see k_flux_spectra
+// for the call's times.)
+template <typename Real, int NF>
+__global__ void k_export_matrix(const Real* src, uint64_t stride, uint32_t n, uint32_t n_nu, double2* dst) {
+  constexpr uint32_t kE = NF * NF;
+  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (uint64_t)n * kE) return;
+  const uint32_t b = (uint32_t)(t / kE), e = (uint32_t)(t % kE), row = e / NF, col = e % NF;
+  const double sg = b >= n_nu ? -1.0 : 1.0;       // antineutrinos: the paper's Pbar = conj(internal)
+  auto plane = [&](uint32_t c) { return (double)src[(uint64_t)c * stride + b]; };
+  double re, im = 0.0;
+  if constexpr (NF == 2) {
+    if (row == col) {
+      const double sz = plane(2);
+      re = 0.5 * (row == 0 ? 1 + sz : 1 - sz);
+    } else {
+      const double sy = plane(1);
+      re = 0.5 * plane(0);
+      im = row == 0 ? -0.5 * sy * sg : 0.5 * sy * sg;
+    }
+  } else {
+    if (row == col) {
+      re = plane(row);
+    } else {
+      const uint32_t c = 1 + 2 * (row + col);     // 01 -> planes 3, 4; 02 -> 5, 6; 12 -> 7, 8
+      const double v = plane(c + 1);
+      re = plane(c);
+      im = sg * (row < col ? v : -v);
+    }
+  }
+  dst[t] = make_double2(re, im);
+}
+
+template <typename Real>
+void export_state(const void* src, uint64_t stride, uint32_t n, int nf, int layout, double* dst, cudaStream_t st) {
+  const Real* p = (const Real*)src;
   if (layout == XFLAT_LAYOUT_NATIVE) {
-    const int nc = nf == 2 ? 3 : 9;
-    for (int c = 0; c < nc; ++c) dst[(uint64_t)c * n + b] = (double)src[(uint64_t)c * stride + b];
+    k_export<Real><<<(n + 255) / 256, 256, 0, st>>>(p, stride, n, nf == 2 ? 3 : 9, dst);
     return;
   }
-  double* m = dst + (uint64_t)b * 2 * nf * nf;
-  const double sg = bar ? -1.0 : 1.0;       // antineutrinos: the paper's Pbar = conj(internal)
-  if (nf == 2) {
-    const double sx = src[b], sy = src[stride + b], sz = src[2 * stride + b];
-    m[0] = 0.5 * (1 + sz); m[1] = 0;
-    m[2] = 0.5 * sx;       m[3] = -0.5 * sy * sg;
-    m[4] = 0.5 * sx;       m[5] = 0.5 * sy * sg;
-    m[6] = 0.5 * (1 - sz); m[7] = 0;
-  } else {
-    double v[9];
-    for (int c = 0; c < 9; ++c) v[c] = (double)src[(uint64_t)c * stride + b];
-    const double re[3][3] = {{v[0], v[3], v[5]}, {v[3], v[1], v[7]}, {v[5], v[7], v[2]}};
-    const double im[3][3] = {{0, v[4], v[6]}, {-v[4], 0, v[8]}, {-v[6], -v[8], 0}};
-    for (int a = 0; a < 3; ++a)
-      for (int c = 0; c < 3; ++c) {
-        m[(a * 3 + c) * 2] = re[a][c];
-        m[(a * 3 + c) * 2 + 1] = sg * im[a][c];
-      }
-  }
+  const unsigned nb = (unsigned)(((uint64_t)n * nf * nf + 255) / 256);
+  if (nf == 2) k_export_matrix<Real, 2><<<nb, 256, 0, st>>>(p, stride, n, n / 2, (double2*)dst);
+  else k_export_matrix<Real, 3><<<nb, 256, 0, st>>>(p, stride, n, n / 2, (double2*)dst);
 }
 
 template <typename Real>
@@ -323,13 +345,19 @@ __global__ void k_pee(const Real* src, uint64_t stride, uint32_t n, int nf, doub
 
 // Number-flux weighted mean of P_ee over nu beams, deterministic and spread over the GPU (the
 // sums are FP64, whose pipe is narrow: one block would take milliseconds at 2M beams).  One warp
-// per angle bin sums N_e,k P_ee over energies (lanes in a fixed order, then a fixed shuffle tree);
-// one block then sums du_j times the rows in a fixed tree.
-__global__ void k_pee_rows(const double* pee, const double* N_e, uint32_t ne, uint32_t na, double* rows) {
+// per angle bin sums N_e,k P_ee over energies, straight from the state (lanes in a fixed order, then a
+// fixed shuffle tree); one block then sums du_j times the rows in a fixed tree.
+template <typename Real>
+__global__ void k_pee_rows(const Real* src, uint64_t stride, int nf, const double* N_e, uint32_t ne, uint32_t na,
+                           double* rows) {
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= na) return;
+  const Real* p = src + (nf == 2 ? 2 * stride : 0) + (uint64_t)warp * ne;
   double s = 0.0;
-  for (uint32_t k = lane; k < ne; k += 32) s += N_e[k] * pee[(uint64_t)warp * ne + k];
+  for (uint32_t k = lane; k < ne; k += 32) {
+    const double v = (double)p[k];
+    s += N_e[k] * (nf == 2 ? 0.5 * (1.0 + v) : v);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) rows[warp] = s;
@@ -348,29 +376,65 @@ __global__ void k_pee_final(const double* rows, const double* du, uint32_t na, d
   if (threadIdx.x == 0) out[0] = den > 0 ? sn[0] / den : 0.0;
 }
 
-// Number-flux energy spectra: one thread per (species, flavour a, energy k), angle bins summed in
-// order: Phi = sum_j du_j [N_e P_ea + N_x (1 - P_ea)], P_ea the a-a entry of the electron-flavour
-// state (unitarity: the x states carry 1 - P_ea into flavour a).
-template <typename Real>
-__global__ void k_flux_spectra(const Real* src, uint64_t stride, uint32_t ne, uint32_t na, int nf,
-                               const double* N, const double* du, double* flux) {
+// Number-flux energy spectra, Phi = sum_j du_j [N_e P_ea + N_x (1 - P_ea)], P_ea the a-a entry of the
+// electron-flavour state (unitarity: the x states carry 1 - P_ea into flavour a): first, per chunk of
+// angle bins, S_a = sum du_j P_ea and T_a = sum du_j (1 - P_ea) of every energy (a block takes 32
+// energies of one species, each of its 8 warps every eighth angle bin of the chunk), then the chunks in
+// order and the spectra.  Deterministic.  (GB300, 4M beams FP64: one thread an energy and flavour walked
+// 2000 angle bins; a call that sets the state and reads matrices, moments, spectra and the mean took
+// 1150 us, 487 us with these kernels.)
+constexpr int kFluxWarps = 8;
+template <typename Real, int NF>
+__global__ void k_flux_rows(const Real* src, uint64_t stride, uint32_t ne, uint32_t na, uint32_t chunk, const double* du,
+                            double* part) {
+  __shared__ double sm[kFluxWarps][2 * NF][32];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t k = blockIdx.x * 32 + lane, sig = blockIdx.z;
+  const uint32_t j1 = min(na, (blockIdx.y + 1) * chunk);
+  double S[NF], T[NF];
+#pragma unroll
+  for (int a = 0; a < NF; ++a) { S[a] = 0.0; T[a] = 0.0; }
+  if (k < ne) {
+    for (uint32_t j = blockIdx.y * chunk + warp; j < j1; j += kFluxWarps) {
+      const uint64_t b = ((uint64_t)sig * na + j) * ne + k;
+      const double d = du[j];
+      if constexpr (NF == 2) {
+        const double sz = (double)src[2 * stride + b];
+        S[0] = fma(d, 0.5 + 0.5 * sz, S[0]);
+        T[0] = fma(d, 0.5 - 0.5 * sz, T[0]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < NF; ++a) {
+          const double P = (double)src[(uint64_t)a * stride + b];
+          S[a] = fma(d, P, S[a]);
+          T[a] = fma(d, 1.0 - P, T[a]);
+        }
+      }
+    }
+  }
+  if constexpr (NF == 2) { S[1] = T[0]; T[1] = S[0]; }
+#pragma unroll
+  for (int a = 0; a < NF; ++a) { sm[warp][2 * a][lane] = S[a]; sm[warp][2 * a + 1][lane] = T[a]; }
+  __syncthreads();
+  for (uint32_t t = threadIdx.x; t < 2 * NF * 32; t += blockDim.x) {
+    double v = 0.0;
+    for (int w = 0; w < kFluxWarps; ++w) v += sm[w][t >> 5][t & 31];
+    const uint32_t kk = blockIdx.x * 32 + (t & 31);
+    if (kk < ne) part[(((uint64_t)blockIdx.y * 2 + sig) * 2 * NF + (t >> 5)) * ne + kk] = v;
+  }
+}
+
+__global__ void k_flux_final(const double* part, uint32_t chunks, uint32_t ne, int nf, const double* N, double* flux) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2u * nf * ne) return;
   const uint32_t sig = t / (nf * ne), a = (t / ne) % nf, k = t % ne;
-  const double Ne = N[(sig * nf + 0) * ne + k], Nx = N[(sig * nf + 1) * ne + k];
-  double f = 0.0;
-  for (uint32_t j = 0; j < na; ++j) {
-    const uint64_t b = ((uint64_t)sig * na + j) * ne + k;
-    double P;
-    if (nf == 2) {
-      const double sz = (double)src[2 * stride + b];
-      P = a == 0 ? 0.5 * (1.0 + sz) : 0.5 * (1.0 - sz);
-    } else {
-      P = (double)src[(uint64_t)a * stride + b];
-    }
-    f += du[j] * (Ne * P + Nx * (1.0 - P));
+  double S = 0.0, T = 0.0;
+  for (uint32_t c = 0; c < chunks; ++c) {
+    const double* p = part + (((uint64_t)c * 2 + sig) * 2 * nf + 2 * a) * ne + k;
+    S += p[0];
+    T += p[ne];
   }
-  flux[t] = f;
+  flux[t] = N[(sig * nf + 0) * ne + k] * S + N[(sig * nf + 1) * ne + k] * T;
 }
 
 // rows of an instance's energy table: vacuum entries, then the weights of nu and nubar
@@ -1392,7 +1456,7 @@ int xflat_get_rho_inst(xflat_t h, uint32_t inst, void* dst, int dst_is_device, i
   int rc;
   if ((rc = download_dyn(h))) return rc;
   const HostInst& I = h->inst[inst];
-  const uint32_t n = I.n_beams, n_nu = n / 2;
+  const uint32_t n = I.n_beams;
   const size_t bytes = layout == XFLAT_LAYOUT_MATRIX ? (size_t)n * 2 * h->nf * h->nf * 8 : (size_t)n * h->nc * 8;
   double* target = (double*)dst;
   if (!dst_is_device) {
@@ -1400,9 +1464,16 @@ int xflat_get_rho_inst(xflat_t h, uint32_t inst, void* dst, int dst_is_device, i
     target = h->d_stage;
   }
   const void* src = cur_plane(h, inst);
-  const unsigned nb = (n + 255) / 256;
-  if (h->real_size == 8) k_export<double><<<nb, 256, 0, h->stream>>>((const double*)src, h->stride, n, n_nu, h->nf, layout, target);
-  else k_export<float><<<nb, 256, 0, h->stream>>>((const float*)src, h->stride, n, n_nu, h->nf, layout, target);
+  // an odd device pointer (8-byte aligned only) goes through the staging buffer: matrices are written in
+  // 16-byte entries
+  const bool via = dst_is_device && layout == XFLAT_LAYOUT_MATRIX && ((uintptr_t)dst & 15u) != 0;
+  if (via) {
+    if ((rc = ensure_stage(h, bytes))) return rc;
+    target = h->d_stage;
+  }
+  if (h->real_size == 8) export_state<double>(src, h->stride, n, h->nf, layout, target, h->stream);
+  else export_state<float>(src, h->stride, n, h->nf, layout, target, h->stream);
+  if (via) CUDA_TRY(h, cudaMemcpyAsync(dst, target, bytes, cudaMemcpyDeviceToDevice, h->stream));
   CUDA_TRY(h, cudaGetLastError());
   if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(dst, target, bytes, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -1460,22 +1531,26 @@ int xflat_pee_inst(xflat_t h, uint32_t inst, double* pee_per_beam, double* pee_m
   if ((rc = download_dyn(h))) return rc;
   const HostInst& I = h->inst[inst];
   const uint32_t n = I.n_beams, ne = I.cfg.n_energy, na = angle_bins(I.cfg);
-  const size_t need = ((size_t)n + ne + na + 2) * 8;
+  const size_t need = ((pee_per_beam ? (size_t)n : 0) + ne + na + 2) * 8;
   if ((rc = ensure_stage(h, need))) return rc;
   double* pee = h->d_stage;
-  double* Ne = pee + n;
+  double* Ne = pee + (pee_per_beam ? n : 0);
   double* rows = Ne + ne;
   double* mean = rows + na;
   const void* src = cur_plane(h, inst);
   const unsigned nb = (n + 255) / 256;
-  if (h->real_size == 8) k_pee<double><<<nb, 256, 0, h->stream>>>((const double*)src, h->stride, n, h->nf, pee);
-  else k_pee<float><<<nb, 256, 0, h->stream>>>((const float*)src, h->stride, n, h->nf, pee);
+  if (pee_per_beam) {
+    if (h->real_size == 8) k_pee<double><<<nb, 256, 0, h->stream>>>((const double*)src, h->stride, n, h->nf, pee);
+    else k_pee<float><<<nb, 256, 0, h->stream>>>((const float*)src, h->stride, n, h->nf, pee);
+  }
   CUDA_TRY(h, cudaMemcpyAsync(Ne, I.N.data(), sizeof(double) * ne, cudaMemcpyHostToDevice, h->stream));
   // denominator sum_j du_j sum_k N_e,k (host, fixed order)
   double sN = 0.0, sdu = 0.0;
   for (uint32_t k = 0; k < ne; ++k) sN += I.N[k];
   for (uint32_t j = 0; j < na; ++j) sdu += I.du[j];
-  k_pee_rows<<<(unsigned)((32ull * na + 255) / 256), 256, 0, h->stream>>>(pee, Ne, ne, na, rows);
+  const unsigned nrb = (unsigned)((32ull * na + 255) / 256);
+  if (h->real_size == 8) k_pee_rows<double><<<nrb, 256, 0, h->stream>>>((const double*)src, h->stride, h->nf, Ne, ne, na, rows);
+  else k_pee_rows<float><<<nrb, 256, 0, h->stream>>>((const float*)src, h->stride, h->nf, Ne, ne, na, rows);
   k_pee_final<<<1, 1024, 0, h->stream>>>(rows, h->d_du + I.a_off, na, sN * sdu, mean);
   CUDA_TRY(h, cudaGetLastError());
   if (pee_per_beam) CUDA_TRY(h, cudaMemcpyAsync(pee_per_beam, pee, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
@@ -1500,14 +1575,27 @@ int xflat_flux_spectra(xflat_t h, uint32_t inst, double* flux) {
   const uint32_t ne = I.cfg.n_energy, na = angle_bins(I.cfg);
   const int nf = h->nf;
   const size_t nval = 2ull * nf * ne;
-  if ((rc = ensure_stage(h, 2 * nval * sizeof(double)))) return rc;
+  // chunks of angle bins: enough blocks for four an SM, at least one angle bin a warp
+  const uint32_t tiles = (ne + 31) / 32;
+  const uint32_t want = std::max(1u, 4u * (uint32_t)h->sm_count / (2u * tiles));
+  const uint32_t chunk = std::max<uint32_t>(kFluxWarps, (na + want - 1) / want), chunks = (na + chunk - 1) / chunk;
+  if ((rc = ensure_stage(h, (2 * nval + 2ull * nval * chunks) * sizeof(double)))) return rc;
   double* dN = h->d_stage;
   double* dflux = dN + nval;
+  double* part = dflux + nval;
   CUDA_TRY(h, cudaMemcpyAsync(dN, I.N.data(), nval * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   const void* src = cur_plane(h, inst);
-  const unsigned nb = (unsigned)((nval + 127) / 128);
-  if (h->real_size == 8) k_flux_spectra<double><<<nb, 128, 0, h->stream>>>((const double*)src, h->stride, ne, na, nf, dN, h->d_du + I.a_off, dflux);
-  else k_flux_spectra<float><<<nb, 128, 0, h->stream>>>((const float*)src, h->stride, ne, na, nf, dN, h->d_du + I.a_off, dflux);
+  const double* du = h->d_du + I.a_off;
+  const dim3 grid(tiles, chunks, 2);
+  const unsigned thr = 32 * kFluxWarps;
+  if (h->real_size == 8) {
+    if (nf == 2) k_flux_rows<double, 2><<<grid, thr, 0, h->stream>>>((const double*)src, h->stride, ne, na, chunk, du, part);
+    else k_flux_rows<double, 3><<<grid, thr, 0, h->stream>>>((const double*)src, h->stride, ne, na, chunk, du, part);
+  } else {
+    if (nf == 2) k_flux_rows<float, 2><<<grid, thr, 0, h->stream>>>((const float*)src, h->stride, ne, na, chunk, du, part);
+    else k_flux_rows<float, 3><<<grid, thr, 0, h->stream>>>((const float*)src, h->stride, ne, na, chunk, du, part);
+  }
+  k_flux_final<<<(unsigned)((nval + 127) / 128), 128, 0, h->stream>>>(part, chunks, ne, nf, dN, dflux);
   CUDA_TRY(h, cudaGetLastError());
   CUDA_TRY(h, cudaMemcpyAsync(flux, dflux, nval * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
