@@ -39,7 +39,7 @@ struct AdjParams {
   double* a;                            // adjoint of the state
   double* ybar;                         // adjoint contributions of the stages so far this step
   double* v;                            // cotangent of the current stage derivative
-  double* gw;                           // [n] dJ/dw_b (w_b = du_j g_{sigma,k})
+  double* gw;                           // [n] du_j dJ/dw_b (w_b = du_j g_{sigma,k})
   double* gth;                          // [n] dJ/dtheta_v per beam
   double* part;                         // [grid][kAdjPartStride] block partials
   double* glob;                         // [kGlobWords] broadcast values
@@ -56,7 +56,7 @@ constexpr int kAdjBlock = 256;
 
 // Per-energy sums over angle bins of the final quantities (one thread per (sigma, k)):
 //   pee_sum[k]    = sum_j du_j (P_ee(nu, j, k) - J)         (k < n_energy; J from the forward launch)
-//   gw_sum[s][k]  = sum_j du_j gw[(s, j, k)]
+//   gw_sum[s][k]  = sum_j gw[(s, j, k)] (gw carries du_j)
 //   gth_sum[s][k] = sum_j gth[(s, j, k)]
 cudaError_t adjoint_energy_sums(const AdjParams& p, double* pee_sum, double* gw_sum, double* gth_sum,
                                 cudaStream_t stream);

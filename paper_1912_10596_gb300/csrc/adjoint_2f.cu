@@ -16,6 +16,12 @@
 //   v4 = h/6 a',  v3 = h/3 a' + h sbar4,  v2 = h/3 a' + h/2 sbar3,  v1 = h/6 a' + h/2 sbar2,
 //   a = a' + sbar4 + sbar3 + sbar2 + sbar1.
 //
+// What bounds it: FP64 operations on GB300's two-lane pipe and the fixed time of a pass (12 a step).  So
+// everything that the beams of an angle row share is tabulated once a step and stage (AdjRow, AdjBack: an
+// assembled K is two FMAs), moments are summed within rows, reductions spread over the lanes, and the
+// next stage's strengths are computed beside the sum over blocks.  200 E x 400 u, 128 steps, K = 64:
+// 43.1 ms with per-beam assembly and five geometries a pass, 32.1 ms so.
+//
 // Memory: the forward launch stores the state every K steps (checkpoints); each backward launch
 // re-runs one segment of K steps forward from its checkpoint, storing every step's start state and
 // stage constants, then runs the segment's steps backwards.  Every pass over the beams ends in a
@@ -26,13 +32,21 @@
 namespace xflat {
 namespace {
 
-constexpr int kAdjGeoSets = 5;       // radii per pass whose geometry is tabulated
-constexpr int kAdjGeoRows = 64;      // angle rows per block the table holds
+constexpr int kAdjSlots = 5;         // stages whose rows are tabulated at a time
+constexpr int kAdjRows = 64;         // angle rows per block the tables hold
+
+// What the beams of an angle row share at a stage: the geometry (q = 1/cos th, t1 = 1/cos th - 1,
+// t2 = 1 - cos th), and K = eta omega (qb0, 0, qb2) + g.
+struct AdjRow { double q, t1, t2, qb0, qb2, g[3]; };
+// ... and at the stage whose adjoint is finished: brd = du (t1 Dbar + J1bar), and q dB/dtheta.
+struct AdjBack { double brd[3], qd0, qd2; };
 
 struct AdjShared {
-  Geo geo[kAdjGeoSets][kAdjGeoRows];    // per pass: geometry of this block's angle rows
+  AdjRow row[kAdjSlots][kAdjRows];
+  AdjBack back[kAdjRows];
   double scratch[32 * 6];
   double tot[8];
+  double str[2];                        // mu, lambda of the formed stage (forward, last block)
   double scf[kAdjStageVals];            // constants of the stage finished in this pass
   double scs[4][kAdjStageVals];         // constants of the formed stage's step (backward: all 4)
   double gl[8];                         // broadcast adjoint moments of the finished stage
@@ -40,44 +54,49 @@ struct AdjShared {
   unsigned int gen;
 };
 
-struct BeamC {
-  double eo, w, u, ow;                  // eta omega, moment weight, u_j, objective weight (nu)
-  uint32_t jj;                          // combined row sigma n_angle + j
-};
-
-__device__ __forceinline__ BeamC beam_consts(const AdjParams& p, uint32_t b) {
-  const uint32_t per = p.n_angle * p.n_energy;
-  const uint32_t sig = b >= per ? 1u : 0u;
-  const uint32_t rem = b - sig * per;
-  const uint32_t j = rem / p.n_energy, k = rem - j * p.n_energy;
-  BeamC c;
-  c.eo = sig ? -p.omega[k] : p.omega[k];
-  c.w = p.du[j] * p.g[sig * p.n_energy + k];
-  c.u = p.u[j];
-  c.ow = sig ? 0.0 : p.du[j] * p.objw[k];
-  c.jj = sig * p.n_angle + j;
-  return c;
+__device__ __forceinline__ void row_geometry(const AdjParams& p, uint32_t jj, double x, AdjRow& r) {
+  const uint32_t j = jj >= p.n_angle ? jj - p.n_angle : jj;
+  const Geo g = geometry(p.u[j], x);
+  r.q = g.q;
+  r.t1 = g.t1;
+  r.t2 = g.t2;
+  r.qb0 = g.q * p.ic.B[0];
+  r.qb2 = g.q * p.ic.B[2];
+}
+// sc: mu D, mu J1, lambda
+__device__ __forceinline__ void row_coupling(const double* sc, AdjRow& r) {
+  r.g[0] = r.q * (sc[0] + r.t2 * sc[3]);
+  r.g[1] = r.q * (sc[1] + r.t2 * sc[4]);
+  r.g[2] = r.q * (sc[6] + sc[2] + r.t2 * sc[5]);
+}
+__device__ __forceinline__ AdjBack row_back(const AdjParams& p, uint32_t jj, const AdjRow& r, const double* gl) {
+  const double du = p.du[jj >= p.n_angle ? jj - p.n_angle : jj];
+  const double c2 = -p.ic.B[2], s2 = p.ic.B[0];              // B = (sin 2th, 0, -cos 2th)
+  AdjBack b;
+  for (int i = 0; i < 3; ++i) b.brd[i] = du * (r.t1 * gl[i] + gl[3 + i]);
+  b.qd0 = r.q * (2.0 * c2);                                   // dB/dtheta = (2 cos 2th, 0, 2 sin 2th)
+  b.qd2 = r.q * (2.0 * s2);
+  return b;
 }
 
-// Geometry (1/cos, 1/cos - 1, 1 - cos) of every angle row of the beams [b0, b1) at up to
-// kAdjGeoSets radii (R^2/r^2 = xof(set)): one FP64 square root and two divisions per (row,
-// radius) instead of per beam, which GB300 would run on its two-lane FP64 pipe.  Returns whether
-// the rows fit the table (same answer in every thread); if not, callers compute per beam.  The
-// caller's __syncthreads publishes the table.
-template <class XOf>
-__device__ bool fill_geo(const AdjParams& p, AdjShared& S, uint32_t b0, uint32_t b1, XOf xof, uint32_t& row0) {
-  row0 = b0 / p.n_energy;
-  const uint32_t last = b1 > b0 ? (b1 - 1) / p.n_energy : row0;
-  const int rows = (int)(last - row0 + 1);
-  if (b1 <= b0 || rows > kAdjGeoRows) return false;
-  for (int t = threadIdx.x; t < kAdjGeoSets * rows; t += blockDim.x) {
-    const int set = t / rows, r = t - set * rows;
-    const uint32_t jj = row0 + r;
-    const uint32_t j = jj >= p.n_angle ? jj - p.n_angle : jj;
-    S.geo[set][r] = geometry(p.u[j], xof(set));
+// This block's beams [b0, b1), its rows from row0 on (tab: they fit the tables; the same in every thread.
+// If not, the row values are computed per beam), and this thread's share: each warp a contiguous run, so
+// that a thread stays in one row for many beams (row sums of the moments, as in the step kernel).
+struct AdjShare {
+  uint32_t b0, b1, row0, rows, first, end;
+  bool tab;
+  __device__ explicit AdjShare(const AdjParams& p) {
+    const uint64_t n = p.n_beams;
+    b0 = (uint32_t)(n * blockIdx.x / gridDim.x);
+    b1 = (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
+    row0 = fast_div(b0, p.ic.div_magic);
+    rows = b1 > b0 ? fast_div(b1 - 1, p.ic.div_magic) - row0 + 1 : 0;
+    tab = rows > 0 && rows <= kAdjRows;
+    const uint32_t run = (b1 - b0 + blockDim.x - 1) / blockDim.x * 32u, w = threadIdx.x >> 5;
+    first = b0 + w * run + (threadIdx.x & 31);
+    end = min(b1, b0 + (w + 1) * run);
   }
-  return true;
-}
+};
 
 __device__ __forceinline__ void ld3(const double* base, uint64_t n, uint32_t b, double (&x)[3]) {
   x[0] = base[b];
@@ -98,11 +117,10 @@ __device__ __forceinline__ double dot(const double (&a)[3], const double (&b)[3]
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// K_b at a stage with constants sc (mu D, mu J1, lambda, x) and geometry g.
-__device__ __forceinline__ void kvec(const double* sc, const Geo& g, double eo, const double* B, double (&K)[3]) {
-  K[0] = g.q * (eo * B[0] + sc[0] + g.t2 * sc[3]);
-  K[1] = g.q * (sc[1] + g.t2 * sc[4]);
-  K[2] = g.q * (eo * B[2] + sc[6] + sc[2] + g.t2 * sc[5]);
+__device__ __forceinline__ void kvec(const AdjRow& r, double eo, double (&K)[3]) {
+  K[0] = fma(eo, r.qb0, r.g[0]);
+  K[1] = r.g[1];
+  K[2] = fma(eo, r.qb2, r.g[2]);
 }
 
 // RK4: stage s (1..4) forms Y_s = y + a_s h k_{s-1}; weights of k_s in the update.
@@ -114,23 +132,33 @@ __device__ __forceinline__ double stage_radius(const AdjParams& p, int n, int s)
   return (p.r0 + (double)n * p.h) + rk_c(s) * p.h;
 }
 
-// Block partials -> grid barrier -> the last block sums them in block order into S.tot.
-template <int NV>
-__device__ int grid_reduce(const AdjParams& p, AdjShared& S, double (&v)[NV]) {
-  block_sum<NV>(v, S.scratch);
-  if (threadIdx.x == 0) {
+// Block partials -> grid barrier -> the last block sums them in block order into S.tot, while one of its
+// idle warps runs `beside` (work that does not need the sums).
+template <int NV, class Beside>
+__device__ int grid_reduce(const AdjParams& p, AdjShared& S, double (&v)[NV], Beside beside) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int idx = 0, left = NV;
+  bool valid = true;
+  const double s = reduce_scatter<NV, 16, double>(v, lane, idx, left, valid);
+  if (valid) S.scratch[warp * NV + idx] = s;
+  __syncthreads();
+  for (int t = threadIdx.x; t < (NV * 16 + 31) / 32 * 32; t += blockDim.x) {
+    const int c = t >> 4, w = t & 15;
+    double x = w < nw && c < NV ? S.scratch[w * NV + c] : 0.0;
 #pragma unroll
-    for (int c = 0; c < NV; ++c) p.part[(size_t)blockIdx.x * kAdjPartStride + c] = v[c];
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (w == 0 && c < NV) p.part[(size_t)blockIdx.x * kAdjPartStride + c] = x;
   }
   const int res = barrier_arrive(p.bar, gridDim.x, p.timeout_ns, p.status, &S.flag, &S.gen) & 0xf;
   if (res == kBarLast) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < NV) {
       double s = 0.0;
       for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(&p.part[(size_t)b * kAdjPartStride + warp]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
       if (lane == 0) S.tot[warp] = s;
+    } else if (warp == NV && lane == 0) {
+      beside();
     }
     __syncthreads();
   }
@@ -148,40 +176,77 @@ __device__ __forceinline__ void release(const AdjParams& p, AdjShared& S) {
 __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int count, bool store_seg,
                               bool store_ck, bool finish) {
   const uint64_t n = p.n_beams;
-  const uint32_t b0 = (uint32_t)(n * blockIdx.x / gridDim.x), b1 = (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
+  const AdjShare sh(p);
   const int P = 4 * count;
   for (int pp = 0; pp <= P; ++pp) {
     if (pp == P && !finish) break;
     const int sp = pp > 0 ? ((pp - 1) & 3) + 1 : 0;        // stage finished in this pass
     const int s = (pp & 3) + 1, m = pp >> 2;                // stage formed in this pass
     const int nstep = n_first + m;
+    const int slot = pp & 1;                                // rows of the formed stage; the other: the finished one's
+    double x_s = 0.0;
+    if (pp < P) {
+      const double r = stage_radius(p, nstep, s);
+      x_s = p.ic.R2 / (r * r);
+    }
     if (pp > 0 && threadIdx.x < kAdjStageVals) S.scf[threadIdx.x] = __ldcg(&p.glob[threadIdx.x]);
-    const double x_s = pp < P ? p.ic.R2 / (stage_radius(p, nstep, s) * stage_radius(p, nstep, s)) : 0.0;
-    // geometry sets: 0 the finished stage (its R^2/r^2 was published with its constants), 1 the
-    // formed stage
-    uint32_t row0;
-    const bool tab = fill_geo(p, S, b0, b1, [&](int set) {
-      return set == 0 ? (pp > 0 ? __ldcg(&p.glob[7]) : 0.0) : set == 1 ? x_s : 0.0;
-    }, row0);
     __syncthreads();
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (uint32_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-      const BeamC c = beam_consts(p, b);
+    // the formed stage's geometry; the finished stage's, tabulated in the pass before, gets its couplings
+    if (sh.tab) {
+      for (uint32_t t = threadIdx.x; t < 2 * sh.rows; t += blockDim.x) {
+        const uint32_t r = t < sh.rows ? t : t - sh.rows;
+        if (t < sh.rows) {
+          if (pp < P) row_geometry(p, sh.row0 + r, x_s, S.row[slot][r]);
+        } else if (pp > 0) {
+          row_coupling(S.scf, S.row[slot ^ 1][r]);
+        }
+      }
+    }
+    __syncthreads();
+    auto finished = [&](uint32_t jj) {
+      if (sh.tab) return S.row[slot ^ 1][jj - sh.row0];
+      AdjRow r;
+      row_geometry(p, jj, S.scf[7], r);
+      row_coupling(S.scf, r);
+      return r;
+    };
+    double acc[6] = {0, 0, 0, 0, 0, 0}, rs[3] = {0, 0, 0};
+    auto flush = [&](uint32_t jj) {
+      const double du = p.du[jj >= p.n_angle ? jj - p.n_angle : jj];
+      double t1;
+      if (sh.tab) {
+        t1 = S.row[slot][jj - sh.row0].t1;
+      } else {
+        AdjRow r;
+        row_geometry(p, jj, x_s, r);
+        t1 = r.t1;
+      }
+      const double dt = du * t1;
+      for (int i = 0; i < 3; ++i) {
+        acc[i] = fma(dt, rs[i], acc[i]);
+        acc[3 + i] = fma(du, rs[i], acc[3 + i]);
+        rs[i] = 0.0;
+      }
+    };
+    uint32_t cur = 0xffffffffu;
+    for (uint32_t b = sh.first; b < sh.end; b += 32) {
+      const uint32_t jj = fast_div(b, p.ic.div_magic), k = b - jj * p.n_energy;
+      const bool bar = jj >= p.n_angle;
       double y[3], kl[3];
       ld3(p.y, n, b, y);
       ld3(p.klast, n, b, kl);
       if (pp > 0) {
-        double ys[3], K[3], k[3], ks[3];
+        const double om = p.omega[k], eo = bar ? -om : om;
+        double ys[3], K[3], kk[3], ks[3];
         const double as = sp == 1 ? 0.0 : rk_a(sp) * p.h;
         for (int i = 0; i < 3; ++i) ys[i] = sp == 1 ? y[i] : y[i] + as * kl[i];
-        const Geo g = tab ? S.geo[0][c.jj - row0] : geometry(c.u, S.scf[7]);
-        kvec(S.scf, g, c.eo, p.ic.B, K);
-        cross(K, ys, k);
+        kvec(finished(jj), eo, K);
+        cross(K, ys, kk);
         if (sp == 1) {
-          for (int i = 0; i < 3; ++i) ks[i] = k[i];
+          for (int i = 0; i < 3; ++i) ks[i] = kk[i];
         } else {
           ld3(p.ksum, n, b, ks);
-          for (int i = 0; i < 3; ++i) ks[i] += rk_w(sp) * k[i];
+          for (int i = 0; i < 3; ++i) ks[i] += rk_w(sp) * kk[i];
         }
         if (sp == 4) {
           for (int i = 0; i < 3; ++i) y[i] = y[i] + (p.h / 6.0) * ks[i];
@@ -189,7 +254,7 @@ __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int
         } else {
           st3(p.ksum, n, b, ks);
         }
-        for (int i = 0; i < 3; ++i) kl[i] = k[i];
+        for (int i = 0; i < 3; ++i) kl[i] = kk[i];
         st3(p.klast, n, b, kl);
       }
       if (pp < P) {
@@ -197,34 +262,25 @@ __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int
           if (store_seg) st3(p.seg + (size_t)m * 3 * n, n, b, y);
           if (store_ck && nstep % p.ck_every == 0) st3(p.ck + (size_t)(nstep / p.ck_every) * 3 * n, n, b, y);
         }
-        double ys[3];
-        const double as = s == 1 ? 0.0 : rk_a(s) * p.h;
-        for (int i = 0; i < 3; ++i) ys[i] = s == 1 ? y[i] : y[i] + as * kl[i];
-        const Geo g = tab ? S.geo[1][c.jj - row0] : geometry(c.u, x_s);
-        const double wt = c.w * g.t1;
-        for (int i = 0; i < 3; ++i) {
-          acc[i] += wt * ys[i];
-          acc[3 + i] += c.w * ys[i];
+        if (jj != cur) {
+          if (cur != 0xffffffffu) flush(cur);
+          cur = jj;
         }
+        const double as = s == 1 ? 0.0 : rk_a(s) * p.h, g = p.g[(bar ? p.n_energy : 0u) + k];
+        for (int i = 0; i < 3; ++i) rs[i] = fma(g, s == 1 ? y[i] : y[i] + as * kl[i], rs[i]);
       }
     }
     if (pp == P) break;
-    const int res = grid_reduce<6>(p, S, acc);
+    if (cur != 0xffffffffu) flush(cur);
+    const int res = grid_reduce<6>(p, S, acc, [&] { strengths(p.ic, stage_radius(p, nstep, s), S.str[0], S.str[1]); });
     if (res == kBarAbort) return false;
     if (res == kBarLast) {
-      if (threadIdx.x == 0) {
-        const double r = stage_radius(p, nstep, s);
-        double mu, lam;
-        strengths(p.ic, r, mu, lam);
-        double sc[kAdjStageVals];
-        for (int i = 0; i < 6; ++i) sc[i] = mu * S.tot[i];
-        sc[6] = lam;
-        sc[7] = x_s;
-        sc[8] = mu;
-        sc[9] = 0.0;
-        for (int i = 0; i < kAdjStageVals; ++i) p.glob[i] = sc[i];
-        if (store_seg)
-          for (int i = 0; i < kAdjStageVals; ++i) p.stage_sc[((size_t)m * 4 + (s - 1)) * kAdjStageVals + i] = sc[i];
+      if (threadIdx.x < kAdjStageVals) {
+        const int i = threadIdx.x;
+        const double mu = S.str[0];
+        const double v = i < 6 ? mu * S.tot[i] : i == 6 ? S.str[1] : i == 7 ? x_s : i == 8 ? mu : 0.0;
+        p.glob[i] = v;
+        if (store_seg) p.stage_sc[((size_t)m * 4 + (s - 1)) * kAdjStageVals + i] = v;
       }
       release(p, S);
     }
@@ -235,18 +291,19 @@ __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int
 // Objective J and the adjoint of the final state; zero the parameter accumulators.
 __device__ bool objective(const AdjParams& p, AdjShared& S) {
   const uint64_t n = p.n_beams;
-  const uint32_t b0 = (uint32_t)(n * blockIdx.x / gridDim.x), b1 = (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
+  const AdjShare sh(p);                  // the beams of forward_steps: each thread reads what it wrote
   double acc[1] = {0.0};
-  for (uint32_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-    const BeamC c = beam_consts(p, b);
+  for (uint32_t b = sh.first; b < sh.end; b += 32) {
+    const uint32_t jj = fast_div(b, p.ic.div_magic), k = b - jj * p.n_energy;
+    const double ow = jj >= p.n_angle ? 0.0 : p.du[jj] * p.objw[k];      // objective weight: nu beams only
     const double sz = p.y[2 * n + b];
-    acc[0] += c.ow * 0.5 * (1.0 + sz);
-    const double a[3] = {0.0, 0.0, 0.5 * c.ow};
+    acc[0] += ow * 0.5 * (1.0 + sz);
+    const double a[3] = {0.0, 0.0, 0.5 * ow};
     st3(p.a, n, b, a);
     p.gw[b] = 0.0;
     p.gth[b] = 0.0;
   }
-  const int res = grid_reduce<1>(p, S, acc);
+  const int res = grid_reduce<1>(p, S, acc, [] {});
   if (res == kBarAbort) return false;
   if (res == kBarLast) {
     if (threadIdx.x == 0) p.glob[kGlobJ] = S.tot[0];
@@ -258,11 +315,9 @@ __device__ bool objective(const AdjParams& p, AdjShared& S) {
 // Backward over the segment's steps [seg_first, seg_first + seg_count), stage by stage.
 __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
   const uint64_t n = p.n_beams;
-  const uint32_t b0 = (uint32_t)(n * blockIdx.x / gridDim.x), b1 = (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
+  const AdjShare sh(p);
   const int count = p.seg_count;
   const int P = 4 * count;
-  const double c2 = -p.ic.B[2], s2 = p.ic.B[0];              // B = (sin 2th, 0, -cos 2th)
-  const double dB[3] = {2.0 * c2, 0.0, 2.0 * s2};             // dB / dtheta_v
   const double h = p.h;
   for (int pp = 0; pp <= P; ++pp) {
     const int sp = pp > 0 ? 4 - ((pp - 1) & 3) : 0;         // stage finished (its moments reduced)
@@ -276,16 +331,51 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
         S.scf[threadIdx.x] = __ldcg(&p.stage_sc[((size_t)mp * 4 + (sp - 1)) * kAdjStageVals + threadIdx.x]);
       if (threadIdx.x < 6) S.gl[threadIdx.x] = __ldcg(&p.glob[kGlobAdj + threadIdx.x]);
     }
-    // geometry sets: 0 the finished stage, 1..4 the stages of the formed stage's step
-    uint32_t row0;
-    const bool tab = fill_geo(p, S, b0, b1, [&](int set) {
-      if (set == 0) return pp > 0 ? __ldcg(&p.stage_sc[((size_t)mp * 4 + (sp - 1)) * kAdjStageVals + 7]) : 0.0;
-      return pp < P ? __ldcg(&p.stage_sc[((size_t)m * 4 + (set - 1)) * kAdjStageVals + 7]) : 0.0;
-    }, row0);
     __syncthreads();
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (uint32_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-      const BeamC c = beam_consts(p, b);
+    // rows: slots 1..4 hold the stages of the formed stage's step, filled once a step (s = 4); slot 0
+    // keeps the step before's stage 1 for the pass that finishes it
+    const bool step_start = s == 4;
+    const int fslot = sp == 1 ? 0 : sp;
+    if (sh.tab) {
+      if (step_start) {
+        for (uint32_t t = threadIdx.x; t < 4 * sh.rows; t += blockDim.x) {
+          const uint32_t st = 1 + t / sh.rows, r = t % sh.rows;
+          if (st == 1 && pp > 0) {
+            S.row[0][r] = S.row[1][r];
+            S.back[r] = row_back(p, sh.row0 + r, S.row[0][r], S.gl);
+          }
+          if (pp < P) {
+            row_geometry(p, sh.row0 + r, S.scs[st - 1][7], S.row[st][r]);
+            row_coupling(S.scs[st - 1], S.row[st][r]);
+          }
+        }
+      } else {
+        for (uint32_t r = threadIdx.x; r < sh.rows; r += blockDim.x)
+          S.back[r] = row_back(p, sh.row0 + r, S.row[fslot][r], S.gl);
+      }
+    }
+    __syncthreads();
+    auto stage_row = [&](int slot, const double* sc, uint32_t jj) {
+      if (sh.tab) return S.row[slot][jj - sh.row0];
+      AdjRow r;
+      row_geometry(p, jj, sc[7], r);
+      row_coupling(sc, r);
+      return r;
+    };
+    double acc[6] = {0, 0, 0, 0, 0, 0}, rs[3] = {0, 0, 0};
+    auto flush = [&](uint32_t jj) {
+      const AdjRow r = stage_row(s, S.scs[s - 1], jj);
+      for (int i = 0; i < 3; ++i) {
+        acc[i] = fma(r.q, rs[i], acc[i]);
+        acc[3 + i] = fma(r.t1, rs[i], acc[3 + i]);
+        rs[i] = 0.0;
+      }
+    };
+    uint32_t cur = 0xffffffffu;
+    for (uint32_t b = sh.first; b < sh.end; b += 32) {
+      const uint32_t jj = fast_div(b, p.ic.div_magic), k = b - jj * p.n_energy;
+      const bool bar = jj >= p.n_angle;
+      const double om = p.omega[k], eo = bar ? -om : om;
       double a[3];
       ld3(p.a, n, b, a);
       double vnext[3] = {0, 0, 0};
@@ -294,16 +384,16 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
         if (sp == 1) ld3(p.seg + (size_t)mp * 3 * n, n, b, ys);
         else ld3(p.ystage + (size_t)(sp - 2) * 3 * n, n, b, ys);
         ld3(p.v, n, b, v);
-        const Geo g = tab ? S.geo[0][c.jj - row0] : geometry(c.u, S.scf[7]);
-        kvec(S.scf, g, c.eo, p.ic.B, K);
-        double br[3];
-        for (int i = 0; i < 3; ++i) br[i] = g.t1 * S.gl[i] + S.gl[3 + i];
+        const AdjRow row = stage_row(fslot, S.scf, jj);
+        const AdjBack bk = sh.tab ? S.back[jj - sh.row0] : row_back(p, jj, row, S.gl);
+        kvec(row, eo, K);
         cross(v, K, t);
+        const double g = p.g[(bar ? p.n_energy : 0u) + k];
         double sb[3];
-        for (int i = 0; i < 3; ++i) sb[i] = t[i] + c.w * br[i];
-        p.gw[b] += dot(ys, br);
+        for (int i = 0; i < 3; ++i) sb[i] = fma(g, bk.brd[i], t[i]);
+        p.gw[b] += dot(ys, bk.brd);
         cross(ys, v, pv);
-        p.gth[b] += g.q * c.eo * dot(pv, dB);
+        p.gth[b] = fma(eo, fma(pv[0], bk.qd0, pv[2] * bk.qd2), p.gth[b]);
         double yb[3];
         if (sp == 4) {
           for (int i = 0; i < 3; ++i) { yb[i] = sb[i]; vnext[i] = (h / 3.0) * a[i] + h * sb[i]; }
@@ -324,15 +414,14 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
         double ys[3], v[3];
         if (s == 4) {
           // stage states of step m from its start state and stored stage constants
-          double y[3], k[3], K[3], yy[3];
+          double y[3], kk[3], K[3], yy[3];
           ld3(p.seg + (size_t)m * 3 * n, n, b, y);
           for (int i = 0; i < 3; ++i) yy[i] = y[i];
           for (int st = 1; st <= 3; ++st) {
-            const Geo g = tab ? S.geo[st][c.jj - row0] : geometry(c.u, S.scs[st - 1][7]);
-            kvec(S.scs[st - 1], g, c.eo, p.ic.B, K);
-            cross(K, yy, k);
+            kvec(stage_row(st, S.scs[st - 1], jj), eo, K);
+            cross(K, yy, kk);
             const double as = rk_a(st + 1) * h;
-            for (int i = 0; i < 3; ++i) yy[i] = y[i] + as * k[i];
+            for (int i = 0; i < 3; ++i) yy[i] = y[i] + as * kk[i];
             st3(p.ystage + (size_t)(st - 1) * 3 * n, n, b, yy);
           }
           for (int i = 0; i < 3; ++i) { ys[i] = yy[i]; v[i] = (h / 6.0) * a[i]; }
@@ -342,30 +431,28 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
           for (int i = 0; i < 3; ++i) v[i] = vnext[i];
         }
         st3(p.v, n, b, v);
+        if (jj != cur) {
+          if (cur != 0xffffffffu) flush(cur);
+          cur = jj;
+        }
         double pv[3];
         cross(ys, v, pv);
-        const Geo g = tab ? S.geo[s][c.jj - row0] : geometry(c.u, S.scs[s - 1][7]);
-        for (int i = 0; i < 3; ++i) {
-          acc[i] += g.q * pv[i];
-          acc[3 + i] += g.t1 * pv[i];
-        }
+        for (int i = 0; i < 3; ++i) rs[i] += pv[i];
       }
     }
     if (pp == P) break;
-    const int res = grid_reduce<6>(p, S, acc);
+    if (cur != 0xffffffffu) flush(cur);
+    const int res = grid_reduce<6>(p, S, acc, [] {});
     if (res == kBarAbort) return false;
     if (res == kBarLast) {
-      if (threadIdx.x == 0) {
-        const double mu = S.scs[s - 1][8];
-        for (int i = 0; i < 6; ++i) p.glob[kGlobAdj + i] = mu * S.tot[i];
-      }
+      if (threadIdx.x < 6) p.glob[kGlobAdj + threadIdx.x] = S.scs[s - 1][8] * S.tot[threadIdx.x];
       release(p, S);
     }
   }
   return true;
 }
 
-__global__ void __launch_bounds__(kAdjBlock, 1) adjoint_kernel(AdjParams p) {
+__global__ void __launch_bounds__(kAdjBlock, 1) adjoint_kernel(const __grid_constant__ AdjParams p) {
   __shared__ AdjShared S;
   if (threadIdx.x == 0) S.gen = ld_acquire(&p.bar->gen);
   __syncthreads();
@@ -376,9 +463,9 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_kernel(AdjParams p) {
   }
   // backward over one segment: re-run it forward from its checkpoint, then reverse it
   const uint64_t n = p.n_beams;
-  const uint32_t b0 = (uint32_t)(n * blockIdx.x / gridDim.x), b1 = (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
+  const AdjShare sh(p);                  // the beams of forward_steps: each thread reads what it wrote
   const double* ck = p.ck + (size_t)(p.seg_first / p.ck_every) * 3 * n;
-  for (uint32_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
+  for (uint32_t b = sh.first; b < sh.end; b += 32) {
     double y[3];
     ld3(ck, n, b, y);
     st3(p.y, n, b, y);
@@ -397,7 +484,7 @@ __global__ void adjoint_sums_kernel(AdjParams p, double* pee_sum, double* gw_sum
   for (uint32_t j = 0; j < p.n_angle; ++j) {
     const uint32_t b = (sig * p.n_angle + j) * p.n_energy + k;
     if (!sig) ps += p.du[j] * (0.5 * (1.0 + p.y[2 * n + b]) - J);
-    gs += p.du[j] * p.gw[b];
+    gs += p.gw[b];
     ts += p.gth[b];
   }
   if (!sig) pee_sum[k] = ps;

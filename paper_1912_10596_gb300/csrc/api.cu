@@ -1659,7 +1659,8 @@ int xflat_adjoint(xflat_t h, double r0_km, double r1_km, uint32_t n_steps, uint3
   for (uint32_t k = 0; k < ne; ++k) objw[k] = I.N[k] / SW;
   int G = adjoint_blocks_per_sm() * h->sm_count;
   if (G < 1) return fail(h, XFLAT_ERR_CUDA, "adjoint kernel does not fit on an SM");
-  G = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)G, ((uint64_t)n + kAdjBlock - 1) / kAdjBlock));
+  // two warps' beams a block at least: a pass of a small problem lasts as long as its busiest SM
+  G = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)G, ((uint64_t)n + 63) / 64));
   // device buffers
   const size_t n3 = 3ull * n;
   const size_t words = ne + 2ull * ne + 2 * na + ne                // omega, g, u, du, objw
