@@ -35,7 +35,7 @@ L2_BYTES = 129 * 1024 * 1024
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
 STEP_TRAFFIC = {"bytes_per_launch": 51251200 + 173570560, "steps_per_launch": 8,
-                "code_sha256": "f8f7c6198b00e64bbe60cdc671a5c71a19647465bee8ab6dce02a883b0b44d34"}
+                "code_sha256": "d401da69cb370a762beb4fc6dd5ded6fa9613eb8c3d3553285bcf821604e7210"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a

@@ -1503,6 +1503,8 @@ struct BlockShared {
   int next_piece;                      // dynamic scheduling: the piece this block processes next
   int keep;                            // single-piece block: launch-invariant set-up already loaded
   unsigned int gen_seen;               // barrier generation this block arrived in
+  unsigned int expected;               // arrivals a pass barrier waits for
+  unsigned long long pass_next;        // pass_barrier's count
 };
 
 // Table view: row (stage s, combined angle index tj) holds Phys::KT values.
@@ -2741,6 +2743,25 @@ __device__ __forceinline__ bool pass_and_sync(const KParams& p, BlockShared<Real
   if (p.trace && threadIdx.x == 0) t0 = globaltimer_ns();
   run_pass<Phys, Tab, Real, kCF, kPass, kKind>(p, bs, dyn_smem);
   if (p.trace && threadIdx.x == 0) t1 = globaltimer_ns();
+  if constexpr (!kFinal) {
+    // stage pass: every block derives the new stage's constants from the accumulators in its next
+    // set-up (run_pass), so the barrier has no serial section (with dynamic scheduling its last block
+    // resets the piece counter, below)
+    if (!p.dyn_sched) {
+      if (!pass_barrier(p.bar, gridDim.x, bs.expected, p.timeout_ns, p.status, &bs.flag, &bs.pass_next)) return false;
+      if (p.trace && threadIdx.x == 0) {
+        const int idx = bs.pass_idx++;
+        if (idx < p.trace_passes) {
+          unsigned long long* t = p.trace + ((size_t)idx * gridDim.x + blockIdx.x) * 4;
+          t[0] = t0;
+          t[1] = t1;
+          t[2] = globaltimer_ns();
+          t[3] = 0ull;
+        }
+      }
+      return true;
+    }
+  }
   const int res = barrier_arrive(p.bar, gridDim.x, p.timeout_ns, p.status, &bs.flag, &bs.gen_seen);
   if ((res & 0xf) == kBarAbort) return false;
   if (p.trace && threadIdx.x == 0) {
@@ -2756,9 +2777,7 @@ __device__ __forceinline__ bool pass_and_sync(const KParams& p, BlockShared<Real
   if ((res & 0xf) == kBarLast && p.dyn_sched && threadIdx.x == 0)
     p.bar->chunk[((bs.gen_seen >> 1) + 1u) & 1u] = 0u;   // the next pass's piece counter (released below)
   if ((res & 0xf) == kBarLast && !kFinal) {
-    // stage pass: every block derives the new stage's constants from the accumulators in its next
-    // set-up (run_pass), so the barrier opens at once (a non-finite partial is reported by the
-    // final pass's serial update)
+    // the barrier opens at once (a non-finite partial is reported by the final pass's serial update)
     if (threadIdx.x == 0) bs.flag = 0;
     barrier_release(p.bar, 0, &bs.gen_seen);
     if (p.trace && threadIdx.x == 0 && bs.pass_idx - 1 < p.trace_passes)
@@ -2823,6 +2842,8 @@ __global__ void __launch_bounds__(kThreads, kMinB) step_kernel(const __grid_cons
     bs.pass_idx = 0;
     bs.keep = 0;
     bs.gen_seen = ld_acquire(&p.bar->gen);        // later barriers track the generation locally
+    bs.expected = gridDim.x + p.bar->extra;
+    bs.pass_next = pass_barrier_base(p.bar, gridDim.x);
   }
   if (p.shard_mode == kShardPass) {
     if (p.shard_pass < 0) run_pass<Phys, Tab, Real, kCF, 0, kInitPass>(p, bs, dyn_smem);
