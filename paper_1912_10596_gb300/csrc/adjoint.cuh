@@ -12,8 +12,7 @@ constexpr int kAdjStageVals = 10;   // per stage: mu D (3), mu J1 (3), lambda, R
 constexpr int kAdjPartStride = 8;   // doubles per block partial
 
 enum AdjMode : int { kAdjForward = 0, kAdjBackward = 1 };
-// broadcast slots: [0, kAdjStageVals) stage constants, then the adjoint moments, then J
-constexpr int kGlobAdj = 16, kGlobJ = 24, kGlobWords = 32;
+constexpr int kGlobJ = 0, kGlobWords = 8;     // results: J
 
 struct AdjParams {
   // problem (instance 0 of a handle)
@@ -41,8 +40,8 @@ struct AdjParams {
   double* v;                            // cotangent of the current stage derivative
   double* gw;                           // [n] du_j dJ/dw_b (w_b = du_j g_{sigma,k})
   double* gth;                          // [n] dJ/dtheta_v per beam
-  double* part;                         // [grid][kAdjPartStride] block partials
-  double* glob;                         // [kGlobWords] broadcast values
+  double* part;                         // [2][grid][kAdjPartStride] block partials
+  double* glob;                         // [kGlobWords] results
   Barrier* bar;
   unsigned long long timeout_ns;
   int* status;

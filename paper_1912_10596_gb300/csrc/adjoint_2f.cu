@@ -20,12 +20,12 @@
 // everything that the beams of an angle row share is tabulated once a step and stage (AdjRow, AdjBack: an
 // assembled K is two FMAs), moments are summed within rows, reductions spread over the lanes, and the
 // next stage's strengths are computed beside the sum over blocks.  200 E x 400 u, 128 steps, K = 64:
-// 43.1 ms with per-beam assembly and five geometries a pass, 32.1 ms so.
+// 43.1 ms with per-beam assembly and five geometries a pass, 32.1 ms so (30.0 with grid_reduce as it is).
 //
 // Memory: the forward launch stores the state every K steps (checkpoints); each backward launch
 // re-runs one segment of K steps forward from its checkpoint, storing every step's start state and
 // stage constants, then runs the segment's steps backwards.  Every pass over the beams ends in a
-// device-wide barrier whose last block sums the block partials in block order (deterministic).
+// device-wide barrier, after which every block sums the block partials in block order (deterministic).
 #include "adjoint.cuh"
 #include "step_kernel.cuh"
 
@@ -51,7 +51,8 @@ struct AdjShared {
   double scs[4][kAdjStageVals];         // constants of the formed stage's step (backward: all 4)
   double gl[8];                         // broadcast adjoint moments of the finished stage
   int flag;
-  unsigned int gen;
+  unsigned int reduces;                 // grid_reduce calls of this launch (the partials' buffer)
+  unsigned long long pass_next;         // pass_barrier's count
 };
 
 __device__ __forceinline__ void row_geometry(const AdjParams& p, uint32_t jj, double x, AdjRow& r) {
@@ -132,11 +133,16 @@ __device__ __forceinline__ double stage_radius(const AdjParams& p, int n, int s)
   return (p.r0 + (double)n * p.h) + rk_c(s) * p.h;
 }
 
-// Block partials -> grid barrier -> the last block sums them in block order into S.tot, while one of its
-// idle warps runs `beside` (work that does not need the sums).
+// Block partials -> grid barrier -> every block sums them in block order into S.tot (the same bits
+// everywhere), while one of its idle warps runs `beside` (work that does not need the sums): what follows
+// from the totals needs no serial section and no second hop through memory.  The partials alternate
+// between two buffers: a block can be at most one reduction ahead of another.  Returns false on a timeout
+// or an abort.  (One last block summing and broadcasting: 200 E x 400 u, 128 steps, 32.1 ms; 30.0 ms so;
+// 64 E x 32 u, 64 steps, 7.3 and 6.2 ms.)
 template <int NV, class Beside>
-__device__ int grid_reduce(const AdjParams& p, AdjShared& S, double (&v)[NV], Beside beside) {
+__device__ bool grid_reduce(const AdjParams& p, AdjShared& S, double (&v)[NV], Beside beside) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  double* part = p.part + (size_t)(S.reduces & 1u) * gridDim.x * kAdjPartStride;
   int idx = 0, left = NV;
   bool valid = true;
   const double s = reduce_scatter<NV, 16, double>(v, lane, idx, left, valid);
@@ -147,27 +153,21 @@ __device__ int grid_reduce(const AdjParams& p, AdjShared& S, double (&v)[NV], Be
     double x = w < nw && c < NV ? S.scratch[w * NV + c] : 0.0;
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (w == 0 && c < NV) p.part[(size_t)blockIdx.x * kAdjPartStride + c] = x;
+    if (w == 0 && c < NV) part[(size_t)blockIdx.x * kAdjPartStride + c] = x;
   }
-  const int res = barrier_arrive(p.bar, gridDim.x, p.timeout_ns, p.status, &S.flag, &S.gen) & 0xf;
-  if (res == kBarLast) {
-    if (warp < NV) {
-      double s = 0.0;
-      for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(&p.part[(size_t)b * kAdjPartStride + warp]);
+  if (!pass_barrier(p.bar, gridDim.x, gridDim.x, p.timeout_ns, p.status, &S.flag, &S.pass_next)) return false;
+  if (threadIdx.x == 0) S.reduces++;
+  if (warp < NV) {
+    double s = 0.0;
+    for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(&part[(size_t)b * kAdjPartStride + warp]);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) S.tot[warp] = s;
-    } else if (warp == NV && lane == 0) {
-      beside();
-    }
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) S.tot[warp] = s;
+  } else if (warp == NV && lane == 0) {
+    beside();
   }
-  return res;
-}
-
-__device__ __forceinline__ void release(const AdjParams& p, AdjShared& S) {
-  __threadfence();
-  barrier_release(p.bar, 0, &S.gen);
+  __syncthreads();
+  return true;
 }
 
 // Forward RK4 over steps [n_first, n_first + count) from p.y.  store_seg: each step's start state
@@ -189,8 +189,6 @@ __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int
       const double r = stage_radius(p, nstep, s);
       x_s = p.ic.R2 / (r * r);
     }
-    if (pp > 0 && threadIdx.x < kAdjStageVals) S.scf[threadIdx.x] = __ldcg(&p.glob[threadIdx.x]);
-    __syncthreads();
     // the formed stage's geometry; the finished stage's, tabulated in the pass before, gets its couplings
     if (sh.tab) {
       for (uint32_t t = threadIdx.x; t < 2 * sh.rows; t += blockDim.x) {
@@ -272,20 +270,18 @@ __device__ bool forward_steps(const AdjParams& p, AdjShared& S, int n_first, int
     }
     if (pp == P) break;
     if (cur != 0xffffffffu) flush(cur);
-    const int res = grid_reduce<6>(p, S, acc, [&] { strengths(p.ic, stage_radius(p, nstep, s), S.str[0], S.str[1]); });
-    if (res == kBarAbort) return false;
-    if (res == kBarLast) {
-      if (threadIdx.x < kAdjStageVals) {
-        const int i = threadIdx.x;
-        const double mu = S.str[0];
-        const double v = i < 6 ? mu * S.tot[i] : i == 6 ? S.str[1] : i == 7 ? x_s : i == 8 ? mu : 0.0;
-        p.glob[i] = v;
-        if (store_seg) p.stage_sc[((size_t)m * 4 + (s - 1)) * kAdjStageVals + i] = v;
-      }
-      release(p, S);
+    if (!grid_reduce<6>(p, S, acc, [&] { strengths(p.ic, stage_radius(p, nstep, s), S.str[0], S.str[1]); })) return false;
+    if (threadIdx.x < kAdjStageVals) {
+      const int i = threadIdx.x;
+      const double mu = S.str[0];
+      const double v = i < 6 ? mu * S.tot[i] : i == 6 ? S.str[1] : i == 7 ? x_s : i == 8 ? mu : 0.0;
+      S.scf[i] = v;
+      if (store_seg && blockIdx.x == 0) p.stage_sc[((size_t)m * 4 + (s - 1)) * kAdjStageVals + i] = v;
     }
+    __syncthreads();
   }
-  return true;
+  // block 0's last stage constants, for the backward sweep of every block
+  return !store_seg || pass_barrier(p.bar, gridDim.x, gridDim.x, p.timeout_ns, p.status, &S.flag, &S.pass_next);
 }
 
 // Objective J and the adjoint of the final state; zero the parameter accumulators.
@@ -303,12 +299,8 @@ __device__ bool objective(const AdjParams& p, AdjShared& S) {
     p.gw[b] = 0.0;
     p.gth[b] = 0.0;
   }
-  const int res = grid_reduce<1>(p, S, acc, [] {});
-  if (res == kBarAbort) return false;
-  if (res == kBarLast) {
-    if (threadIdx.x == 0) p.glob[kGlobJ] = S.tot[0];
-    release(p, S);
-  }
+  if (!grid_reduce<1>(p, S, acc, [] {})) return false;
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.glob[kGlobJ] = S.tot[0];
   return true;
 }
 
@@ -329,7 +321,6 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
     if (pp > 0) {
       if (threadIdx.x < kAdjStageVals)
         S.scf[threadIdx.x] = __ldcg(&p.stage_sc[((size_t)mp * 4 + (sp - 1)) * kAdjStageVals + threadIdx.x]);
-      if (threadIdx.x < 6) S.gl[threadIdx.x] = __ldcg(&p.glob[kGlobAdj + threadIdx.x]);
     }
     __syncthreads();
     // rows: slots 1..4 hold the stages of the formed stage's step, filled once a step (s = 4); slot 0
@@ -442,19 +433,19 @@ __device__ bool backward_steps(const AdjParams& p, AdjShared& S) {
     }
     if (pp == P) break;
     if (cur != 0xffffffffu) flush(cur);
-    const int res = grid_reduce<6>(p, S, acc, [] {});
-    if (res == kBarAbort) return false;
-    if (res == kBarLast) {
-      if (threadIdx.x < 6) p.glob[kGlobAdj + threadIdx.x] = S.scs[s - 1][8] * S.tot[threadIdx.x];
-      release(p, S);
-    }
+    if (!grid_reduce<6>(p, S, acc, [] {})) return false;
+    if (threadIdx.x < 6) S.gl[threadIdx.x] = S.scs[s - 1][8] * S.tot[threadIdx.x];
+    __syncthreads();
   }
   return true;
 }
 
 __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_kernel(const __grid_constant__ AdjParams p) {
   __shared__ AdjShared S;
-  if (threadIdx.x == 0) S.gen = ld_acquire(&p.bar->gen);
+  if (threadIdx.x == 0) {
+    S.pass_next = pass_barrier_base(p.bar, gridDim.x);
+    S.reduces = 0;
+  }
   __syncthreads();
   if (p.mode == kAdjForward) {
     if (!forward_steps(p, S, 0, p.n_steps, false, true, true)) return;

@@ -1667,7 +1667,7 @@ int xflat_adjoint(xflat_t h, double r0_km, double r1_km, uint32_t n_steps, uint3
                      + 3 * n3 + (size_t)n_ck * n3 + (size_t)K * n3 // y, ksum, klast, ck, seg
                      + (size_t)K * 4 * kAdjStageVals + 3 * n3      // stage_sc, ystage
                      + 3 * n3 + 2ull * n                           // a, ybar, v, gw, gth
-                     + (size_t)G * kAdjPartStride + kGlobWords     // part, glob
+                     + 2 * (size_t)G * kAdjPartStride + kGlobWords // part, glob
                      + 5ull * ne;                                  // pee_sum, gw_sum, gth_sum
   double* base = nullptr;
   Barrier* bar = nullptr;
@@ -1703,7 +1703,7 @@ int xflat_adjoint(xflat_t h, double r0_km, double r1_km, uint32_t n_steps, uint3
   p.ystage = take(3 * n3);
   p.a = take(n3); p.ybar = take(n3); p.v = take(n3);
   p.gw = take(n); p.gth = take(n);
-  p.part = take((size_t)G * kAdjPartStride);
+  p.part = take(2 * (size_t)G * kAdjPartStride);
   p.glob = take(kGlobWords);
   double* d_pee = take(ne);
   double* d_gws = take(2ull * ne);
