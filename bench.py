@@ -34,14 +34,14 @@ L2_BYTES = 129 * 1024 * 1024
 # DRAM traffic of one timed launch of the step kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
-STEP_TRAFFIC = {"bytes_per_launch": 51251200 + 173570560, "steps_per_launch": 8,
-                "code_sha256": "d401da69cb370a762beb4fc6dd5ded6fa9613eb8c3d3553285bcf821604e7210"}
+STEP_TRAFFIC = {"bytes_per_launch": 51172864 + 173309184, "steps_per_launch": 8,
+                "code_sha256": "c9a5142bdfd810d0261fc61ba9066188133ff09a4b2f480666a855d45c2d1d6a"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a
 # longer launch issues a little less): with the step time and the sampled SM clock it gives the
 # kernel's place under its instruction-issue ceiling (4 warp instructions per clock per SM).
-STEP_INSTRUCTIONS = {"warp_inst_per_step": 112215206, "code_sha256": STEP_TRAFFIC["code_sha256"]}
+STEP_INSTRUCTIONS = {"warp_inst_per_step": 112196243, "code_sha256": STEP_TRAFFIC["code_sha256"]}
 
 
 def issue_roofline(ms_per_step, sm_mhz, n_sm):

@@ -29,7 +29,7 @@
 //
 // Reduction.  FP64 path: each thread accumulates its beams' contributions in double, each block
 // reduces them with a fixed shuffle/shared-memory tree in double and adds its partial to the
-// instance accumulator as a 128-bit fixed-point integer (exact to 2^-64).  Mixed path: each beam's
+// instance accumulator as two integers in units of 2^-12 and 2^-64 (exact to 2^-64, no carry).  Mixed path: each beam's
 // contribution (an FP32 weight times an FP32 state) is summed per thread without rounding loss as an
 // unevaluated (hi, lo) pair (MomAcc<float>); at the end of the pass the pair goes to integers in units
 // of the instance's 2^-S (the FP32 weights carry that power-of-two scale), and the sums over lanes,
@@ -401,6 +401,10 @@ struct Phys2 {
   __device__ static inline Real tnorm2(const Real (&y)[3]) {
     return Real(0.5) * (y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
   }
+  // The larger norm of two states given by their components' leading 21 bits, or a little less
+  __device__ static inline Real norm_floor(const Real (&a)[3], const Real (&b)[3]) {
+    return sqrt(fmax(tnorm2(a), tnorm2(b)));
+  }
   // Frobenius norm of the traceless matrix (e.sigma)/2, scaled so it cannot overflow; +inf if not finite
   __device__ static inline Real enorm(const Real (&e)[3]) {
     const Real m = fmax(fabs(e[0]), fmax(fabs(e[1]), fabs(e[2])));
@@ -531,6 +535,12 @@ struct Phys3 {
     const Real d0 = y[0] - t, d1 = y[1] - t, d2 = y[2] - t;
     return d0 * d0 + d1 * d1 + d2 * d2 +
            2 * (y[3] * y[3] + y[4] * y[4] + y[5] * y[5] + y[6] * y[6] + y[7] * y[7] + y[8] * y[8]);
+  }
+  // The larger norm of two states given by their components' leading 21 bits, or a little less: taking
+  // the trace off amplifies the truncation (2^-20 of the diagonal) where a state is nearly 1/3
+  __device__ static inline Real norm_floor(const Real (&a)[9], const Real (&b)[9]) {
+    const Real d = fabs(a[0]) + fabs(a[1]) + fabs(a[2]) + fabs(b[0]) + fabs(b[1]) + fabs(b[2]);
+    return fmax(sqrt(fmax(tnorm2(a), tnorm2(b))) - Real(4e-6) * d, Real(0));
   }
   // full Frobenius norm of the Hermitian matrix, scaled against overflow; +inf if not finite
   __device__ static inline Real enorm(const Real (&e)[9]) {
@@ -705,6 +715,7 @@ struct Phys2E {
     }
   }
   __device__ static inline Real tnorm2(const Real (&y)[3]) { return Phys2<Real>::tnorm2(y); }
+  __device__ static inline Real norm_floor(const Real (&a)[3], const Real (&b)[3]) { return Phys2<Real>::norm_floor(a, b); }
   __device__ static inline Real enorm(const Real (&e)[3]) { return Phys2<Real>::enorm(e); }
   __device__ static inline void normalise(Real (&y)[3]) { Phys2<Real>::normalise(y); }
   __device__ static inline void purify(Real (&y)[3]) { Phys2<Real>::normalise(y); }
@@ -1699,8 +1710,8 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
     if (Tab::kAdaptive) {
       // split final pass (y holds y5): k_S = f(y5) with the moments of y5, the embedded error, and the
       // squared error ratio (its square root is taken once per block).  Only the largest ratio counts:
-      // an FP32 estimate of it (components by their leading 21 bits, so within 2e-5) passes over every
-      // beam that cannot exceed the largest found so far in the block, so the FP64 norms, square root
+      // an FP32 estimate of it (components by their leading 21 bits; never below the ratio by more than
+      // the 1e-3 it is raised by, norm_floor) passes over every beam that cannot exceed the largest found so far in the block, so the FP64 norms, square root
       // and division -- a fifth of a DP45 step's FP64 work -- are left for a few beams a block.
       Real Kv[Phys::NG], kS[NC], e[NC];
       Phys::K(tv.row(Tab::S, tj), bm, Kv);
@@ -1715,9 +1726,10 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
         of[i] = lead_f32(yo[i]);
       }
       using P32 = typename Phys::template With<float>;
-      const float df = bs.atol_f + bs.rtol_f * sqrtf(fmaxf(P32::tnorm2(of), P32::tnorm2(yf)));
+      const float df = bs.atol_f + bs.rtol_f * P32::norm_floor(of, yf);
       const float rf = __fdividef(P32::tnorm2(ef), df * df);
-      if (!(rf * 1.001f < __int_as_float(*(volatile int*)&bs.emax_f))) {       // also where rf is not a number
+      // also where rf is not a number, and where the squares leave FP32's range
+      if (!(rf * 1.001f < __int_as_float(*(volatile int*)&bs.emax_f)) || !(df < 1.0e18f)) {
         const Real no = Phys::tnorm2(yo), n5 = Phys::tnorm2(y);
         if (!(no <= rbig<Real>())) bad = 1;                     // non-finite input state: fatal
         const Real den = bs.atol + bs.rtol * sqrt(fmax(no, n5));

@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 
 from bulb_inputs import Workload, coherent_unit_states
-from oracle.integrate import evolve_adaptive, evolve_fixed, evolve_lie_adaptive
+from oracle.integrate import dp45_step, evolve_adaptive, evolve_fixed, evolve_lie_adaptive
 from oracle.physics import Bulb
 from parity_util import beams, make_solver
 
@@ -77,3 +77,26 @@ def test_batches_in_static_slices_and_in_pieces(xf, sizes, precision):
         assert diff < (1e-12 if precision == "fp64" else 1e-6), (sizes[i], diff)
         one.close()
     s.close()
+
+
+@pytest.mark.parametrize("delta", [1.0, 1e-5, 1e-6])
+def test_error_maximum_of_nearly_unpolarised_states(xf, delta):
+    """The FP32 estimate that spares most beams the FP64 error norm must not pass over the largest
+    ratio: states delta away from 1/3, whose norms are differences of nearly equal numbers, with a
+    purely relative tolerance.  last_err against the oracle's; the FP64 rounding of the embedded error
+    (1e-15 of a unit state) is below 1e-9 / delta of it, the error being above 1e-6 delta."""
+    h = 1e-3
+    wl = Workload(name="mix", n_flavor=3, n_energy=40, n_angle=90, integrator="dp45", precision="fp64", dm2=(7.5e-5, -2.4e-3),
+                  theta=(0.59, 0.15, 0.785), matter="constant", lambda_const=1e3, rtol=1e-2, atol=0.0, r0=50.0)
+    Y = np.eye(3) / 3 + delta * (state(wl, seed=5) - np.eye(3) / 3)
+    s = make_solver(xf, wl, h0_km=h, h_max_km=h)
+    s.set_rho(beams(Y), wl.r0)
+    Y = s.get_rho().reshape(Y.shape)
+    s.evolve(wl.r0, wl.r0 + h)
+    st = s.stats()
+    s.close()
+    b = Bulb(wl)
+    h = (wl.r0 + h) - wl.r0
+    err = dp45_step(b.rhs, wl.r0, Y, h, b.rhs(wl.r0, Y), wl.atol, wl.rtol)[1]
+    assert (st.accepted, st.rejected) == (1, 0) and err > 1e-4
+    assert abs(st.last_err / err - 1) < 1e-9 / delta
