@@ -58,7 +58,7 @@ enum xflat_precision {
   XFLAT_FP64 = 0,             /* every per-beam operation in IEEE double                         */
   XFLAT_MIXED = 1             /* per-beam precession in float, including each beam's moment
                                  contribution w s; the sum of the contributions over beams is
-                                 FP64-accurate (per-thread TwoSum pairs, then integer sums across
+                                 FP64-accurate (per-thread hi + lo pairs, then integer sums across
                                  threads, warps, blocks and the grid: exact and order-free); the
                                  error norm is the exact maximum of the per-beam error ratios with
                                  its square root and the step-size controller in double; |s|
@@ -394,7 +394,7 @@ int xflat_debug_fail_alloc(uint32_t nth);
  * device memory).  host_out != NULL: synchronise and copy the trace out: for pass i and block b,
  * host_out[(i*grid + b)*4 + 0..3] = %globaltimer (ns) at the pass start, after the block's beams and
  * reduction, after the device-wide barrier let it go, and 1 if the block arrived last (then the
- * third stamp is its arrival).  *grid_out (nullable) receives the number of blocks. */
+ * third stamp is its arrival; stage passes of handles without dynamic pieces have no last block).  *grid_out (nullable) receives the number of blocks. */
 int xflat_debug_trace(xflat_t h, uint32_t n_passes, uint64_t* host_out, uint32_t* grid_out);
 
 #ifdef __cplusplus
