@@ -1862,7 +1862,7 @@ int xflat_shard_partials(xflat_t h, int64_t* words) {
   uint32_t nw = 0;
   xflat_shard_info(h, nullptr, &nw);
   const int nm = (int)(nw - 2) / 2, slot = shard_slot(h);
-  constexpr int kWords = kAccCopies * kNMMax * 2;
+  constexpr int kWords = kAccWordsPerSlot;
   std::vector<unsigned long long> acc(kWords);
   unsigned long long em = 0;
   int nonfin = 0;
@@ -1871,11 +1871,12 @@ int xflat_shard_partials(xflat_t h, int64_t* words) {
   CUDA_TRY(h, cudaMemcpyAsync(&nonfin, h->d_nonfinite, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   for (int c = 0; c < nm; ++c) {
-    unsigned __int128 t = 0;
+    // FP64: the words of fx_add
+    unsigned __int128 t = h->real_size == 4 ? 0 : (unsigned __int128)(__int128)(long long)acc[((size_t)kAccCopies * kNMMax + c) * 2] << 67;
     for (int cp = 0; cp < kAccCopies; ++cp) {
       const unsigned long long* w = acc.data() + ((size_t)cp * kNMMax + c) * 2;
       if (h->real_size == 4) t += (unsigned __int128)(__int128)(long long)w[0];   // one signed word
-      else t += (unsigned __int128)((__int128)(long long)w[1] * (1ll << 52) + (long long)w[0]);   // see fx_add
+      else t += (unsigned __int128)((__int128)(long long)w[1] * (1ll << 30) + (long long)w[0]);
     }
     words[2 * c] = (int64_t)(unsigned long long)t;
     words[2 * c + 1] = (int64_t)(unsigned long long)(t >> 64);
@@ -1893,7 +1894,7 @@ int xflat_shard_set_totals(xflat_t h, const int64_t* words) {
   uint32_t nw = 0;
   xflat_shard_info(h, nullptr, &nw);
   const int nm = (int)(nw - 2) / 2, slot = shard_slot(h);
-  constexpr int kWords = kAccCopies * kNMMax * 2;
+  constexpr int kWords = kAccWordsPerSlot;
   std::vector<unsigned long long> acc(kWords, 0ull);    // the total in copy 0, the other copies 0
   for (int c = 0; c < nm; ++c) {
     const __int128 t = (__int128)(((unsigned __int128)(unsigned long long)words[2 * c + 1] << 64) |
@@ -1901,9 +1902,10 @@ int xflat_shard_set_totals(xflat_t h, const int64_t* words) {
     if (h->real_size == 4) {
       acc[(size_t)c * 2] = (unsigned long long)words[2 * c];
     } else {
-      // the two signed words of fx_add: the total's low 52 bits and the rest
-      acc[(size_t)c * 2] = (unsigned long long)t & ((1ull << 52) - 1);
-      acc[(size_t)c * 2 + 1] = (unsigned long long)(long long)(t >> 52);
+      // the words of fx_add: the total's bits from 67 on, the 37 below them and the low 30
+      acc[((size_t)kAccCopies * kNMMax + c) * 2] = (unsigned long long)(long long)(t >> 67);
+      acc[(size_t)c * 2 + 1] = (unsigned long long)(t >> 30) & ((1ull << 37) - 1);
+      acc[(size_t)c * 2] = (unsigned long long)t & ((1ull << 30) - 1);
     }
     if (h->real_size == 4) {
       // a mixed accumulator is one signed 64-bit word: the total must fit it

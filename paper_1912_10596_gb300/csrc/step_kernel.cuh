@@ -29,7 +29,8 @@
 //
 // Reduction.  FP64 path: each thread accumulates its beams' contributions in double, each block
 // reduces them with a fixed shuffle/shared-memory tree in double and adds its partial to the
-// instance accumulator as two integers in units of 2^-12 and 2^-64 (exact to 2^-64, no carry).  Mixed path: each beam's
+// instance accumulator as integers in units of 2^-34 and 2^-64 (exact to 2^-64, no carry; a third word for
+// partials of 8 and more, up to 2^63).  Mixed path: each beam's
 // contribution (an FP32 weight times an FP32 state) is summed per thread without rounding loss as an
 // unevaluated (hi, lo) pair (MomAcc<float>); at the end of the pass the pair goes to integers in units
 // of the instance's 2^-S (the FP32 weights carry that power-of-two scale), and the sums over lanes,
@@ -802,15 +803,28 @@ __device__ __forceinline__ bool index_ok(const KParams& p, bool ok, int site, lo
 #define XFLAT_INDEX_OK(p, cond, site, v) true
 #endif
 
-// Add x (|x| < 2^51) to a fixed-point accumulator of two signed words, acc2[1] in units of 2^-12 and
-// acc2[0] in units of 2^-64, truncating |x| below 2^-64: x = hi 2^-12 + lo 2^-64 exactly, |lo| < 2^52, so
-// hundreds of blocks cannot overflow a word, no carry passes between them and neither addition waits
-// for the other's result.
-__device__ __forceinline__ void fx_add(unsigned long long* acc2, double x) {
-  const double hi_d = trunc(x * 4096.0);
-  const long long lo = (long long)((x * 4096.0 - hi_d) * 4503599627370496.0);        // exact difference, 2^52
-  atomicAdd(&acc2[0], (unsigned long long)lo);
-  atomicAdd(&acc2[1], (unsigned long long)(long long)hi_d);
+// Add x (|x| < 2^63) to the fixed-point accumulators of component c of a stage slot, truncating |x| below
+// 2^-64.  x = big 2^3 + hi 2^-34 + lo 2^-64 exactly, with |hi| < 2^37 and |lo| < 2^30 in two words of one
+// copy: no carry passes between them, and neither addition waits for the other's result.  A piece makes one
+// addition; an instance has fewer than 2^31 beams in pieces of 124 and more (but for the ends of slices), so
+// fewer than 2^25 pieces, and the sum of all copies of a word stays below 2^62.  big is zero for weights that
+// sum to a few units, as normalised ones do; else it goes to the slot's one word for large partials.  Returns
+// false when the running sum leaves the range.
+__device__ __forceinline__ bool fx_add(unsigned long long* slot, int copy, int c, double x) {
+  unsigned long long* a = slot + ((size_t)copy * kNMMax + c) * 2;
+  bool ok = true;
+  if (fabs(x) >= 8.0) {
+    const double b = trunc(x * 0.125);
+    const long long big = (long long)b;
+    const long long sum = (long long)atomicAdd(slot + ((size_t)kAccCopies * kNMMax + c) * 2, (unsigned long long)big) + big;
+    ok = sum < (1ll << 60) && sum > -(1ll << 60);
+    x = fma(-8.0, b, x);
+  }
+  const double hi_d = trunc(x * 17179869184.0);                                      // 2^34
+  const long long lo = (long long)((x * 17179869184.0 - hi_d) * 1073741824.0);       // exact difference, 2^30
+  atomicAdd(&a[0], (unsigned long long)lo);
+  atomicAdd(&a[1], (unsigned long long)(long long)hi_d);
+  return ok;
 }
 
 template <class Tab>
@@ -885,6 +899,7 @@ __device__ __forceinline__ double acc_component(const unsigned long long* acc_sl
     for (int cp = 0; cp < kAccCopies; ++cp) sum += (long long)__ldcg(acc_slot + ((size_t)cp * kNMMax + c) * 2);
     return (double)sum * unit;                                   // 2^-S of the instance
   } else {
+    const long long big = (long long)__ldcg(acc_slot + ((size_t)kAccCopies * kNMMax + c) * 2);
     long long hi = 0, lo = 0;
 #pragma unroll
     for (int cp = 0; cp < kAccCopies; ++cp) {
@@ -893,7 +908,7 @@ __device__ __forceinline__ double acc_component(const unsigned long long* acc_sl
       lo += (long long)v.x;
       hi += (long long)v.y;
     }
-    const __int128 sum = ((__int128)hi << 52) + lo;                    // units of 2^-64
+    const __int128 sum = ((__int128)big << 67) + ((__int128)hi << 30) + lo;   // units of 2^-64 (fx_add)
     return (double)(long long)(sum >> 64) + (double)(unsigned long long)sum * 5.421010862427522e-20;
   }
 }
@@ -941,13 +956,13 @@ __device__ __forceinline__ T reduce_scatter(T (&v)[N], int lane, int& idx, int& 
 }
 
 // Block sums of the threads' moment partials v (double, or integers of the instance's unit in the
-// mixed kernels) into one copy of the instance's accumulators: reduce-scatter in each warp, one
+// mixed kernels) into one copy of the accumulators of an instance's stage slot: reduce-scatter in each warp, one
 // shared-memory row a warp, a half-warp tree a component over up to 16 warps, and one fixed-point
 // addition a component.  In a fixed order, so the result depends on the block decomposition only.
 // ovf: a thread's partial left the integer range (mixed).  A sum that is not finite or out of range
-// rejects an adaptive trial step (reject) and is fatal for a fixed step.
+// (FP64: 2^63 and more) rejects an adaptive trial step (reject) and is fatal otherwise.
 template <int NM, typename T>
-__device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsigned long long* acc_copy,
+__device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsigned long long* acc_slot, int copy,
                                             unsigned long long* errmax, int* nonfinite, bool reject) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int idx = 0, left = NM;
@@ -966,10 +981,9 @@ __device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsi
     bool ok;
     if constexpr (T(0.5) == T(0)) {
       ok = !any_ovf && x < kFixLimit && x > -kFixLimit;
-      if (ok) atomicAdd(acc_copy + 2 * c, (unsigned long long)x);
+      if (ok) atomicAdd(acc_slot + ((size_t)copy * kNMMax + c) * 2, (unsigned long long)x);
     } else {
-      ok = fabs(x) <= 1.7e308;
-      if (ok) fx_add(acc_copy + 2 * c, x);
+      ok = fabs(x) < 9223372036854775808.0 && fx_add(acc_slot, copy, c, x);
     }
     if (!ok) {
       if (reject) atomicMax(errmax, 0x7ff0000000000000ull);
@@ -981,9 +995,9 @@ __device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsi
 // FP64 kernels share one copy of it over their passes (noinline): inlined, its code was out of the
 // instruction cache at every pass.
 template <int NM>
-__device__ __noinline__ void reduce_moments_shared(double (&v)[NM], double* red, unsigned long long* acc_copy,
+__device__ __noinline__ void reduce_moments_shared(double (&v)[NM], double* red, unsigned long long* acc_slot, int copy,
                                                    unsigned long long* errmax, int* nonfinite, bool reject) {
-  reduce_moments<NM, double>(v, 0, red, acc_copy, errmax, nonfinite, reject);
+  reduce_moments<NM, double>(v, 0, red, acc_slot, copy, errmax, nonfinite, reject);
 }
 
 // The block's largest squared error ratio (FP32; infinity where not finite) and non-finite flag.
@@ -1013,7 +1027,7 @@ __device__ int serial_update(const KParams& p, int slot, bool final_pass, bool i
   for (int i = threadIdx.x; i < p.n_inst; i += blockDim.x) {
     const InstConst& ic = p.ic[i];
     InstDyn& d = p.dyn[i];
-    const unsigned long long* acc = p.acc + (size_t)i * kAccWordsPerInst + (size_t)slot * kAccCopies * kNMMax * 2;
+    const unsigned long long* acc = p.acc + (size_t)i * kAccWordsPerInst + (size_t)slot * kAccWordsPerSlot;
     const bool have_moments = !(final_pass && !Tab::kFinalMoments);
     const bool adaptive_final = final_pass && Tab::kAdaptive && !Tab::kFinalMoments;   // FSAL
     // ---- every load first (no store may sit between them) -------------------------------
@@ -1146,7 +1160,7 @@ __device__ int serial_update(const KParams& p, int slot, bool final_pass, bool i
 // (the fence in serial_geometry publishes the stores before the release).
 template <class Tab>
 __device__ void clear_late_slots(const KParams& p) {
-  constexpr int kWords = kAccCopies * kNMMax * 2;
+  constexpr int kWords = kAccWordsPerSlot;
   constexpr int kLate = Tab::S - Tab::kPasses + 1;
   for (int t = threadIdx.x; t < p.n_inst * kLate * kWords; t += blockDim.x) {
     const int inst = t / (kLate * kWords), rem = t % (kLate * kWords);
@@ -2307,7 +2321,7 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
   const int n_jj = pc.n_jj;
   // constant c of the newest stage
   auto newest_constant = [&](int c) {
-    const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)newest * kAccCopies * kNMMax * 2;
+    const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)newest * kAccWordsPerSlot;
     InstDyn* dw = p.dyn + pc.inst;
     double v = 0.0;
     if (c < Phys::NM) {
@@ -2448,7 +2462,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
   // into a cleared slot until at least one barrier later, and block 0's stores are fenced at its
   // next arrival.
   if (kKind != kInitPass && blockIdx.x == 0) {
-    constexpr int kWords = kAccCopies * kNMMax * 2;
+    constexpr int kWords = kAccWordsPerSlot;
     constexpr int kSlots = kPass == 0 ? 2 : (kPass >= 2 ? 1 : 0);
     for (int t = threadIdx.x; t < p.n_inst * kSlots * kWords; t += blockDim.x) {
       const int inst = t / (kSlots * kWords), rem = t % (kSlots * kWords), q = rem / kWords;
@@ -2684,11 +2698,12 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     }
     // reduce this piece into the instance accumulators: the error maximum (final pass of an
     // adaptive tableau) and the moments (every pass but a final one without moments); a
-    // non-finite moment rejects an adaptive trial step and is fatal for a fixed step
+    // non-finite moment rejects an adaptive trial step and is fatal for a fixed step and for the moments of
+    // the current state (init pass)
     constexpr bool kErrMax = kKind == kFinalPass && Tab::kAdaptive;
-    constexpr bool kRejectOverflow = Tab::kAdaptive;
-    unsigned long long* acc_copy = p.acc + (size_t)pc.inst * kAccWordsPerInst +
-                                   ((size_t)slot * kAccCopies + blockIdx.x % kAccCopies) * kNMMax * 2;
+    constexpr bool kRejectOverflow = Tab::kAdaptive && kKind != kInitPass;
+    unsigned long long* acc_slot = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)slot * kAccWordsPerSlot;
+    const int copy = blockIdx.x % kAccCopies;
     if constexpr (sizeof(Real) == 4) {
       // mixed precision: each thread's (hi, lo) partial sums go to integers of the instance's
       // acc_unit, and every further sum is an integer addition (exact, order-free).  A thread or block
@@ -2716,7 +2731,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
             v[i] = biased_fix<1>(h, acc.lo[i], bias[i / NC], ovf);
           }
         }
-        reduce_moments<NM, long long>(v, ovf, reinterpret_cast<long long*>(red), acc_copy, &p.errmax[pc.inst],
+        reduce_moments<NM, long long>(v, ovf, reinterpret_cast<long long*>(red), acc_slot, copy, &p.errmax[pc.inst],
                                       &p.nonfinite[pc.inst], kRejectOverflow);
       }
     } else {
@@ -2740,7 +2755,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
         double v[NM];                                        // a copy: the accumulators stay in registers
 #pragma unroll
         for (int i = 0; i < NM; ++i) v[i] = acc.v[i];
-        reduce_moments_shared<NM>(v, red, acc_copy, &p.errmax[pc.inst], &p.nonfinite[pc.inst], kRejectOverflow);
+        reduce_moments_shared<NM>(v, red, acc_slot, copy, &p.errmax[pc.inst], &p.nonfinite[pc.inst], kRejectOverflow);
       }
     }
   }
