@@ -596,10 +596,20 @@ static_assert(vec_beams<Phys2<float>, float>() == 2 && vec_beams<Phys2E<float>, 
 // another.  A large piece is a third of a block's vector iterations of a pass, between 16 and 64 of
 // them, a small one a quarter of that, between 4 and 8 (GB300, mixed DP45, 8 steps: 17 instances, 48
 // iterations a block, 5.41 ms in pieces of 64 and 8, 5.23 ms in 16 and 4; 64 instances, 181
-// iterations, 15.8 ms in 64 and 8, 16.8 ms in 32 and 4).  Below kDynMinIters iterations a block's
-// static slice is better (3 instances, 8 iterations: 1.22 ms static, 1.62 to 1.81 ms in pieces; 4
-// instances: 1.84 and 1.74 ms).
-constexpr uint32_t kDynTailPct = 15, kDynMinIters = 10;
+// iterations, 15.8 ms in 64 and 8, 16.8 ms in 32 and 4).
+//
+// Below kDynMinIters iterations a block's static slice is better (3 instances, 8 iterations: 1.22 ms
+// static, 1.62 to 1.81 ms in pieces; 4 instances: 1.84 and 1.74 ms) -- except for the mixed two-flavour
+// bulb kernels where a static block holds kDynMinPieces pieces: its time there is the pieces' set-ups and
+// angle rows, not its beams, and slices of equal beams are far from equal (12 instances of 16 to 400
+// energies, 1.2M beams, up to 11 pieces a block, 6 DP45 steps: 2.79 ms static, 1.38 ms in pieces; 3
+// instances, 500,000 beams, up to 4 pieces: 1.23 and 0.95 ms).  Large pieces are then a block's share of
+// iterations, 8 at least (16 instances, 500,000 beams, up to 4 pieces: 1.09 ms static, 1.24 ms in pieces
+// of 16 iterations, 1.02 ms in pieces of 8).  Over 141 such batches of 2 to 64 instances and 60,000 to
+// 1,200,000 beams no call is slower than with static slices, the mean is 11 % faster.  FP64 and
+// three-flavour blocks are bound by their beams: with 4 to 21 pieces a block static slices are 3 to 12 %
+// faster there.
+constexpr uint32_t kDynTailPct = 15, kDynMinIters = 10, kDynMinPieces = 4;
 void build_dynamic_pieces(xflat_t h) {
   h->pieces.clear();
   h->blk.assign(h->grid + 1, 0);
@@ -623,7 +633,7 @@ void build_dynamic_pieces(xflat_t h) {
   uint64_t total = 0;
   for (auto& I : h->inst) total += I.n_beams;
   const uint32_t iters = (uint32_t)std::min<uint64_t>(total / ((uint64_t)h->grid * beams_per_thread(h) * h->block), 1u << 20);
-  const uint32_t big = std::min(64u, std::max(16u, iters / 3)), small = std::min(8u, big / 4);
+  const uint32_t big = iters < kDynMinIters ? std::max(8u, iters) : std::min(64u, std::max(16u, iters / 3)), small = std::min(8u, big / 4);
   std::vector<uint64_t> split(h->inst.size());
   for (uint32_t i = 0; i < h->inst.size(); ++i) {
     split[i] = ((uint64_t)h->inst[i].n_beams * (100 - kDynTailPct) / 100) / kAlignBeams * kAlignBeams;
@@ -930,9 +940,14 @@ int setup_launch_shape(xflat_t h, const xflat_config& c) {
   }
   h->grid = (int)G;
   // Several instances: blocks take pieces from a counter once each has kDynMinIters vector iterations
-  // of work per pass (see build_dynamic_pieces).
+  // of work per pass, or (mixed two-flavour bulb kernels) kDynMinPieces static pieces (see
+  // build_dynamic_pieces).
   h->dyn_sched = h->inst.size() > 1 && !h->shard && T >= G * beams_per_thread(h) * (uint64_t)h->block * kDynMinIters;
   build_pieces(h, h->grid);
+  if (h->inst.size() > 1 && !h->shard && mixed_2f && !h->dyn_sched) {
+    for (int b = 0; b < h->grid; ++b) h->dyn_sched = h->dyn_sched || h->blk[b + 1] - h->blk[b] >= (int)kDynMinPieces;
+    if (h->dyn_sched) build_pieces(h, h->grid);
+  }
   h->smem = smem_bytes(h->nf, h->real_size, h->max_jj, table_stages(h->integrator), h->block, h->extended);
   if (h->d_pieces) cudaFree(h->d_pieces);
   if (h->d_blk) cudaFree(h->d_blk);
