@@ -1259,9 +1259,9 @@ __device__ __forceinline__ void vstore_at(const KParams& p, int span, Real* ptr,
   if (XFLAT_SPAN_OK(p, span, ptr, N * sizeof(Real), site)) vstore(ptr, v);
 }
 
-// sqrt(x) and 1/sqrt(x) to rounding for x in the normal FP32 range: Newton steps from the hardware's
-// FP32 reciprocal square root, no division (the library's FP64 square root and division are chains of
-// 673 and 429 cycles on GB300)
+// sqrt(x) and 1/sqrt(x) to rounding: Newton steps from the hardware's FP32 reciprocal square root, no
+// division (the library's FP64 square root and division are chains of 673 and 429 cycles on GB300; only an
+// FP64 x beyond the seed's range takes them).  x is at least 1e-10 (FP32: 1e-6), see rotate.
 __device__ __forceinline__ void sqrt_pair(float x, float& t, float& r) {
   r = rsqrtf(x);
   r = fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
@@ -1269,6 +1269,11 @@ __device__ __forceinline__ void sqrt_pair(float x, float& t, float& r) {
   t = fmaf(0.5f * r, fmaf(-t, t, x), t);
 }
 __device__ __forceinline__ void sqrt_pair(double x, double& t, double& r) {
+  if (!(x < 1.0e38)) {
+    t = sqrt(x);
+    r = 1.0 / t;
+    return;
+  }
   r = (double)rsqrtf((float)x);
   r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
   r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
