@@ -809,11 +809,12 @@ __device__ __forceinline__ bool index_ok(const KParams& p, bool ok, int site, lo
 // addition; an instance has fewer than 2^31 beams in pieces of 124 and more (but for the ends of slices), so
 // fewer than 2^25 pieces, and the sum of all copies of a word stays below 2^62.  big is zero for weights that
 // sum to a few units, as normalised ones do; else it goes to the slot's one word for large partials.  Returns
-// false when the running sum leaves the range.
+// false when the running sum leaves the range.  (Ranges are tested on the bits: an FP64 comparison is one
+// more link in a chain of 65-cycle operations at the end of every pass.)
 __device__ __forceinline__ bool fx_add(unsigned long long* slot, int copy, int c, double x) {
   unsigned long long* a = slot + ((size_t)copy * kNMMax + c) * 2;
   bool ok = true;
-  if (fabs(x) >= 8.0) {
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x40200000) {                              // |x| >= 8
     const double b = trunc(x * 0.125);
     const long long big = (long long)b;
     const long long sum = (long long)atomicAdd(slot + ((size_t)kAccCopies * kNMMax + c) * 2, (unsigned long long)big) + big;
@@ -983,7 +984,7 @@ __device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsi
       ok = !any_ovf && x < kFixLimit && x > -kFixLimit;
       if (ok) atomicAdd(acc_slot + ((size_t)copy * kNMMax + c) * 2, (unsigned long long)x);
     } else {
-      ok = fabs(x) < 9223372036854775808.0 && fx_add(acc_slot, copy, c, x);
+      ok = (__double2hiint(x) & 0x7fffffff) < 0x43e00000 && fx_add(acc_slot, copy, c, x);     // |x| < 2^63
     }
     if (!ok) {
       if (reject) atomicMax(errmax, 0x7ff0000000000000ull);
