@@ -803,29 +803,33 @@ __device__ __forceinline__ bool index_ok(const KParams& p, bool ok, int site, lo
 #define XFLAT_INDEX_OK(p, cond, site, v) true
 #endif
 
-// Add x (|x| < 2^63) to the fixed-point accumulators of component c of a stage slot, truncating |x| below
-// 2^-64.  x = big 2^3 + hi 2^-34 + lo 2^-64 exactly, with |hi| < 2^37 and |lo| < 2^30 in two words of one
-// copy: no carry passes between them, and neither addition waits for the other's result.  A piece makes one
+// Add x to the fixed-point accumulators of component c of a stage slot, truncating |x| below 2^-64.
+// x = big 2^3 + hi 2^-34 + lo 2^-64 exactly, with |hi| < 2^37 and |lo| < 2^30 in two words of one copy: no
+// carry passes between them, and neither addition waits for the other's result.  A piece makes one
 // addition; an instance has fewer than 2^31 beams in pieces of 124 and more (but for the ends of slices), so
-// fewer than 2^25 pieces, and the sum of all copies of a word stays below 2^62.  big is zero for weights that
-// sum to a few units, as normalised ones do; else it goes to the slot's one word for large partials.  Returns
-// false when the running sum leaves the range.  (Ranges are tested on the bits: an FP64 comparison is one
-// more link in a chain of 65-cycle operations at the end of every pass.)
-__device__ __forceinline__ bool fx_add(unsigned long long* slot, int copy, int c, double x) {
-  unsigned long long* a = slot + ((size_t)copy * kNMMax + c) * 2;
-  bool ok = true;
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40200000) {                              // |x| >= 8
-    const double b = trunc(x * 0.125);
-    const long long big = (long long)b;
-    const long long sum = (long long)atomicAdd(slot + ((size_t)kAccCopies * kNMMax + c) * 2, (unsigned long long)big) + big;
-    ok = sum < (1ll << 60) && sum > -(1ll << 60);
-    x = fma(-8.0, b, x);
-  }
+// fewer than 2^25 pieces, and the sum of all copies of a word stays below 2^62.  big is zero for weights
+// that sum to a few units, as normalised ones do; else it goes to the slot's one word for large partials.
+// Returns false when x or the running sum leaves the range, 2^63.  (The common range is tested on the bits
+// and the rest is a function of its own: an FP64 comparison is one more link in the chain of 65-cycle
+// operations that ends every pass.)
+__device__ __forceinline__ void fx_add_small(unsigned long long* a, double x) {
   const double hi_d = trunc(x * 17179869184.0);                                      // 2^34
   const long long lo = (long long)((x * 17179869184.0 - hi_d) * 1073741824.0);       // exact difference, 2^30
   atomicAdd(&a[0], (unsigned long long)lo);
   atomicAdd(&a[1], (unsigned long long)(long long)hi_d);
-  return ok;
+}
+static __device__ __noinline__ bool fx_add_large(unsigned long long* slot, int copy, int c, double x) {
+  if (!(fabs(x) < 9223372036854775808.0)) return false;
+  const double b = trunc(x * 0.125);
+  const long long big = (long long)b;
+  const long long sum = (long long)atomicAdd(slot + ((size_t)kAccCopies * kNMMax + c) * 2, (unsigned long long)big) + big;
+  fx_add_small(slot + ((size_t)copy * kNMMax + c) * 2, fma(-8.0, b, x));
+  return sum < (1ll << 60) && sum > -(1ll << 60);
+}
+__device__ __forceinline__ bool fx_add(unsigned long long* slot, int copy, int c, double x) {
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x40200000) return fx_add_large(slot, copy, c, x);   // |x| >= 8
+  fx_add_small(slot + ((size_t)copy * kNMMax + c) * 2, x);
+  return true;
 }
 
 template <class Tab>
@@ -984,7 +988,7 @@ __device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsi
       ok = !any_ovf && x < kFixLimit && x > -kFixLimit;
       if (ok) atomicAdd(acc_slot + ((size_t)copy * kNMMax + c) * 2, (unsigned long long)x);
     } else {
-      ok = (__double2hiint(x) & 0x7fffffff) < 0x43e00000 && fx_add(acc_slot, copy, c, x);     // |x| < 2^63
+      ok = fx_add(acc_slot, copy, c, x);
     }
     if (!ok) {
       if (reject) atomicMax(errmax, 0x7ff0000000000000ull);
@@ -1262,7 +1266,12 @@ __device__ __forceinline__ void vstore_at(const KParams& p, int span, Real* ptr,
 
 // sqrt(x) and 1/sqrt(x) to rounding: Newton steps from the hardware's FP32 reciprocal square root, no
 // division (the library's FP64 square root and division are chains of 673 and 429 cycles on GB300; only an
-// FP64 x beyond the seed's range takes them).  x is at least 1e-10 (FP32: 1e-6), see rotate.
+// FP64 x beyond the seed's range takes them, by a test on its bits: an FP64 comparison there cost 1 % of a
+// call of 8 Lie RK4 steps of 4096 beams).  x is at least about 1e-10 (FP32: 1e-6), see rotate.
+static __device__ __noinline__ void sqrt_pair_library(double x, double& t, double& r) {
+  t = sqrt(x);
+  r = 1.0 / t;
+}
 __device__ __forceinline__ void sqrt_pair(float x, float& t, float& r) {
   r = rsqrtf(x);
   r = fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
@@ -1270,9 +1279,8 @@ __device__ __forceinline__ void sqrt_pair(float x, float& t, float& r) {
   t = fmaf(0.5f * r, fmaf(-t, t, x), t);
 }
 __device__ __forceinline__ void sqrt_pair(double x, double& t, double& r) {
-  if (!(x < 1.0e38)) {
-    t = sqrt(x);
-    r = 1.0 / t;
+  if (__double2hiint(x) >= 0x47e00000) {                       // 2^127 and more, or not a number
+    sqrt_pair_library(x, t, r);
     return;
   }
   r = (double)rsqrtf((float)x);
@@ -1289,8 +1297,10 @@ template <typename Real>
 __device__ __forceinline__ void rotate(const Real (&Om)[3], Real (&y)[3]) {
   const Real t2 = Om[0] * Om[0] + Om[1] * Om[1] + Om[2] * Om[2];
   Real a, b;
-  const Real eps = sizeof(Real) == 4 ? Real(1e-3) : Real(1e-5);
-  if (t2 > eps * eps) {
+  bool tiny;
+  if constexpr (sizeof(Real) == 4) tiny = !(t2 > Real(1e-3) * Real(1e-3));
+  else tiny = __double2hiint(t2) < 0x3ddb7cdf;                 // below about 1e-10, from the leading bits
+  if (!tiny) {
     Real t, r, sh, ch;
     sqrt_pair(t2, t, r);
     if constexpr (sizeof(Real) == 4) sincosf(0.5f * t, &sh, &ch);
