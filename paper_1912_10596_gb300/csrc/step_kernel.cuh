@@ -1738,11 +1738,12 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       return;
     }
     if (Tab::kAdaptive) {
-      // split final pass (y holds y5): k_S = f(y5) with the moments of y5, the embedded error, and the
-      // squared error ratio (its square root is taken once per block).  Only the largest ratio counts:
-      // an FP32 estimate of it (components by their leading 21 bits; never below the ratio by more than
-      // the 1e-3 it is raised by, norm_floor) passes over every beam that cannot exceed the largest found so far in the block, so the FP64 norms, square root
-      // and division -- a fifth of a DP45 step's FP64 work -- are left for a few beams a block.
+      // split final pass (y holds y5, whose moments the pass before reduced): k_S = f(y5), the embedded
+      // error, and the squared error ratio (its square root is taken once per block).  Only the largest
+      // ratio counts: an FP32 estimate of it (components by their leading 21 bits; never below the ratio
+      // by more than the 1e-3 it is raised by, norm_floor) passes over every beam that cannot exceed the
+      // largest found so far in the block, so the FP64 norms, square root and division -- a fifth of a
+      // DP45 step's FP64 work -- are left for a few beams a block.
       Real Kv[Phys::NG], kS[NC], e[NC];
       Phys::K(tv.row(Tab::S, tj), bm, Kv);
       Phys::f(Kv, y, kS);
@@ -1758,8 +1759,10 @@ struct PassBody<Phys, Tab, Real, false, kPass, kKind> {
       using P32 = typename Phys::template With<float>;
       const float df = bs.atol_f + bs.rtol_f * P32::norm_floor(of, yf);
       const float rf = __fdividef(P32::tnorm2(ef), df * df);
-      // also where rf is not a number, and where the squares leave FP32's range
-      if (!(rf * 1.001f < __int_as_float(*(volatile int*)&bs.emax_f)) || !(df < 1.0e18f)) {
+      // also where rf is not a number, and where the squares leave FP32's range: with df above 1e-12 they
+      // lose bits only where the squared ratio is below 1e-13
+      const float found = __int_as_float(*(volatile int*)&bs.emax_f);
+      if (!(rf * 1.001f < found && found > 1.0e-13f && df > 1.0e-12f && df < 1.0e18f)) {
         const Real no = Phys::tnorm2(yo), n5 = Phys::tnorm2(y);
         if (!(no <= rbig<Real>())) bad = 1;                     // non-finite input state: fatal
         const Real den = bs.atol + bs.rtol * sqrt(fmax(no, n5));
