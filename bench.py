@@ -35,7 +35,7 @@ L2_BYTES = 129 * 1024 * 1024
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
 STEP_TRAFFIC = {"bytes_per_launch": 51172864 + 173309184, "steps_per_launch": 8,
-                "code_sha256": "321434dd5e85ab2221a5a649b8f23c9dcc6d97b8b920a42b67814af5610d2a51"}
+                "code_sha256": "adf87e349e764bd2ed7f780f7d7b1cc8ba8063bb23c1964f8d70ee0ad34d3250"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a

@@ -826,7 +826,7 @@ int clear_sync_words(xflat_t h) {
   CUDA_TRY(h, cudaMemsetAsync(h->d_words, 0, 2 * sizeof(int), h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_nonfinite, 0, h->inst.size() * sizeof(int), h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->d_errmax, 0, h->inst.size() * sizeof(unsigned long long), h->stream));
-  CUDA_TRY(h, cudaMemsetAsync(h->d_acc, 0, h->inst.size() * kAccWordsPerInst * sizeof(unsigned long long), h->stream));
+  CUDA_TRY(h, cudaMemsetAsync(h->d_acc, 0, h->inst.size() * acc_words_per_inst(h->real_size) * sizeof(unsigned long long), h->stream));
   return XFLAT_OK;
 }
 
@@ -1136,7 +1136,7 @@ int create_impl(const xflat_config* cfgs, uint32_t n, xflat_t* out) {
   }
   if (dev_alloc(&h->d_ic, sizeof(InstConst) * n) != cudaSuccess ||
       dev_alloc(&h->d_dyn, sizeof(InstDyn) * n) != cudaSuccess ||
-      dev_alloc(&h->d_acc, sizeof(unsigned long long) * n * kAccWordsPerInst) != cudaSuccess ||
+      dev_alloc(&h->d_acc, sizeof(unsigned long long) * n * acc_words_per_inst(h->real_size)) != cudaSuccess ||
       dev_alloc(&h->d_errmax, sizeof(unsigned long long) * n) != cudaSuccess ||
       dev_alloc(&h->d_nonfinite, sizeof(int) * n) != cudaSuccess ||
       dev_alloc(&h->d_etab, (size_t)eoff * h->real_size) != cudaSuccess ||
@@ -1877,7 +1877,7 @@ int xflat_shard_partials(xflat_t h, int64_t* words) {
   uint32_t nw = 0;
   xflat_shard_info(h, nullptr, &nw);
   const int nm = (int)(nw - 2) / 2, slot = shard_slot(h);
-  constexpr int kWords = kAccWordsPerSlot;
+  const int kWords = acc_words_per_slot(h->real_size);
   std::vector<unsigned long long> acc(kWords);
   unsigned long long em = 0;
   int nonfin = 0;
@@ -1909,7 +1909,7 @@ int xflat_shard_set_totals(xflat_t h, const int64_t* words) {
   uint32_t nw = 0;
   xflat_shard_info(h, nullptr, &nw);
   const int nm = (int)(nw - 2) / 2, slot = shard_slot(h);
-  constexpr int kWords = kAccWordsPerSlot;
+  const int kWords = acc_words_per_slot(h->real_size);
   std::vector<unsigned long long> acc(kWords, 0ull);    // the total in copy 0, the other copies 0
   for (int c = 0; c < nm; ++c) {
     const __int128 t = (__int128)(((unsigned __int128)(unsigned long long)words[2 * c + 1] << 64) |

@@ -961,9 +961,10 @@ __device__ __forceinline__ T reduce_scatter(T (&v)[N], int lane, int& idx, int& 
 }
 
 // Block sums of the threads' moment partials v (double, or integers of the instance's unit in the
-// mixed kernels) into one copy of the accumulators of an instance's stage slot: reduce-scatter in each warp, one
-// shared-memory row a warp, a half-warp tree a component over up to 16 warps, and one fixed-point
-// addition a component.  In a fixed order, so the result depends on the block decomposition only.
+// mixed kernels) into one copy of the accumulators of an instance's stage slot (mixed: acc_slot is that
+// copy): reduce-scatter in each warp, one shared-memory row a warp, a half-warp tree a component over up to
+// 16 warps, and one fixed-point addition a component.  In a fixed order, so the result depends on the block
+// decomposition only.
 // ovf: a thread's partial left the integer range (mixed).  A sum that is not finite or out of range
 // (FP64: 2^63 and more) rejects an adaptive trial step (reject) and is fatal otherwise.
 template <int NM, typename T>
@@ -986,7 +987,7 @@ __device__ __forceinline__ void reduce_moments(T (&v)[NM], int ovf, T* red, unsi
     bool ok;
     if constexpr (T(0.5) == T(0)) {
       ok = !any_ovf && x < kFixLimit && x > -kFixLimit;
-      if (ok) atomicAdd(acc_slot + ((size_t)copy * kNMMax + c) * 2, (unsigned long long)x);
+      if (ok) atomicAdd(acc_slot + 2 * c, (unsigned long long)x);
     } else {
       ok = fx_add(acc_slot, copy, c, x);
     }
@@ -1032,7 +1033,7 @@ __device__ int serial_update(const KParams& p, int slot, bool final_pass, bool i
   for (int i = threadIdx.x; i < p.n_inst; i += blockDim.x) {
     const InstConst& ic = p.ic[i];
     InstDyn& d = p.dyn[i];
-    const unsigned long long* acc = p.acc + (size_t)i * kAccWordsPerInst + (size_t)slot * kAccWordsPerSlot;
+    const unsigned long long* acc = p.acc + (size_t)i * acc_words_per_inst(sizeof(Real)) + (size_t)slot * acc_words_per_slot(sizeof(Real));
     const bool have_moments = !(final_pass && !Tab::kFinalMoments);
     const bool adaptive_final = final_pass && Tab::kAdaptive && !Tab::kFinalMoments;   // FSAL
     // ---- every load first (no store may sit between them) -------------------------------
@@ -1163,14 +1164,14 @@ __device__ int serial_update(const KParams& p, int slot, bool final_pass, bool i
 // Accumulator slots of the stages kPasses..S (no pass of their own index clears them), zeroed by
 // the last block of the final barrier: nobody accumulates into or reads them until the next step
 // (the fence in serial_geometry publishes the stores before the release).
-template <class Tab>
+template <class Tab, typename Real>
 __device__ void clear_late_slots(const KParams& p) {
-  constexpr int kWords = kAccWordsPerSlot;
+  constexpr int kWords = acc_words_per_slot(sizeof(Real));
   constexpr int kLate = Tab::S - Tab::kPasses + 1;
   for (int t = threadIdx.x; t < p.n_inst * kLate * kWords; t += blockDim.x) {
     const int inst = t / (kLate * kWords), rem = t % (kLate * kWords);
     const int slot = Tab::kPasses + rem / kWords;
-    p.acc[(size_t)inst * kAccWordsPerInst + (size_t)slot * kWords + rem % kWords] = 0ull;
+    p.acc[(size_t)inst * acc_words_per_inst(sizeof(Real)) + (size_t)slot * kWords + rem % kWords] = 0ull;
   }
 }
 
@@ -2340,7 +2341,7 @@ __device__ __noinline__ void setup_piece(const KParams& p, BlockShared<Real, Phy
   const int n_jj = pc.n_jj;
   // constant c of the newest stage
   auto newest_constant = [&](int c) {
-    const unsigned long long* accs = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)newest * kAccWordsPerSlot;
+    const unsigned long long* accs = p.acc + (size_t)pc.inst * acc_words_per_inst(sizeof(Real)) + (size_t)newest * acc_words_per_slot(sizeof(Real));
     InstDyn* dw = p.dyn + pc.inst;
     double v = 0.0;
     if (c < Phys::NM) {
@@ -2481,12 +2482,12 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
   // into a cleared slot until at least one barrier later, and block 0's stores are fenced at its
   // next arrival.
   if (kKind != kInitPass && blockIdx.x == 0) {
-    constexpr int kWords = kAccWordsPerSlot;
+    constexpr int kWords = acc_words_per_slot(sizeof(Real));
     constexpr int kSlots = kPass == 0 ? 2 : (kPass >= 2 ? 1 : 0);
     for (int t = threadIdx.x; t < p.n_inst * kSlots * kWords; t += blockDim.x) {
       const int inst = t / (kSlots * kWords), rem = t % (kSlots * kWords), q = rem / kWords;
       const int zslot = kPass == 0 ? q : kPass;
-      p.acc[(size_t)inst * kAccWordsPerInst + (size_t)zslot * kWords + rem % kWords] = 0ull;
+      p.acc[(size_t)inst * acc_words_per_inst(sizeof(Real)) + (size_t)zslot * kWords + rem % kWords] = 0ull;
     }
   }
   const unsigned need = stages_needed<Tab, kPass, kKind>();
@@ -2721,7 +2722,8 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
     // the current state (init pass)
     constexpr bool kErrMax = kKind == kFinalPass && Tab::kAdaptive;
     constexpr bool kRejectOverflow = Tab::kAdaptive && kKind != kInitPass;
-    unsigned long long* acc_slot = p.acc + (size_t)pc.inst * kAccWordsPerInst + (size_t)slot * kAccWordsPerSlot;
+    unsigned long long* acc_slot =
+        p.acc + (size_t)pc.inst * acc_words_per_inst(sizeof(Real)) + (size_t)slot * acc_words_per_slot(sizeof(Real));
     const int copy = blockIdx.x % kAccCopies;
     if constexpr (sizeof(Real) == 4) {
       // mixed precision: each thread's (hi, lo) partial sums go to integers of the instance's
@@ -2750,7 +2752,7 @@ __device__ void run_pass(const KParams& p, BlockShared<Real, Phys>& bs, unsigned
             v[i] = biased_fix<1>(h, acc.lo[i], bias[i / NC], ovf);
           }
         }
-        reduce_moments<NM, long long>(v, ovf, reinterpret_cast<long long*>(red), acc_slot, copy, &p.errmax[pc.inst],
+        reduce_moments<NM, long long>(v, ovf, reinterpret_cast<long long*>(red), acc_slot + (size_t)copy * kNMMax * 2, 0, &p.errmax[pc.inst],
                                       &p.nonfinite[pc.inst], kRejectOverflow);
       }
     } else {
@@ -2831,7 +2833,7 @@ __device__ __forceinline__ bool pass_and_sync(const KParams& p, BlockShared<Real
   } else if ((res & 0xf) == kBarLast) {
     const int mine = serial_update<Phys, Tab, Real>(p, 0, true, false);
     const int all = __syncthreads_and(mine);
-    clear_late_slots<Tab>(p);
+    clear_late_slots<Tab, Real>(p);
     serial_geometry<Tab>(p);
     if (threadIdx.x == 0) {
       *p.all_done = all;
@@ -2902,7 +2904,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) step_kernel(const __grid_cons
     const bool init = p.shard_mode == kShardSerialInit;
     const int mine = serial_update<Phys, Tab, Real>(p, init ? 1 : 0, !init, init);
     const int all = __syncthreads_and(mine);
-    if (!init) clear_late_slots<Tab>(p);
+    if (!init) clear_late_slots<Tab, Real>(p);
     serial_geometry<Tab>(p);
     if (threadIdx.x == 0) *p.all_done = all;
     return;

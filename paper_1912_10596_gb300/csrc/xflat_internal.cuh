@@ -25,10 +25,10 @@ constexpr int kNSCMax = 20;
 // (block index mod kAccCopies), so the integer atomics of hundreds of blocks spread over several
 // L2 lines instead of queueing on one; the last block sums the copies (exact integer sums).
 constexpr int kAccCopies = 8;
-// accumulator words: [stage slot][copy][component][2] per instance, where copy kAccCopies holds the FP64
-// kernels' words for partials of 8 and more (fx_add)
-constexpr int kAccWordsPerSlot = (kAccCopies + 1) * kNMMax * 2;
-constexpr int kAccWordsPerInst = kMaxStages * kAccWordsPerSlot;
+// accumulator words: [stage slot][copy][component][2] per instance; FP64 kernels have one copy more, whose
+// words hold the upper parts of partials of 8 and more (fx_add)
+constexpr int acc_words_per_slot(size_t real_size) { return (kAccCopies + (real_size == 8 ? 1 : 0)) * kNMMax * 2; }
+constexpr int acc_words_per_inst(size_t real_size) { return kMaxStages * acc_words_per_slot(real_size); }
 
 enum Integrator : int { kRK4 = 0, kDP45 = 1, kLieRK4 = 2, kExpMid = 3, kLieAdaptive = 4 };
 enum Matter : int { kMatterNone = 0, kMatterPower = 1, kMatterConst = 2, kMatterTable = 3 };
