@@ -2,7 +2,8 @@
 
 For one workload it times a few radial steps for every candidate (threads per block, resident
 blocks per SM) -- which also selects the kernel's register budget, see csrc/kernels_2f.cu -- and
-returns the fastest.  Results are cached per (GPU, workload signature) in _build/autotune.json.
+returns the fastest.  Results are cached per (GPU, workload signature, library) in
+_build/autotune.json.
 All timing runs through the library's own launches (xflat_advance) with CUDA events.
 """
 from __future__ import annotations
@@ -13,14 +14,32 @@ import os
 HERE = os.path.dirname(os.path.abspath(__file__))
 CACHE = os.path.join(HERE, "_build", "autotune.json")
 
-# (block_size, blocks_per_sm): 768 or 512 resident threads per SM
+# (block_size, blocks_per_sm); (0, 0) is the library's own choice.
+# Mixed two-flavour bulb kernels: 768 or 512 resident threads per SM (the library's choice is among them)
 CANDIDATES_MIXED_2F = [(256, 3), (256, 2), (512, 1), (128, 6), (128, 4)]
-CANDIDATES_OTHER = [(256, 1), (128, 2)]
+# All others.  The library's choice also sizes the block to a small problem and takes the two-block FP64
+# kernels, which (256, 1) excludes and (128, 2) does not fill.
+CANDIDATES_OTHER = [(0, 0), (256, 1), (256, 2), (128, 2)]
 
 
-def _signature(cfg, n_inst, gpu):
+def _candidates(xf, cfg):
+    if cfg.precision != xf.MIXED or cfg.n_flavor != 2:
+        return CANDIDATES_OTHER
+    return CANDIDATES_MIXED_2F + ([(0, 0)] if cfg.n_phi >= 2 else [])
+
+
+def _library(xf):
+    """Hash of the loaded library's sources and flags (written beside it by the build)."""
+    try:
+        with open(xf._LIB_PATH + ".sha256") as f:
+            return f.read().strip()[:16]
+    except OSError:
+        return "unknown"
+
+
+def _signature(xf, cfg, n_inst, gpu):
     return (f"{gpu}|nf{cfg.n_flavor}|p{cfg.precision}|i{cfg.integrator}|"
-            f"E{cfg.n_energy}|u{cfg.n_angle}|n{n_inst}")
+            f"E{cfg.n_energy}|u{cfg.n_angle}|phi{cfg.n_phi}|n{n_inst}|lib{_library(xf)}")
 
 
 def _time(xf, torch, cfgs, spectra, r_end, steps, warmup):
@@ -52,7 +71,7 @@ def tune(xf, cfgs, spectra, r_end, steps=6, warmup=2, use_cache=True, log=None):
     import torch
 
     gpu = torch.cuda.get_device_name()
-    key = _signature(cfgs[0], len(cfgs), gpu)
+    key = _signature(xf, cfgs[0], len(cfgs), gpu)
     cache = {}
     if use_cache and os.path.exists(CACHE):
         try:
@@ -61,10 +80,8 @@ def tune(xf, cfgs, spectra, r_end, steps=6, warmup=2, use_cache=True, log=None):
             cache = {}
     if key in cache:
         return tuple(cache[key]["best"])
-    mixed2f = cfgs[0].precision == xf.MIXED and cfgs[0].n_flavor == 2
-    cands = CANDIDATES_MIXED_2F if mixed2f else CANDIDATES_OTHER
     results = {}
-    for bs, bps in cands:
+    for bs, bps in _candidates(xf, cfgs[0]):
         trial = []
         for c in cfgs:
             t = xf.xflat_config.from_buffer_copy(c)
