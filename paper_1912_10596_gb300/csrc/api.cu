@@ -344,23 +344,25 @@ __global__ void k_pee(const Real* src, uint64_t stride, uint32_t n, int nf, doub
 }
 
 // Number-flux weighted mean of P_ee over nu beams, deterministic and spread over the GPU (the
-// sums are FP64, whose pipe is narrow: one block would take milliseconds at 2M beams).  One warp
-// per angle bin sums N_e,k P_ee over energies, straight from the state (lanes in a fixed order, then a
-// fixed shuffle tree); one block then sums du_j times the rows in a fixed tree.
+// sums are FP64, whose pipe is narrow: one block would take milliseconds at 2M beams).  A warp, or the
+// 2^lg lanes of it that an angle bin's energies fill, sums N_e,k P_ee over energies, straight from the
+// state (lanes in a fixed order, then a fixed shuffle tree; the lanes left out would add zeros); one block
+// then sums du_j times the rows in a fixed tree.  (The FP64 pipe takes a warp instruction's time whatever
+// its active lanes: GB300, a call with 400,000 angle bins of one energy 627 us with a warp a bin, 411 us so.)
 template <typename Real>
 __global__ void k_pee_rows(const Real* src, uint64_t stride, int nf, const double* N_e, uint32_t ne, uint32_t na,
-                           double* rows) {
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= na) return;
-  const Real* p = src + (nf == 2 ? 2 * stride : 0) + (uint64_t)warp * ne;
+                           int lg, double* rows) {
+  const uint32_t row = (blockIdx.x * blockDim.x + threadIdx.x) >> lg, lane = threadIdx.x & ((1u << lg) - 1u);
   double s = 0.0;
-  for (uint32_t k = lane; k < ne; k += 32) {
-    const double v = (double)p[k];
-    s += N_e[k] * (nf == 2 ? 0.5 * (1.0 + v) : v);
+  if (row < na) {
+    const Real* p = src + (nf == 2 ? 2 * stride : 0) + (uint64_t)row * ne;
+    for (uint32_t k = lane; k < ne; k += 1u << lg) {
+      const double v = (double)p[k];
+      s += N_e[k] * (nf == 2 ? 0.5 * (1.0 + v) : v);
+    }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if (lane == 0) rows[warp] = s;
+  for (int o = 1 << lg >> 1; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 1 << lg);
+  if (row < na && lane == 0) rows[row] = s;
 }
 
 __global__ void k_pee_final(const double* rows, const double* du, uint32_t na, double den, double* out) {
@@ -1563,9 +1565,11 @@ int xflat_pee_inst(xflat_t h, uint32_t inst, double* pee_per_beam, double* pee_m
   double sN = 0.0, sdu = 0.0;
   for (uint32_t k = 0; k < ne; ++k) sN += I.N[k];
   for (uint32_t j = 0; j < na; ++j) sdu += I.du[j];
-  const unsigned nrb = (unsigned)((32ull * na + 255) / 256);
-  if (h->real_size == 8) k_pee_rows<double><<<nrb, 256, 0, h->stream>>>((const double*)src, h->stride, h->nf, Ne, ne, na, rows);
-  else k_pee_rows<float><<<nrb, 256, 0, h->stream>>>((const float*)src, h->stride, h->nf, Ne, ne, na, rows);
+  int lg = 0;
+  while (lg < 5 && (1u << lg) < ne) ++lg;
+  const unsigned nrb = (unsigned)((((uint64_t)na << lg) + 255) / 256);
+  if (h->real_size == 8) k_pee_rows<double><<<nrb, 256, 0, h->stream>>>((const double*)src, h->stride, h->nf, Ne, ne, na, lg, rows);
+  else k_pee_rows<float><<<nrb, 256, 0, h->stream>>>((const float*)src, h->stride, h->nf, Ne, ne, na, lg, rows);
   k_pee_final<<<1, 1024, 0, h->stream>>>(rows, h->d_du + I.a_off, na, sN * sdu, mean);
   CUDA_TRY(h, cudaGetLastError());
   if (pee_per_beam) CUDA_TRY(h, cudaMemcpyAsync(pee_per_beam, pee, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
