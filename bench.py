@@ -35,7 +35,7 @@ L2_BYTES = 129 * 1024 * 1024
 # dram__bytes_write.sum of one ncu capture of an 8-step launch after the L2 flush).  It holds only for that launch size and for the kernel
 # code it was taken on, identified by kernel_code_hash(); otherwise the benchmark reports null.
 STEP_TRAFFIC = {"bytes_per_launch": 51172864 + 173309184, "steps_per_launch": 8,
-                "code_sha256": "adf87e349e764bd2ed7f780f7d7b1cc8ba8063bb23c1964f8d70ee0ad34d3250"}
+                "code_sha256": "d118a5231e33b9bcf12949ef29d2c0b0bf5cb1695ff709432c954a1979ab19bd"}
 KERNEL_SOURCES = ["step_kernel.cuh", "xflat_internal.cuh", "kernels_2f.cu"]
 # Warp instructions of one radial step of the same kernel code (smsp__inst_executed.sum of one ncu
 # capture of a one-step launch, which also carries the launch's first set-up, so a step inside a
@@ -606,8 +606,8 @@ def measure_configs(only=None):
         range_run(big, "fp64", "lie_adaptive", 1e-6, big.r1)
         range_run(big, "fp64", "lie_adaptive", 1e-9, big.r1)
         range_run(big, "mixed", "dp45", 1e-6, big.r1, n_per_launch=256)
-        # three flavours, both hierarchies: the adaptive exact propagators (3 x 3 Eq. U by
-        # eigen-decomposition) over the whole 11 -> 1000 km, and explicit DP45 from R for comparison
+        # three flavours, both hierarchies: the adaptive exact propagators (3 x 3 Eq. U in
+        # closed form) over the whole 11 -> 1000 km, and explicit DP45 from R for comparison
         for dm31 in (2.4e-3, -2.4e-3):
             wl3 = workload_3f_fp64(dm31)
             range_run(wl3, "mixed", "lie_adaptive", 1e-6, wl3.r1)

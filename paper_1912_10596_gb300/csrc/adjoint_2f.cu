@@ -46,7 +46,7 @@ struct AdjShared {
   AdjBack back[kAdjRows];
   double scratch[32 * 6];
   double tot[8];
-  double str[2];                        // mu, lambda of the formed stage (forward, last block)
+  double str[2];                        // mu, lambda of the formed stage (forward)
   double scf[kAdjStageVals];            // constants of the stage finished in this pass
   double scs[4][kAdjStageVals];         // constants of the formed stage's step (backward: all 4)
   double gl[8];                         // broadcast adjoint moments of the finished stage

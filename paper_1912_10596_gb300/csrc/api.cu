@@ -888,15 +888,14 @@ int refresh_moments(xflat_t h) {
 
 int setup_launch_shape(xflat_t h, const xflat_config& c) {
   // mixed two-flavour kernels exist at two register budgets: 768 resident threads per SM (80
-  // registers) and 512 (128 registers); the request picks the one that fits.  Every other kernel
-  // is built for one 256-thread block per SM.  Default for the mixed two-flavour bulb kernels: one
-  // 512-thread block per SM while both state buffers fit the L2 (the passes are then bound by
-  // issue: the 80-register budget spills, and two co-resident blocks finish their passes at
-  // different times), three 256-thread blocks once the state streams from HBM (more loads in
-  // flight); 256 threads otherwise.  (GB300, DP45, 28M beams in 64 instances with dynamic piece
-  // scheduling: 1.86 ms per step at 256 x 3 against 1.96 ms at 256 x 2 and about 2.2 ms at
-  // 512 x 1; 4M beams in one instance: 0.186 ms per one-step launch at 512 x 1 against 0.224 ms
-  // at 256 x 3.)
+  // registers) and 512 (128 registers); the request picks the one that fits.  The other kernels
+  // are built for one 256-thread block per SM, FP64 RK4 and DP45 of two flavours also for two.  Default
+  // for the mixed two-flavour bulb kernels: one 512-thread block per SM while both state buffers fit the
+  // L2 (the passes are then bound by issue: the 80-register budget spills, and two co-resident blocks
+  // finish their passes at different times), two 256-thread blocks once the state streams from HBM; 256
+  // threads otherwise.  (GB300, DP45, 28M beams in 64 instances with dynamic piece scheduling: 1.74 ms
+  // per step at 256 x 2, 1.81 to 1.89 at 256 x 3 and 2.05 at 512 x 1; 4M beams in one instance: 0.186 ms
+  // per one-step launch at 512 x 1 against 0.224 ms at 256 x 3; both before the scalar table rows.)
   const bool mixed_2f = h->nf == 2 && !h->extended && h->real_size == 4;
   int l2_bytes = 0;
   cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, h->device);

@@ -214,10 +214,13 @@ __device__ __forceinline__ void geometry_f(double u, double x, float& q, float& 
 //   s = fma(w, y, hi),  z = hi - s,  lo += fma(w, y, z),  hi = s.
 // hi starts at a bias 1.5 2^m with 2^(m-1) at least the sum of the contributions' magnitudes, so it
 // stays in one binade: z is exact (both are multiples of the same 2^(m-23)), fma(w, y, z) is the part
-// of the exact product that hi did not take, rounded near 2^(m-48), and lo's own roundings lie there
-// too -- as in a double accumulator, and the product itself is not rounded first.  (TwoSum on the
-// rounded product takes eight operations and needs no bias.)  At the end of a pass hi is an integer
-// count of 2^(m-23) read off its bits (biased_fix) and every further sum is an integer addition.  The
+// of the exact product that hi did not take, rounded to 2^(m-48), and the product itself is not rounded
+// first; lo's own roundings are near 2^(m-48) times the square root of the n contributions.  2^m is at most
+// 16 (n + 2) wmax (run_pass), so with weights of wbar on average the error of a thread's sum is about
+// n 2^-46 wmax / wbar of it, coarser than a double's but below the 2^-24 roundings of the states and weights
+// while n wmax / wbar is below 2^22.  (TwoSum on the rounded product takes eight operations and needs no
+// bias.)  At the end of a pass hi is an integer count of 2^(m-23) read off its bits (biased_fix) and every
+// further sum is an integer addition.  The
 // FP32 weights carry a per-instance power-of-two scale (InstConst::acc_unit = 2^-S) so that the
 // integers are in units of 2^-S; no FP64 instruction is issued per beam (GB300's FP64 pipe is ~1/68
 // of its FP32 rate).  Components come in groups with a bias each (D, J1, and Jc, Js): their weights
@@ -406,15 +409,6 @@ struct Phys2 {
   __device__ static inline Real norm_floor(const Real (&a)[3], const Real (&b)[3]) {
     return sqrt(fmax(tnorm2(a), tnorm2(b)));
   }
-  // Frobenius norm of the traceless matrix (e.sigma)/2, scaled so it cannot overflow; +inf if not finite
-  __device__ static inline Real enorm(const Real (&e)[3]) {
-    const Real m = fmax(fabs(e[0]), fmax(fabs(e[1]), fabs(e[2])));
-    if (!(m <= rbig<Real>())) return Real(INFINITY);
-    if (m == Real(0)) return Real(0);
-    const Real inv = Real(1) / m;
-    const Real a = e[0] * inv, b = e[1] * inv, c = e[2] * inv;
-    return m * sqrt(Real(0.5) * (a * a + b * b + c * c));
-  }
   __device__ static inline void normalise(Real (&y)[3]) {
     const Real n2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
     const Real inv = Real(1) / sqrt(n2);
@@ -542,21 +536,6 @@ struct Phys3 {
   __device__ static inline Real norm_floor(const Real (&a)[9], const Real (&b)[9]) {
     const Real d = fabs(a[0]) + fabs(a[1]) + fabs(a[2]) + fabs(b[0]) + fabs(b[1]) + fabs(b[2]);
     return fmax(sqrt(fmax(tnorm2(a), tnorm2(b))) - Real(4e-6) * d, Real(0));
-  }
-  // full Frobenius norm of the Hermitian matrix, scaled against overflow; +inf if not finite
-  __device__ static inline Real enorm(const Real (&e)[9]) {
-    Real m = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) m = fmax(m, fabs(e[i]));
-    if (!(m <= rbig<Real>())) return Real(INFINITY);
-    if (m == Real(0)) return Real(0);
-    const Real inv = Real(1) / m;
-    Real d = 0, o = 0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) d += (e[i] * inv) * (e[i] * inv);
-#pragma unroll
-    for (int i = 3; i < 9; ++i) o += (e[i] * inv) * (e[i] * inv);
-    return m * sqrt(d + 2 * o);
   }
   __device__ static inline void normalise(Real (&)[9]) {}
   // Mixed-precision exponential steps: restore the idempotency of the (pure) density matrix that
@@ -717,7 +696,6 @@ struct Phys2E {
   }
   __device__ static inline Real tnorm2(const Real (&y)[3]) { return Phys2<Real>::tnorm2(y); }
   __device__ static inline Real norm_floor(const Real (&a)[3], const Real (&b)[3]) { return Phys2<Real>::norm_floor(a, b); }
-  __device__ static inline Real enorm(const Real (&e)[3]) { return Phys2<Real>::enorm(e); }
   __device__ static inline void normalise(Real (&y)[3]) { Phys2<Real>::normalise(y); }
   __device__ static inline void purify(Real (&y)[3]) { Phys2<Real>::normalise(y); }
 };
@@ -781,12 +759,11 @@ static __device__ __noinline__ void bounds_fault(const KParams& p, int site, lon
     atomicExch(reinterpret_cast<unsigned long long*>(&p.bar->bounds_off), (unsigned long long)off);
   atomicCAS(p.status, 0, 3 /* XFLAT_ERR_CUDA */);
 }
-__device__ __forceinline__ bool span_ok(const KParams& p, int id, const void* ptr, unsigned bytes, int site,
-                                        unsigned align = 0) {
+__device__ __forceinline__ bool span_ok(const KParams& p, int id, const void* ptr, unsigned bytes, int site) {
   const Span sp = p.span[id];
   const char* c = static_cast<const char*>(ptr);
   const bool ok = sp.lo != nullptr && c >= sp.lo && c + bytes <= sp.lo + sp.bytes &&
-                  (reinterpret_cast<uintptr_t>(c) % (align ? align : bytes)) == 0;
+                  (reinterpret_cast<uintptr_t>(c) % bytes) == 0;
   if (!ok) bounds_fault(p, site, sp.lo ? (long long)(c - sp.lo) : -1ll);
   return ok;
 }
@@ -795,11 +772,9 @@ __device__ __forceinline__ bool index_ok(const KParams& p, bool ok, int site, lo
   return ok;
 }
 #define XFLAT_SPAN_OK(p, id, ptr, bytes, site) ::xflat::span_ok((p), (id), (ptr), (bytes), (site))
-#define XFLAT_SPAN_OK_AL(p, id, ptr, bytes, align, site) ::xflat::span_ok((p), (id), (ptr), (bytes), (site), (align))
 #define XFLAT_INDEX_OK(p, cond, site, v) ::xflat::index_ok((p), (cond), (site), (long long)(v))
 #else
 #define XFLAT_SPAN_OK(p, id, ptr, bytes, site) true
-#define XFLAT_SPAN_OK_AL(p, id, ptr, bytes, align, site) true
 #define XFLAT_INDEX_OK(p, cond, site, v) true
 #endif
 
@@ -835,10 +810,6 @@ __device__ __forceinline__ bool fx_add(unsigned long long* slot, int copy, int c
 template <class Tab>
 __device__ __forceinline__ double stage_c(int i) { return Tab::c(i); }
 
-// ------------------------------------------------------------------------------------------
-// The last block to arrive: reduce accumulators, derive stage constants, run the controller.
-// Every value another block may have written since this SM last looked is read through L2
-// (__ldcg), never from a possibly stale L1 line; the loads are issued before any branch on them.
 // 0.9 Err^(-1/P), the unclamped step-size factor, in double (P = 5 for the 5(4) pair, 2 for the
 // 2(1) pair).  The caller clamps it to [0.2, 5], which decides alone below Err = (0.9/5)^P and
 // above (0.9/0.2)^P, so only (a slightly wider) range is computed: a float seed refined by two
@@ -860,8 +831,6 @@ __device__ __forceinline__ double controller_factor(double err) {
   return 0.9 * y;
 }
 
-// mu(r) and lambda(r) at one radius (double).
-// mu(r) and lambda(r) from 1/r
 // lambda(r) from a matter table: the interval [r_i, r_{i+1}) holding r by binary search, then
 // lambda_i (r / r_i)^p_i (the end values outside the table)
 __device__ inline double table_strength(const double* t, int n, double r) {
@@ -874,6 +843,7 @@ __device__ inline double table_strength(const double* t, int n, double r) {
   }
   return t[3 * lo + 1] * pow(r / t[3 * lo], t[3 * lo + 2]);
 }
+// mu(r) and lambda(r) from 1/r
 __device__ __forceinline__ void strengths_inv(const InstConst& ic, double inv, double& mu, double& lam) {
   mu = ic.geom == kGeomHomogeneous ? ic.mu_const : ic.mu_coef * inv * inv;
   lam = 0.0;
@@ -1025,6 +995,10 @@ __device__ __forceinline__ void reduce_error(float em, int bad, float* red, unsi
   }
 }
 
+// The serial section of a step's final barrier and of the moment launch, in the last block: the
+// instances' stage constants from the accumulators, the controller and the step bookkeeping.  Every value
+// another block may have written since this SM last looked is read through L2 (__ldcg), never from a
+// possibly stale L1 line; the loads are issued before any branch on them.
 template <class Phys, class Tab, typename Real>
 __device__ int serial_update(const KParams& p, int slot, bool final_pass, bool init) {
   constexpr int NM = Phys::NM;
@@ -2877,9 +2851,9 @@ __device__ __forceinline__ void one_pass(const KParams& p, BlockShared<Real, Phy
 
 // kThreads x kMinB: the block size and resident blocks per SM the register budget is sized for.
 // FP64 work runs on GB300's narrow FP64 pipe (about 1/68 of the FP32 rate), which one 256-thread
-// block per SM already keeps busy, so FP64 kernels are built for that (whole register file, no
-// spills).  The FP32 two-flavour kernels are latency-bound; they are built for 768 resident threads
-// per SM (256 x 3) and for 512 (256 x 2, or one 512-thread block: the SM's two halves of the work
+// block per SM already keeps busy, so FP64 kernels are built for that (whole register file, no spills), the
+// two-flavour RK4 and DP45 also for two blocks (kernels_2f.cu).  The FP32 two-flavour kernels are
+// latency-bound; they are built for 768 resident threads per SM (256 x 3) and for 512 (256 x 2, or one 512-thread block: the SM's two halves of the work
 // then finish together instead of the older block's warps finishing first), and the launch shape
 // is chosen by measurement (the autotuner in paper_1912_10596_gb300/autotune.py).
 template <class Phys, class Tab, typename Real, bool kCF, int kMinB, int kThreads = 256>

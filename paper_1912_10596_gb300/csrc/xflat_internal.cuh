@@ -3,9 +3,10 @@
 // Work decomposition.  All instances' beams live in one set of SoA planes.  The beams of the whole
 // problem are cut into G equal contiguous slices, one per persistent block; the intersection of a
 // slice with an instance is a "piece".  A block processes its pieces one after the other and adds
-// each piece's moments to its instance's fixed-point accumulators; the last block to arrive at the
-// device-wide barrier converts them and derives the next stage's constants before it releases the
-// other blocks.
+// each piece's moments to its instance's fixed-point accumulators; after the device-wide barrier every
+// block derives the next stage's constants from them in its set-up.  Only a step's final barrier (and the
+// moment launch's) has a serial section: its last block runs the step bookkeeping before it releases the
+// others.
 #pragma once
 
 #include <cstdint>
@@ -23,7 +24,7 @@ constexpr int kNMMax = 18;
 constexpr int kNSCMax = 20;
 // Blocks add their moment partials to one of kAccCopies copies of an instance's accumulators
 // (block index mod kAccCopies), so the integer atomics of hundreds of blocks spread over several
-// L2 lines instead of queueing on one; the last block sums the copies (exact integer sums).
+// L2 lines instead of queueing on one; every reader sums the copies (exact integer sums).
 constexpr int kAccCopies = 8;
 // accumulator words: [stage slot][copy][component][2] per instance; FP64 kernels have one copy more, whose
 // words hold the upper parts of partials of 8 and more (fx_add)
@@ -144,49 +145,6 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t l, uint64_t magic) {
   return (uint32_t)(((uint64_t)l * magic) >> 40);
 }
 
-// Deterministic block sum of NV doubles per thread (fixed shuffle tree, then fixed smem tree).
-// Result valid in thread 0.  scratch: >= 32 * NV doubles.
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double* scratch) {
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) scratch[warp * NV + i] = v[i];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double s = lane < nw ? scratch[lane * NV + i] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      v[i] = s;
-    }
-  }
-}
-
-__device__ __forceinline__ double block_max(double v, double* scratch) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    double s = lane < nw ? scratch[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_down_sync(0xffffffffu, s, o));
-    v = s;
-  }
-  return v;
-}
-
 // Device-wide barrier.  Returns kBarLast in every thread of the one block that arrived last (that
 // block must call barrier_release after its serial work), kBarReleased elsewhere after the
 // release, or kBarAbort.  Every wait is bounded by timeout_ns: on expiry the block records
@@ -286,13 +244,6 @@ __device__ __forceinline__ bool pass_barrier(Barrier* bar, unsigned int n_blocks
   }
   __syncthreads();
   return *s_flag != kBarAbort;
-}
-
-__device__ __forceinline__ bool barrier_aborted(Barrier* bar, int* s_flag) {
-  __syncthreads();
-  if (threadIdx.x == 0) *s_flag = ld_acquire_int(&bar->abort);
-  __syncthreads();
-  return *s_flag != 0;
 }
 
 }  // namespace xflat

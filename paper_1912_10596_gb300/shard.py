@@ -12,7 +12,7 @@ one of two ways:
   library pass by pass with that exchange (``exchange_words``).
 
 The exchange is exact and deterministic: a partial moment is carried as the FP64 device
-accumulators' own 128-bit fixed-point pair (hi 2^64 + lo = trunc(x 2^64), lo an unsigned and hi a
+accumulators' sum, a 128-bit fixed-point pair (hi 2^64 + lo = trunc(x 2^64), lo an unsigned and hi a
 signed 64-bit word); ranks all-gather the pairs and add them as exact integers, so the total does
 not depend on the number of ranks, their order or the shard boundaries.
 """
